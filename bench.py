@@ -188,13 +188,17 @@ def level_sizes(G):
     return out
 
 
-def algorithmic_bytes(slot, lv, s, cb=4):
+def algorithmic_bytes(slot, lv, s, cb=4, noff=0):
     """Bytes one launch must move at minimum (s-byte values of the hierarchy,
     CG vectors FP64, int32 row pointers and P / R indices; the finest
     matrix's column index takes cb bytes an entry: 4 as int32, 1 when the
-    pattern is stored as one-byte offsets).  lv: level sizes list."""
+    pattern is stored as one-byte offsets).  With noff in 1..8 offsets the
+    finest matrix's pattern is one mask byte a row.  lv: level sizes list."""
     L0 = lv[0]
     n, nnz = L0["n"], L0["nnz"]
+    if 0 < noff <= 8 and slot in ("cg_spmv", "smooth0_l0", "sweep_l0"):
+        return {"cg_spmv": n + 8 * nnz + 16 * n, "smooth0_l0": n + nnz * s + 2 * n * s + 8 * n,
+                "sweep_l0": n + nnz * s + 2 * n * s + 16 * n}[slot]
     nc, nnzP = L0["nagg"], L0["nnzP"]
     nnzc = lv[1]["nnz"] if len(lv) > 1 else 0
     if slot == "cg_spmv":      # q = A p, p.q: ptr, col, val(f64), p, q
@@ -301,6 +305,7 @@ def run_mode(B, torch, w, mode, ptr, col, vals, f, warm_idx, timed_idx, flush, p
         "rebuilds": sum(s.rebuilt for s, _ in infos),
         "all_converged": all(i.status == 0 for _, i in infos),
         "wall_s": wall, "launches": launches, "levels": level_sizes(G), "col_bytes": G.pattern_info()[0],
+        "noffsets": G.pattern_info()[1],
     }
     return G, res, prof, u
 
@@ -580,7 +585,7 @@ def run_ours(args):
         per_raw = ms / cnt
         # solve kernels are timed inside a graph: the empty pair's time is the timing overhead
         per = per_raw - overhead_ms if name in GRAPH_TIMED and per_raw > 2 * overhead_ms else per_raw
-        by = algorithmic_bytes(name, part["levels"], s, part["col_bytes"])
+        by = algorithmic_bytes(name, part["levels"], s, part["col_bytes"], part.get("noffsets", 0))
         fl = algorithmic_flops(name, part["levels"], mixed=s == 4)
         kernels[name] = {"ms_total_per_step": per * cnt / len(timed_idx), "launches_per_step": cnt / len(timed_idx),
                          "us_per_launch": per * 1e3, "us_per_launch_timed": per_raw * 1e3,

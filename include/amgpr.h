@@ -188,7 +188,9 @@ amg_status amg_export_level_vec(amg_ctx *ctx, int32_t level, int32_t *d_agg, uin
  * Otherwise, after a full setup, when every offset fits in 16 bits, the
  * offsets themselves are read: *col_bytes = 2 (the coarser levels use the
  * same rule).  Otherwise the int32 columns: *col_bytes = 4; *noffsets = 0 in
- * both cases.  Values and arithmetic are the same either way.
+ * both cases.  A pattern of at most eight offsets that its rows fill to three
+ * quarters is held by diagonals instead, with one byte a row naming the offsets
+ * present (reported as *col_bytes = 1 and *noffsets the same).  Values and arithmetic are the same either way.
  * AMG_ERR_STATE before a pattern is set. */
 amg_status amg_pattern_info(const amg_ctx *ctx, int32_t *col_bytes, int32_t *noffsets);
 /* Coarsest LU factors (n_L x n_L row-major, FP64) and pivots. */

@@ -66,6 +66,11 @@ struct amg_ctx {
     int32_t *fine_coff = nullptr, *coff_table = nullptr;
     int *coff_count = nullptr;
     int fine_ncoff = 0;
+    // ... or the stencil form, when they are at most kMaxStencil and the rows
+    // fill it: the finest level's kernels then read its values by diagonals
+    Stencil sten;
+    uint8_t *sten_mask = nullptr;
+    bool a_val_stale = false;  // stencil form: A_val (CSR) is older than S_val
     // hierarchy
     int nlev = 0;
     Level lev[kMaxLevels];
@@ -76,6 +81,7 @@ struct amg_ctx {
     // system matrix of the solve (aliases level 0 except under full reuse)
     double *A_sys = nullptr;
     double *A_sys_own = nullptr;
+    double *S_sys = nullptr, *S_sys_own = nullptr;  // the same by diagonals (stencil form)
     // CG
     double *cg_r = nullptr, *cg_z = nullptr, *cg_p = nullptr, *cg_q = nullptr, *cg_t = nullptr;
     // per-block partial sums of the CG reductions, one set per reduction so
@@ -206,6 +212,7 @@ void free_hierarchy(amg_ctx *ctx) {
     ctx->lu = ctx->inv = ctx->luT = nullptr;
     ctx->piv = nullptr;
     ctx->graph_valid = false;
+    ctx->a_val_stale = false;
 }
 
 // read the device status word (synchronises the stream) and map it
@@ -418,7 +425,18 @@ amg_status numeric_rebuild(amg_ctx *ctx, const double *d_val, bool galerkin, con
     const amg_params &p = ctx->prm;
     Level &F = ctx->lev[0];
     const bool mx = mixed(ctx);
+    const bool sten = F.sten.noff > 0;
+    // a stencil's values go to their diagonals only; the finest stage 1 reads
+    // the caller's CSR values (FP64) or their FP32 copy
+    const double *a64 = sten ? d_val : F.A_val;
+    if (sten && d_val != F.A_val) ctx->a_val_stale = true;
     auto ingest = [&](int32_t r0, int32_t r1) {
+        if (sten) {
+            launch_ingest_stencil(r0, r1, F.A_ptr, d_val, F.sten, p.smoother, p.jacobi_omega, F.S_val,
+                                  mx ? F.S_valf : nullptr, mx ? F.A_valf : nullptr, mx ? nullptr : F.m,
+                                  mx ? F.mf : nullptr, ctx->d_st, ctx->s);
+            return;
+        }
         launch_ingest_fine(r0, r1, F.A_ptr, d_val, F.dia, p.smoother, p.jacobi_omega,
                            d_val == F.A_val ? nullptr : F.A_val, mx ? F.A_valf : nullptr, mx ? nullptr : F.m,
                            mx ? F.mf : nullptr, ctx->d_st, ctx->s);
@@ -433,7 +451,7 @@ amg_status numeric_rebuild(amg_ctx *ctx, const double *d_val, bool galerkin, con
             if (!ck_ap) continue;
             const int64_t e0 = ck->ap[c], ne = (int64_t)ck->ap[c + 1] - e0;
             if (mx) launch_gather_apply<float>(ne, F.g1_ptr + e0, F.g1_idx, F.g1_wf, F.A_valf, F.AP_valf + e0, ctx->s);
-            else launch_gather_apply<double>(ne, F.g1_ptr + e0, F.g1_idx, F.g1_w, F.A_val, F.AP_val + e0, ctx->s);
+            else launch_gather_apply<double>(ne, F.g1_ptr + e0, F.g1_idx, F.g1_w, a64, F.AP_val + e0, ctx->s);
             // the coarse rows whose A P rows are now all there
             Level &C1 = ctx->lev[1];
             const int64_t o0 = ck->ac[c], no = (int64_t)ck->ac[c + 1] - o0;
@@ -454,7 +472,7 @@ amg_status numeric_rebuild(amg_ctx *ctx, const double *d_val, bool galerkin, con
                 if (s1) { ProfScope ps_(ctx, AMG_PROF_AP_L0, l == 0); launch_gather_apply<float>(L.nnzAP, L.g1_ptr, L.g1_idx, L.g1_wf, L.A_valf, L.AP_valf, ctx->s); }
                 if (s1) { ProfScope ps_(ctx, AMG_PROF_RAP_L0, l == 0); launch_gather_apply<float>(C.nnz, L.g2_ptr, L.g2_idx, L.g2_wf, L.AP_valf, C.A_valf, ctx->s); }
             } else {
-                if (s1) { ProfScope ps_(ctx, AMG_PROF_AP_L0, l == 0); launch_gather_apply<double>(L.nnzAP, L.g1_ptr, L.g1_idx, L.g1_w, L.A_val, L.AP_val, ctx->s); }
+                if (s1) { ProfScope ps_(ctx, AMG_PROF_AP_L0, l == 0); launch_gather_apply<double>(L.nnzAP, L.g1_ptr, L.g1_idx, L.g1_w, l == 0 ? a64 : L.A_val, L.AP_val, ctx->s); }
                 if (s1) { ProfScope ps_(ctx, AMG_PROF_RAP_L0, l == 0); launch_gather_apply<double>(C.nnz, L.g2_ptr, L.g2_idx, L.g2_w, L.AP_val, C.A_val, ctx->s); }
             }
         } else if (galerkin) {
@@ -462,7 +480,7 @@ amg_status numeric_rebuild(amg_ctx *ctx, const double *d_val, bool galerkin, con
                 { ProfScope ps_(ctx, AMG_PROF_AP_L0, l == 0); launch_ap_numeric_f32(L, L.A_valf, ctx->s); }
                 { ProfScope ps_(ctx, AMG_PROF_RAP_L0, l == 0); launch_rap_numeric_f32(L, C.A_ptr, C.A_valf, ctx->s); }
             } else {
-                { ProfScope ps_(ctx, AMG_PROF_AP_L0, l == 0); launch_ap_numeric_f64(L, L.A_val, ctx->s); }
+                { ProfScope ps_(ctx, AMG_PROF_AP_L0, l == 0); launch_ap_numeric_f64(L, l == 0 ? a64 : L.A_val, ctx->s); }
                 { ProfScope ps_(ctx, AMG_PROF_RAP_L0, l == 0); launch_rap_numeric_f64(L, C.A_ptr, C.A_val, ctx->s); }
             }
         }
@@ -492,7 +510,7 @@ amg_status build_delta16(amg_ctx *ctx) {
     float ratio[kMaxLevels] = {};
     for (int l = 0; l < ctx->nlev; ++l) {
         Level &L = ctx->lev[l];
-        if (!L.A_cidx && L.n > 0 && L.nnz > 0) {
+        if (!L.A_cidx && !L.sten.noff && L.n > 0 && L.nnz > 0) {
             TRY(alloc(ctx, &buf[l], (size_t)L.nnz));
             launch_col_delta16(L.n, L.A_ptr, L.A_col, 0.0f, buf[l], flags + l, ctx->s);
         }
@@ -527,7 +545,11 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
     F.nnz = nnz;
     F.A_ptr = ctx->fine_ptr;
     F.A_col = ctx->fine_col;
-    if (ctx->fine_ncoff) {
+    if (ctx->sten.noff) {
+        F.sten = ctx->sten;
+        TRY(alloc(ctx, &F.S_val, F.sten.nvals(n)));
+        if (mixed(ctx)) TRY(alloc(ctx, &F.S_valf, F.sten.nvals(n)));
+    } else if (ctx->fine_ncoff) {
         F.A_cidx = ctx->fine_cidx;
         F.A_coff = ctx->fine_coff;
         F.A_ncoff = ctx->fine_ncoff;
@@ -701,6 +723,8 @@ amg_status ensure_persistent(amg_ctx *ctx, int32_t n, int32_t nnz) {
     ctx->fine_coff = ctx->coff_table = nullptr;
     ctx->coff_count = nullptr;
     ctx->fine_ncoff = 0;
+    ctx->sten = Stencil{};
+    ctx->sten_mask = nullptr;
     ctx->n = n;
     ctx->nnz = nnz;
     TRY(alloc(ctx, &ctx->fine_ptr, (size_t)n + 1, true));
@@ -715,7 +739,7 @@ amg_status ensure_persistent(amg_ctx *ctx, int32_t n, int32_t nnz) {
     TRY(alloc(ctx, &ctx->cg_u, nv, true));
     ctx->graph_valid = false;
     {
-        const size_t nb = (size_t)cg_blocks((int64_t)nv);
+        const size_t nb = (size_t)kCgMaxBlocks;
         TRY(alloc(ctx, &ctx->partial, 5 * nb, true));
         ctx->part_pq = ctx->partial;
         ctx->part_rr = ctx->partial + nb;
@@ -736,8 +760,29 @@ amg_status ensure_persistent(amg_ctx *ctx, int32_t n, int32_t nnz) {
     TRY(alloc(ctx, &ctx->stage_val, nvals(ctx), true));
     TRY(alloc(ctx, &ctx->stage_f, nv, true));
     TRY(alloc(ctx, &ctx->stage_u, nv, true));
-    ctx->A_sys_own = nullptr;
+    ctx->A_sys_own = ctx->S_sys_own = nullptr;
     if (ctx->prm.mode == AMG_MODE_FULL_REUSE) TRY(alloc(ctx, &ctx->A_sys_own, nvals(ctx), true));
+    return AMG_OK;
+}
+
+// The stencil form of a pattern with few offsets: where its rows fill at least
+// three quarters of the diagonals (so that reading the absent entries' zeros
+// costs less than the row pointers and column bytes it saves).
+amg_status stencil_pattern(amg_ctx *ctx, const std::vector<int32_t> &off) {
+    ctx->sten = Stencil{};
+    if (off.size() > (size_t)kMaxStencil || 4 * (int64_t)ctx->nnz < 3 * (int64_t)ctx->n * (int64_t)off.size())
+        return AMG_OK;
+    Stencil S;
+    S.noff = (int)off.size();
+    for (int d = 0; d < S.noff; ++d) S.off[d] = off[(size_t)d];
+    if (!ctx->sten_mask) TRY(alloc(ctx, &ctx->sten_mask, (size_t)ctx->n, true));
+    S.mask = ctx->sten_mask;
+    TRY(reset_status(ctx));
+    launch_stencil_mask(ctx->n, ctx->fine_ptr, ctx->fine_col, S, ctx->sten_mask, ctx->d_st, ctx->s);
+    TRY(check_device(ctx, "stencil pattern"));
+    if (ctx->A_sys_own && !ctx->S_sys_own)
+        TRY(alloc(ctx, &ctx->S_sys_own, (size_t)(((int64_t)ctx->n + 31) / 32 * 32 * kMaxStencil), true));
+    ctx->sten = S;
     return AMG_OK;
 }
 
@@ -748,6 +793,7 @@ amg_status ensure_persistent(amg_ctx *ctx, int32_t n, int32_t nnz) {
 // finest level's matrix kernels then move 3 bytes less per entry.
 amg_status compress_pattern(amg_ctx *ctx) {
     ctx->fine_ncoff = 0;
+    ctx->sten = Stencil{};
     if (blockmode(ctx) || ctx->n >= (1 << 30)) return AMG_OK;
     if (!ctx->fine_cidx) {
         TRY(alloc(ctx, &ctx->fine_cidx, (size_t)ctx->nnz, true));
@@ -769,6 +815,11 @@ amg_status compress_pattern(amg_ctx *ctx) {
         if (v != kColOffsetEmpty) off.push_back(v);
     if ((int)off.size() != cnt) return AMG_OK;
     std::sort(off.begin(), off.end());
+    TRY(stencil_pattern(ctx, off));
+    if (ctx->sten.noff) {
+        ctx->fine_ncoff = cnt;
+        return AMG_OK;
+    }
     CK(cudaMemcpyAsync(ctx->fine_coff, off.data(), sizeof(int32_t) * off.size(), cudaMemcpyHostToDevice, ctx->s));
     TRY(reset_status(ctx));
     launch_col_offsets_encode(ctx->n, ctx->fine_ptr, ctx->fine_col, ctx->fine_coff, cnt, ctx->fine_cidx, ctx->d_st,
@@ -796,14 +847,38 @@ amg_status set_pattern(amg_ctx *ctx, int32_t n, int32_t nnz, const int32_t *d_pt
     return AMG_OK;
 }
 
-// the finest level's column indices as the matrix kernels read them
-ColIdx fine_cols(const amg_ctx *ctx) {
-    return ColIdx{ctx->fine_col, ctx->fine_ncoff ? ctx->fine_cidx : nullptr, ctx->fine_coff, ctx->fine_ncoff,
-                  ctx->nlev > 0 ? ctx->lev[0].A_c16 : nullptr};
+// the system matrix as the Krylov kernels read it
+FineMat fine_mat(const amg_ctx *ctx) {
+    FineMat A;
+    A.ptr = ctx->fine_ptr;
+    A.col.col = ctx->fine_col;
+    A.val = ctx->A_sys;
+    A.sten = ctx->sten;
+    A.sval = ctx->S_sys;
+    if (!ctx->sten.noff && ctx->fine_ncoff) {
+        A.col.cidx = ctx->fine_cidx;
+        A.col.off = ctx->fine_coff;
+        A.col.noff = ctx->fine_ncoff;
+    } else if (ctx->nlev > 0) {
+        A.col.c16 = ctx->lev[0].A_c16;
+    }
+    return A;
 }
 
 void update_sys(amg_ctx *ctx) {
     ctx->A_sys = ctx->A_sys_own ? ctx->A_sys_own : blockmode(ctx) ? ctx->lev[0].Ab : ctx->lev[0].A_val;
+    ctx->S_sys = ctx->A_sys_own ? ctx->S_sys_own : ctx->lev[0].S_val;
+}
+
+// full reuse: the system matrix is apart from the hierarchy's
+amg_status copy_sys(amg_ctx *ctx, const double *d_val) {
+    if (!ctx->A_sys_own) return AMG_OK;
+    if (ctx->sten.noff) {
+        launch_csr_to_stencil(ctx->n, ctx->fine_ptr, d_val, ctx->sten, ctx->S_sys_own, ctx->s);
+        return AMG_OK;
+    }
+    CK(cudaMemcpyAsync(ctx->A_sys_own, d_val, sizeof(double) * nvals(ctx), cudaMemcpyDeviceToDevice, ctx->s));
+    return AMG_OK;
 }
 
 // ---------------------------------------------------------------- V-cycle
@@ -1038,8 +1113,7 @@ void enqueue_cg_iter_a(amg_ctx *ctx, double *u, int use_h, cudaGraphConditionalH
     CgState *cg = ctx->cg;
     {
         ProfScope ps_(ctx, AMG_PROF_CG_SPMV, true);
-        launch_spmv_dot(n, ctx->fine_ptr, fine_cols(ctx), ctx->A_sys, ctx->cg_p, ctx->cg_q, ctx->part_pq, cg,
-                        ctx->s);
+        launch_spmv_dot(n, fine_mat(ctx), ctx->cg_p, ctx->cg_q, ctx->part_pq, cg, ctx->s);
     }
     {
         ProfScope ps_(ctx, AMG_PROF_CG_UPDATE, true);
@@ -1055,8 +1129,7 @@ void enqueue_cg_iter_a(amg_ctx *ctx, double *u, int use_h, cudaGraphConditionalH
 void enqueue_cg_iter_b(amg_ctx *ctx, const double *f, double *u) {
     const int32_t n = ctx->n;
     CgState *cg = ctx->cg;
-    launch_true_residual(n, ctx->fine_ptr, fine_cols(ctx), ctx->A_sys, f, u, ctx->cg_t, ctx->part_tt,
-                         cg, 0, ctx->s);
+    launch_true_residual(n, fine_mat(ctx), f, u, ctx->cg_t, ctx->part_tt, cg, 0, ctx->s);
     launch_replace_r(n, cg, ctx->cg_t, ctx->cg_r, mixed(ctx) ? ctx->cg_z : nullptr, ctx->part_rzo, cg_smooth0(ctx),
                      ctx->s);
 }
@@ -1076,9 +1149,7 @@ void enqueue_cg_iter_c(amg_ctx *ctx, int use_h, cudaGraphConditionalHandle h) {
 // the true relative residual of the returned iterate
 void enqueue_cg_epilogue(amg_ctx *ctx, const double *f, double *u) {
     const int32_t n = ctx->n;
-    launch_true_residual(n, ctx->fine_ptr, fine_cols(ctx), ctx->A_sys, f, u, ctx->cg_t, ctx->part_tt,
-                         ctx->cg, 1,
-                         ctx->s);
+    launch_true_residual(n, fine_mat(ctx), f, u, ctx->cg_t, ctx->part_tt, ctx->cg, 1, ctx->s);
 }
 
 void drop_graph(amg_ctx *ctx) {
@@ -1252,19 +1323,19 @@ void enqueue_bi_iter(amg_ctx *ctx, const double *f, double *u, int use_h, cudaGr
     launch_bi_rho(n, ctx->bi_rh, ctx->cg_r, part, st, ctx->s);
     launch_bi_p(n, ctx->cg_r, ctx->cg_q, ctx->cg_p, st, ctx->s);
     vcycle(ctx, ctx->cg_p, ctx->cg_z, &st->done);
-    launch_bi_spmv_rv(n, bs, ctx->fine_ptr, ctx->fine_col, ctx->A_sys, ctx->cg_z, ctx->cg_q, ctx->bi_rh, part, st, ctx->s);
+    launch_bi_spmv_rv(n, bs, fine_mat(ctx), ctx->cg_z, ctx->cg_q, ctx->bi_rh, part, st, ctx->s);
     launch_bi_s(n, ctx->cg_r, ctx->cg_q, ctx->bi_s, part, st, ctx->s);
     launch_bi_half(n, ctx->cg_z, ctx->bi_s, u, ctx->cg_r, st, ctx->s);
     vcycle(ctx, ctx->bi_s, ctx->bi_sh, &st->skip);
-    launch_bi_spmv_t(n, bs, ctx->fine_ptr, ctx->fine_col, ctx->A_sys, ctx->bi_sh, ctx->bi_s, ctx->cg_t, part, st, ctx->s);
+    launch_bi_spmv_t(n, bs, fine_mat(ctx), ctx->bi_sh, ctx->bi_s, ctx->cg_t, part, st, ctx->s);
     launch_bi_xr(n, ctx->cg_z, ctx->bi_sh, ctx->bi_s, ctx->cg_t, u, ctx->cg_r, part, st, ctx->s);
-    launch_bi_true(n, bs, ctx->fine_ptr, ctx->fine_col, ctx->A_sys, f, u, ctx->cg_t, part, st, 0, ctx->s);
+    launch_bi_true(n, bs, fine_mat(ctx), f, u, ctx->cg_t, part, st, 0, ctx->s);
     launch_bi_replace(n, ctx->cg_t, ctx->cg_r, st, ctx->s);
     launch_bi_end(st, use_h, h, ctx->s);
 }
 
 void enqueue_bi_epilogue(amg_ctx *ctx, const double *f, double *u) {
-    launch_bi_true((int32_t)nvec(ctx), ctx->prm.block_size, ctx->fine_ptr, ctx->fine_col, ctx->A_sys, f, u, ctx->cg_t, ctx->partial, ctx->bi, 1,
+    launch_bi_true((int32_t)nvec(ctx), ctx->prm.block_size, fine_mat(ctx), f, u, ctx->cg_t, ctx->partial, ctx->bi, 1,
                    ctx->s);
 }
 
@@ -1569,8 +1640,7 @@ amg_status amg_full_setup(amg_ctx *ctx, int32_t n, int32_t nnz, const int32_t *d
         free_hierarchy(ctx);
         return st;
     }
-    if (ctx->A_sys_own)
-        CK(cudaMemcpyAsync(ctx->A_sys_own, d_val, sizeof(double) * nvals(ctx), cudaMemcpyDeviceToDevice, ctx->s));
+    TRY(copy_sys(ctx, d_val));
     update_sys(ctx);
     ctx->last_rebuilt = 1;
     ctx->steps_since_full = 0;
@@ -1596,9 +1666,7 @@ amg_status partial_rebuild_impl(amg_ctx *ctx, const double *d_val, const FineChu
         for (int l = 0; l + 1 < ctx->nlev; ++l)
             if (!ctx->lev[l].gather_ready) TRY(build_gather(ctx, l));
     TRY(numeric_rebuild(ctx, d_val, true, ck));
-    if (ctx->A_sys_own)
-        CK(cudaMemcpyAsync(ctx->A_sys_own, d_val, sizeof(double) * nvals(ctx), cudaMemcpyDeviceToDevice,
-                           ctx->s));
+    TRY(copy_sys(ctx, d_val));
     TRY(check_device(ctx, "partial rebuild"));
     update_sys(ctx);
     ctx->last_rebuilt = 0;
@@ -1705,8 +1773,7 @@ amg_status amg_step(amg_ctx *ctx, int32_t n, int32_t nnz, const int32_t *d_ptr, 
             if (st != AMG_OK) free_hierarchy(ctx);
         }
         if (st == AMG_OK) {
-            CK(cudaMemcpyAsync(ctx->A_sys_own, d_val, sizeof(double) * nvals(ctx), cudaMemcpyDeviceToDevice,
-                               ctx->s));
+            TRY(copy_sys(ctx, d_val));
             update_sys(ctx);
             ctx->last_rebuilt = rebuild ? 1 : 0;
         }
@@ -1841,6 +1908,11 @@ amg_status amg_export_csr(amg_ctx *ctx, int32_t level, int32_t which, int32_t *d
     if (d_ptr) CK(cudaMemcpyAsync(d_ptr, ptr, sizeof(int32_t) * ((size_t)nrows + 1), cudaMemcpyDeviceToDevice, ctx->s));
     if (d_col) CK(cudaMemcpyAsync(d_col, col, sizeof(int32_t) * (size_t)nnz, cudaMemcpyDeviceToDevice, ctx->s));
     if (d_val) {
+        if (which == 0 && level == 0 && ctx->a_val_stale) {
+            // a stencil's last values are held by diagonals
+            launch_stencil_to_csr(L.n, L.A_ptr, L.S_val, L.sten, L.A_val, ctx->s);
+            ctx->a_val_stale = false;
+        }
         if (blockmode(ctx) && which == 0)
             CK(cudaMemcpyAsync(d_val, L.Ab, sizeof(double) * 16 * (size_t)nnz, cudaMemcpyDeviceToDevice, ctx->s));
         else if (mixed(ctx) && valf) launch_copy_cast<float, double>(nnz, valf, d_val, nullptr, ctx->s);

@@ -63,6 +63,27 @@ struct ColIdx {
     const int16_t *c16 = nullptr;
 };
 
+// A stencil's matrix by diagonals: every row's columns are row + off[d] for the
+// d set in the row's mask byte (offsets ascending, so d runs in column order).
+// Values of the 32 rows of slice i / 32 lie diagonal by diagonal, entry d of
+// row i at ((i / 32) * noff + d) * 32 + i % 32, zero where the row has none.
+// A warp's loads of values and of the vector are then whole lines, a row needs
+// one byte of pattern, and nothing has to be read before the loads can start;
+// with CSR rows of 7 entries each load of a warp touched 7 (FP32) or 14 (FP64)
+// lines, and the finest level's kernels were bound by those L1 accesses.
+// Measured at 192^3 (mixed) per launch, CSR -> diagonals: residual 77.4 -> 50.8
+// us (6.28 TB/s, 92% of the measured copy), sweep with r.z 72.8 -> 62.9, q = A p
+// 118.8 -> 116.1 (8 FP64 operations a row: the FP64 pipe bounds it near 106);
+// 64^3 (FP64): 7.7 -> 6.1, 11.0 -> 10.3, 12.4 -> 11.4.
+// noff = 0: the pattern is no such stencil.
+constexpr int kMaxStencil = 8;
+struct Stencil {
+    int noff = 0;
+    int32_t off[kMaxStencil] = {};
+    const uint8_t *mask = nullptr;
+    size_t nvals(int64_t n) const { return (size_t)((n + 31) / 32) * 32 * (size_t)noff; }
+};
+
 template <class V>
 struct VecSet {
     V *u = nullptr, *f = nullptr, *r = nullptr, *t = nullptr;
@@ -80,6 +101,10 @@ struct Level {
     ColIdx cols() const { return ColIdx{A_col, A_cidx, A_coff, A_ncoff, A_c16}; }
     double *A_val = nullptr;   // FP64 values (level 0: the hierarchy's copy of the fine matrix)
     float *A_valf = nullptr;   // FP32 values (mixed precision)
+    // the finest level's values by diagonals, when its pattern is a stencil
+    Stencil sten;
+    double *S_val = nullptr;
+    float *S_valf = nullptr;
     // transfer operators (absent on the coarsest level)
     int32_t nc = 0, nnzP = 0, nnzR = 0, nnzAP = 0;
     int32_t *P_ptr = nullptr, *P_col = nullptr;
@@ -237,6 +262,18 @@ void launch_smoother_f32(int32_t n, const int32_t *ptr, const float *val, const 
 void launch_ingest_fine(int32_t row0, int32_t row1, const int32_t *ptr, const double *val_in, const int32_t *dia,
                         int type, double wj, double *val_out, float *valf_out, double *m, float *mf, int *st,
                         cudaStream_t s);
+// the same for a stencil pattern: the values by diagonals (and their FP32 copy),
+// and the FP32 copy in CSR order
+void launch_ingest_stencil(int32_t row0, int32_t row1, const int32_t *ptr, const double *val_in, const Stencil &S,
+                           int type, double wj, double *sval, float *svalf, float *valf_out, double *m, float *mf,
+                           int *st, cudaStream_t s);
+// a stencil pattern's row masks; CSR values to diagonals and back
+void launch_stencil_mask(int32_t n, const int32_t *ptr, const int32_t *col, const Stencil &S, uint8_t *mask, int *st,
+                         cudaStream_t s);
+void launch_csr_to_stencil(int32_t n, const int32_t *ptr, const double *val, const Stencil &S, double *sval,
+                           cudaStream_t s);
+void launch_stencil_to_csr(int32_t n, const int32_t *ptr, const double *sval, const Stencil &S, double *val,
+                           cudaStream_t s);
 void launch_cast_f32(int64_t n, const double *in, float *out, cudaStream_t s);
 
 // coarsest level: dense LU and explicit inverse
@@ -274,6 +311,16 @@ void launch_copy_cast(int64_t n, const TI *in, TO *out, const int *skip, cudaStr
 
 // CG (FP64); reductions finish in the last block of the producing kernel
 int cg_blocks(int64_t n);
+constexpr int kCgMaxBlocks = 152 * 4;  // the most blocks (and so partials) of a Krylov kernel
+// the system matrix as the Krylov kernels read it: by diagonals (sval) when its
+// pattern is a stencil, else CSR
+struct FineMat {
+    const int32_t *ptr = nullptr;
+    ColIdx col;
+    const double *val = nullptr;
+    Stencil sten;
+    const double *sval = nullptr;
+};
 // The V-cycle's first pre-smoothing step from u = 0 on the finest level,
 // u0 = m o r, written by the kernel that produces r (so that step needs no
 // per-entry product); at most one of the two pointer pairs is set.
@@ -290,8 +337,8 @@ void launch_cg_init(int32_t n, const double *f, double *u, double *r, double *pa
 void launch_dot(int32_t n, const double *x, const double *y, double *partial, const int *skip, CgState *cg, int target,
                 cudaStream_t s);
 void launch_cg_set_rz_p(int32_t n, const double *z, double *p, CgState *cg, cudaStream_t s);
-void launch_spmv_dot(int32_t n, const int32_t *ptr, const ColIdx &col, const double *val, const double *p,
-                     double *q, double *partial, CgState *cg, cudaStream_t s);
+void launch_spmv_dot(int32_t n, const FineMat &A, const double *p, double *q, double *partial, CgState *cg,
+                     cudaStream_t s);
 // the compressed form of a pattern: collect the distinct offsets column - row
 // into an open-addressed table of kColOffsetSlots ints (empty:
 // kColOffsetEmpty, the int of four 0x80 bytes; *count the distinct keys,
@@ -312,8 +359,8 @@ void launch_col_offsets_encode(int32_t n, const int32_t *ptr, const int32_t *col
 void launch_cg_update_ur(int32_t n, CgState *cg, const double *p, const double *q, double *u, double *r,
                          double *partial, const double *zo, double *part_zo, int use_h, cudaGraphConditionalHandle hb,
                          const Smooth0Out &z0, cudaStream_t s);
-void launch_true_residual(int32_t n, const int32_t *ptr, const ColIdx &col, const double *val, const double *f,
-                          const double *u, double *t, double *partial, CgState *cg, int force, cudaStream_t s);
+void launch_true_residual(int32_t n, const FineMat &A, const double *f, const double *u, double *t, double *partial,
+                          CgState *cg, int force, cudaStream_t s);
 void launch_replace_r(int32_t n, CgState *cg, const double *t, double *r, const double *zo, double *part_zo,
                       const Smooth0Out &z0, cudaStream_t s);
 void launch_cg_update_p(int32_t n, CgState *cg, const double *z, double *p, int use_h, cudaGraphConditionalHandle h,
@@ -324,17 +371,17 @@ void launch_bi_init(int32_t n, const double *f, double *x, double *r, double *rh
                     double *partial, BiState *st, double tol, int maxiter, cudaStream_t s);
 void launch_bi_rho(int32_t n, const double *rh, const double *r, double *partial, BiState *st, cudaStream_t s);
 void launch_bi_p(int32_t n, const double *r, const double *v, double *p, BiState *st, cudaStream_t s);
-void launch_bi_spmv_rv(int32_t n, int bs, const int32_t *ptr, const int32_t *col, const double *val,
-                       const double *ph, double *v, const double *rh, double *partial, BiState *st, cudaStream_t s);
+void launch_bi_spmv_rv(int32_t n, int bs, const FineMat &A, const double *ph, double *v, const double *rh,
+                       double *partial, BiState *st, cudaStream_t s);
 void launch_bi_s(int32_t n, const double *r, const double *v, double *sv, double *partial, BiState *st,
                  cudaStream_t s);
 void launch_bi_half(int32_t n, const double *ph, const double *sv, double *x, double *r, BiState *st, cudaStream_t s);
-void launch_bi_spmv_t(int32_t n, int bs, const int32_t *ptr, const int32_t *col, const double *val,
-                      const double *sh, const double *sv, double *t, double *partial, BiState *st, cudaStream_t s);
+void launch_bi_spmv_t(int32_t n, int bs, const FineMat &A, const double *sh, const double *sv, double *t,
+                      double *partial, BiState *st, cudaStream_t s);
 void launch_bi_xr(int32_t n, const double *ph, const double *sh, const double *sv, const double *t, double *x,
                   double *r, double *partial, BiState *st, cudaStream_t s);
-void launch_bi_true(int32_t n, int bs, const int32_t *ptr, const int32_t *col, const double *val, const double *f,
-                    const double *x, double *t, double *partial, BiState *st, int force, cudaStream_t s);
+void launch_bi_true(int32_t n, int bs, const FineMat &A, const double *f, const double *x, double *t, double *partial,
+                    BiState *st, int force, cudaStream_t s);
 void launch_bi_replace(int32_t n, const double *t, double *r, BiState *st, cudaStream_t s);
 void launch_bi_end(BiState *st, int use_h, cudaGraphConditionalHandle h, cudaStream_t s);
 // (BiCGStab vectors have n = bs * nodes entries; bs = 4 for the block matrix)

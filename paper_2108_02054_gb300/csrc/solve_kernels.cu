@@ -20,6 +20,7 @@ namespace amgpr {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kCgThreads = 512;
 
 inline int nblocks(int64_t n, int t = kThreads) {
     int64_t b = (n + t - 1) / t;
@@ -352,6 +353,106 @@ __global__ void k_ingest_fine(int32_t row0, int32_t n, const int32_t *__restrict
     else mi = aii != 0.0 ? div_rn(wj, div_recip(aii)) : 0.0;
     if (m) m[i] = mi;
     if (mf) mf[i] = f64_to_f32_rn(mi);
+}
+
+// fine level of a stencil pattern: one warp per slice of 32 rows reads the
+// slice's contiguous CSR values once (coalesced, through shared memory), flags
+// non-finite entries, and writes the values by diagonals (and the FP32 copies)
+// with the smoother, each row's squares summed in column order
+constexpr int kIngestWarps = 8;
+template <int NOFF>
+__global__ void __launch_bounds__(kIngestWarps * 32)
+k_ingest_stencil(int32_t row0, int32_t n, const int32_t *__restrict__ ptr, const double *__restrict__ in, Stencil S,
+                 int type, double wj, double *__restrict__ sval, float *__restrict__ svalf,
+                 float *__restrict__ valf_out, double *__restrict__ m, float *__restrict__ mf, int *st) {
+    __shared__ double buf[kIngestWarps][32 * NOFF];
+    __shared__ float buff[kIngestWarps][32 * NOFF];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int noff = NOFF == kMaxStencil ? S.noff : NOFF;
+    const int32_t r0 = row0 + (int32_t)((((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) << 5);
+    if (r0 >= n) return;  // warp-uniform
+    const int32_t i = r0 + lane;
+    const bool row = i < n;
+    const int32_t p0 = ptr[r0], p1 = ptr[min(r0 + 32, n)];
+    const unsigned mk = row ? S.mask[i] : 0u;
+    int32_t k = row ? ptr[i] - p0 : 0;
+    bool finite = true;
+#pragma unroll
+    for (int c = 0; c < NOFF; ++c) {  // a slice holds at most 32 noff values
+        const int32_t p = p0 + c * 32 + lane;
+        if (p < p1) {
+            const double v = in[p];
+            finite = finite && finite_bits(v);
+            buf[w][p - p0] = v;
+            if (svalf) {
+                const float vf = f64_to_f32_rn(v);
+                buff[w][p - p0] = vf;
+                valf_out[p] = vf;
+            }
+        }
+    }
+    if (__any_sync(0xffffffffu, !finite) && lane == 0) atomicOr(st, DEV_ERR_NONFINITE);
+    __syncwarp();
+    const size_t base = (size_t)(r0 >> 5) * (size_t)noff * 32 + lane;
+    double s = 0.0, aii = 0.0;
+#pragma unroll
+    for (int d = 0; d < NOFF; ++d) {
+        if (NOFF == kMaxStencil && d >= noff) break;
+        double v = 0.0;
+        float vf = 0.f;
+        if ((mk >> d) & 1u) {
+            v = buf[w][k];
+            if (svalf) vf = buff[w][k];
+            ++k;
+            s = fma(v, v, s);
+            if (S.off[d] == 0) aii = v;
+        }
+        sval[base + (size_t)d * 32] = v;
+        if (svalf) svalf[base + (size_t)d * 32] = vf;
+    }
+    if (!row) return;
+    double mi;
+    if (type == AMG_SMOOTHER_SPAI0) mi = s != 0.0 ? div_rn(aii, div_recip(s)) : 0.0;
+    else mi = aii != 0.0 ? div_rn(wj, div_recip(aii)) : 0.0;
+    if (m) m[i] = mi;
+    if (mf) mf[i] = f64_to_f32_rn(mi);
+}
+
+// row masks of a stencil pattern (an offset missing from the table flags the status word)
+__global__ void k_stencil_mask(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col, Stencil S,
+                               uint8_t *__restrict__ mask, int *st) {
+    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    unsigned m = 0u;
+    for (int32_t p = ptr[i]; p < ptr[i + 1]; ++p) {
+        const int32_t d = col[p] - i;
+        unsigned bit = 0u;
+#pragma unroll
+        for (int k = 0; k < kMaxStencil; ++k)
+            if (k < S.noff && S.off[k] == d) bit = 1u << k;
+        if (bit == 0u || (m & bit)) atomicOr(st, DEV_ERR_STATE);
+        m |= bit;
+    }
+    mask[i] = (uint8_t)m;
+}
+__global__ void k_csr_to_stencil(int32_t n, const int32_t *__restrict__ ptr, const double *__restrict__ val, Stencil S,
+                                 double *__restrict__ sval) {
+    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (n + 31) / 32 * 32) return;
+    const unsigned m = i < n ? S.mask[i] : 0u;
+    int32_t p = i < n ? ptr[i] : 0;
+    double *o = sval + (size_t)(i >> 5) * (size_t)S.noff * 32 + (i & 31);
+    for (int d = 0; d < S.noff; ++d) o[d * 32] = ((m >> d) & 1u) ? val[p++] : 0.0;
+}
+__global__ void k_stencil_to_csr(int32_t n, const int32_t *__restrict__ ptr, const double *__restrict__ sval, Stencil S,
+                                 double *__restrict__ val) {
+    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const unsigned m = S.mask[i];
+    int32_t p = ptr[i];
+    const double *o = sval + (size_t)(i >> 5) * (size_t)S.noff * 32 + (i & 31);
+    for (int d = 0; d < S.noff; ++d)
+        if ((m >> d) & 1u) val[p++] = o[d * 32];
 }
 
 __global__ void k_cast_f32(int64_t n, const double *__restrict__ in, float *__restrict__ out) {
@@ -1309,9 +1410,12 @@ __global__ void k_coarse_solve(int32_t n, const double *__restrict__ inv, const 
 }
 
 // ------------------------------------------------------------------ V-cycle pieces
-// Every matrix-vector piece takes LPR lanes per row (a power of two <= 32,
-// chosen per level from the row length and count): the lanes stride over the
-// row and combine with xor shuffles.  LPR = 1 is the plain sequential row sum.
+// Every matrix-vector piece takes the matrix as a row policy:
+//  - CsrRows: LPR lanes per row (a power of two <= 32, chosen per level from
+//    the row length and count): the lanes stride over the row and combine with
+//    xor shuffles.  LPR = 1 is the plain sequential row sum.
+//  - StencilRows (the finest level of a stencil pattern): one lane per row,
+//    every load of the row issued before the sum.
 template <int LPR, class V>
 __device__ __forceinline__ V group_sum(V s) {
 #pragma unroll
@@ -1319,24 +1423,86 @@ __device__ __forceinline__ V group_sum(V s) {
     return s;
 }
 
+template <class V, int LPR>
+struct CsrRows {
+    using value = V;
+    static constexpr int lanes = LPR;
+    const int32_t *__restrict__ ptr;
+    ColIdx ci;
+    const V *__restrict__ val;
+    __device__ __forceinline__ void stage(int32_t *s_off) const { stage_col_offsets(ci, s_off); }
+    // lane sub's part of row i's sum of a_ij x(j)
+    template <class X>
+    __device__ __forceinline__ V dot(const int32_t *s_off, int32_t i, int sub, X x) const {
+        V s = 0;
+        for (int32_t p = ptr[i] + sub; p < ptr[i + 1]; p += LPR) s = fma(val[p], x(col_at(ci, s_off, i, p)), s);
+        return s;
+    }
+};
+
+// NOFF diagonals (NOFF = kMaxStencil: any number up to it).  ORD > 1 forms the
+// sum in the order of ORD CSR lanes (part k % ORD of the row's k-th entry, then
+// the xor tree), so that FP32 results do not depend on which policy runs.
+template <class V, int NOFF, int ORD>
+struct StencilRows {
+    using value = V;
+    static constexpr int lanes = 1;
+    Stencil S;
+    const V *__restrict__ val;
+    int32_t n;
+    __device__ __forceinline__ void stage(int32_t *) const {}
+    template <class X>
+    __device__ __forceinline__ V dot(const int32_t *, int32_t i, int, X x) const {
+        const int noff = NOFF == kMaxStencil ? S.noff : NOFF;
+        const unsigned m = S.mask[i];
+        const V *__restrict__ a = val + ((size_t)(i >> 5) * (size_t)noff) * 32 + (i & 31);
+        // every load is issued at once and depends on nothing loaded: an absent
+        // entry's value is a stored zero and its column is clamped into range,
+        // and the mask only selects whose products enter the sum
+        V v[NOFF], xv[NOFF];
+#pragma unroll
+        for (int d = 0; d < NOFF; ++d) {
+            v[d] = (NOFF < kMaxStencil || d < noff) ? a[d * 32] : V(0);
+            xv[d] = x(min(max(i + S.off[d], 0), n - 1));
+        }
+        V acc[ORD];
+#pragma unroll
+        for (int q = 0; q < ORD; ++q) acc[q] = V(0);
+        int k = 0;
+#pragma unroll
+        for (int d = 0; d < NOFF; ++d) {
+            const bool has = (m >> d) & 1u;
+#pragma unroll
+            for (int q = 0; q < ORD; ++q) {
+                const V t = fma(v[d], xv[d], acc[q]);
+                acc[q] = has && (ORD == 1 || (k & (ORD - 1)) == q) ? t : acc[q];
+            }
+            if (ORD > 1) k += has;
+        }
+#pragma unroll
+        for (int o = ORD / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < o; ++q) acc[q] += acc[q + o];
+        return acc[0];
+    }
+};
+
 // zero-guess pre-smoothing fused with the residual: u = m o f, r = f - A u
-template <class V, class TF, int LPR>
-__global__ void k_smooth0_residual(int32_t n, const int32_t *__restrict__ ptr, ColIdx ci,
-                                   const V *__restrict__ val, const V *__restrict__ m, const TF *__restrict__ f,
-                                   V *__restrict__ u, V *__restrict__ r, const int *skip) {
+template <class M, class TF>
+__global__ void k_smooth0_residual(int32_t n, M A, const typename M::value *__restrict__ m, const TF *__restrict__ f,
+                                   typename M::value *__restrict__ u, typename M::value *__restrict__ r,
+                                   const int *skip) {
+    using V = typename M::value;
+    constexpr int LPR = M::lanes;
     __shared__ int32_t s_off[kMaxColOffsets];
     pdl_wait();
     if (skipped(skip)) return;
-    stage_col_offsets(ci, s_off);
+    A.stage(s_off);
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int32_t i = (int32_t)(gt / LPR);
     const int sub = (int)(gt % LPR);
     V s = 0;
-    if (i < n)
-        for (int32_t p = ptr[i] + sub; p < ptr[i + 1]; p += LPR) {
-            const int32_t j = col_at(ci, s_off, i, p);
-            s = fma(val[p], m[j] * (V)f[j], s);
-        }
+    if (i < n) s = A.dot(s_off, i, sub, [&](int32_t j) { return m[j] * (V)f[j]; });
     s = group_sum<LPR>(s);
     if (i < n && sub == 0) {
         const V fi = (V)f[i];
@@ -1346,21 +1512,20 @@ __global__ void k_smooth0_residual(int32_t n, const int32_t *__restrict__ ptr, C
 }
 
 // u_out = u_in + m o (f - A u_in)
-template <class V, class TF, class TO, int LPR>
-__global__ void k_smooth_sweep(int32_t n, const int32_t *__restrict__ ptr, ColIdx ci,
-                               const V *__restrict__ val, const V *__restrict__ m, const TF *__restrict__ f,
-                               const V *__restrict__ u_in, TO *__restrict__ u_out, const int *skip) {
+template <class M, class TF, class TO>
+__global__ void k_smooth_sweep(int32_t n, M A, const typename M::value *__restrict__ m, const TF *__restrict__ f,
+                               const typename M::value *__restrict__ u_in, TO *__restrict__ u_out, const int *skip) {
+    using V = typename M::value;
+    constexpr int LPR = M::lanes;
     __shared__ int32_t s_off[kMaxColOffsets];
     pdl_wait();
     if (skipped(skip)) return;
-    stage_col_offsets(ci, s_off);
+    A.stage(s_off);
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int32_t i = (int32_t)(gt / LPR);
     const int sub = (int)(gt % LPR);
     V s = 0;
-    if (i < n)
-        for (int32_t p = ptr[i] + sub; p < ptr[i + 1]; p += LPR)
-            s = fma(val[p], u_in[col_at(ci, s_off, i, p)], s);
+    if (i < n) s = A.dot(s_off, i, sub, [&](int32_t j) { return u_in[j]; });
     s = group_sum<LPR>(s);
     if (i < n && sub == 0) u_out[i] = (TO)fma(m[i], (V)f[i] - s, u_in[i]);
 }
@@ -1369,15 +1534,17 @@ __global__ void k_smooth_sweep(int32_t n, const int32_t *__restrict__ ptr, ColId
 // z = u_in + m o (r - A u_in) and a per-block partial of r.z (block_sum order)
 __device__ double block_sum(double v);
 __device__ bool cg_reduce(double d, double *partial, unsigned *counter, double *total);
-template <class V, int LPR>
-__global__ void k_smooth_sweep_dot(int32_t n, const int32_t *__restrict__ ptr, ColIdx ci,
-                                   const V *__restrict__ val, const V *__restrict__ m, const double *__restrict__ f,
-                                   const V *__restrict__ u_in, double *__restrict__ z, double *__restrict__ partial,
-                                   CgState *cg, const int *skip) {
+template <class M>
+__global__ void __launch_bounds__(kCgThreads)
+k_smooth_sweep_dot(int32_t n, M A, const typename M::value *__restrict__ m, const double *__restrict__ f,
+                   const typename M::value *__restrict__ u_in, double *__restrict__ z, double *__restrict__ partial,
+                   CgState *cg, const int *skip) {
+    using V = typename M::value;
+    constexpr int LPR = M::lanes;
     __shared__ int32_t s_off[kMaxColOffsets];
     pdl_wait();
     if (skipped(skip)) return;
-    stage_col_offsets(ci, s_off);
+    A.stage(s_off);
     const int64_t total = (int64_t)n * LPR;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     double d = 0.0;
@@ -1386,9 +1553,7 @@ __global__ void k_smooth_sweep_dot(int32_t n, const int32_t *__restrict__ ptr, C
         const int32_t i = (int32_t)(gt / LPR);
         const int sub = (int)(gt % LPR);
         V s = 0;
-        if (gt < total)
-            for (int32_t p = ptr[i] + sub; p < ptr[i + 1]; p += LPR)
-                s = fma(val[p], u_in[col_at(ci, s_off, i, p)], s);
+        if (gt < total) s = A.dot(s_off, i, sub, [&](int32_t j) { return u_in[j]; });
         s = group_sum<LPR>(s);
         if (gt < total && sub == 0) {
             const double fi = f[i];
@@ -1402,21 +1567,20 @@ __global__ void k_smooth_sweep_dot(int32_t n, const int32_t *__restrict__ ptr, C
     if (cg_reduce(d, partial, &cg->ctr[CG_CTR_RZ], &rz) && threadIdx.x == 0) cg->rz_next = rz;
 }
 
-template <class V, class TF, int LPR>
-__global__ void k_residual(int32_t n, const int32_t *__restrict__ ptr, ColIdx ci,
-                           const V *__restrict__ val, const TF *__restrict__ f, const V *__restrict__ u,
-                           V *__restrict__ r, const int *skip) {
+template <class M, class TF>
+__global__ void k_residual(int32_t n, M A, const TF *__restrict__ f, const typename M::value *__restrict__ u,
+                           typename M::value *__restrict__ r, const int *skip) {
+    using V = typename M::value;
+    constexpr int LPR = M::lanes;
     __shared__ int32_t s_off[kMaxColOffsets];
     pdl_wait();
     if (skipped(skip)) return;
-    stage_col_offsets(ci, s_off);
+    A.stage(s_off);
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int32_t i = (int32_t)(gt / LPR);
     const int sub = (int)(gt % LPR);
     V s = 0;
-    if (i < n)
-        for (int32_t p = ptr[i] + sub; p < ptr[i + 1]; p += LPR)
-            s = fma(val[p], u[col_at(ci, s_off, i, p)], s);
+    if (i < n) s = A.dot(s_off, i, sub, [&](int32_t j) { return u[j]; });
     s = group_sum<LPR>(s);
     if (i < n && sub == 0) r[i] = (V)f[i] - s;
 }
@@ -1477,10 +1641,7 @@ __global__ void k_copy_cast(int64_t n, const TI *__restrict__ in, TO *__restrict
 // single-block kernel is needed and the sums stay deterministic.
 // 512 threads a block at every size (256 below kCgLargeN measured 1% slower
 // per CG iteration at 64^3: 16 warps per SM hid less latency than 32)
-constexpr int kCgThreads = 512;
-constexpr int kCgMaxBlocks = 152 * 4;  // long vectors: four blocks of 512 per SM
 constexpr int64_t kCgLargeN = (int64_t)152 * 8 * 256 * 4;
-inline int cg_threads(int64_t) { return kCgThreads; }
 
 // deterministic block sum (fixed lane / warp order)
 __device__ double block_sum(double v) {
@@ -1614,24 +1775,19 @@ __global__ void k_cg_set_rz_p(int32_t n, const double *__restrict__ z, double *_
 }
 
 // q = A p; the last block forms p.q and alpha = r.z / p.q (breakdown: p.q <= 0)
-__global__ void k_spmv_dot(int32_t n, const int32_t *__restrict__ ptr, ColIdx ci,
-                           const double *__restrict__ val, const double *__restrict__ p, double *__restrict__ q,
-                           double *__restrict__ partial, CgState *cg) {
+template <class M>
+__global__ void __launch_bounds__(kCgThreads)
+k_spmv_dot(int32_t n, M A, const double *__restrict__ p, double *__restrict__ q, double *__restrict__ partial,
+           CgState *cg) {
     __shared__ int32_t s_off[kMaxColOffsets];
     pdl_wait();
     if (cg->done) return;
-    stage_col_offsets(ci, s_off);
+    A.stage(s_off);
     // r.z of the previous iteration becomes current (read only by the last block)
     if (blockIdx.x == 0 && threadIdx.x == 0) cg->rz = cg->rz_next;
     double d = 0.0;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        if (ci.cidx)
-            for (int32_t e = ptr[i]; e < ptr[i + 1]; ++e) s = fma(val[e], p[i + s_off[ci.cidx[e]]], s);
-        else if (ci.c16)
-            for (int32_t e = ptr[i]; e < ptr[i + 1]; ++e) s = fma(val[e], p[i + (int32_t)ci.c16[e]], s);
-        else
-            for (int32_t e = ptr[i]; e < ptr[i + 1]; ++e) s = fma(val[e], p[ci.col[e]], s);
+        const double s = A.dot(s_off, i, 0, [&](int32_t j) { return p[j]; });
         q[i] = s;
         d = fma(p[i], s, d);
     }
@@ -1691,19 +1847,17 @@ __global__ void k_cg_update_ur(int32_t n, CgState *cg, const double *__restrict_
 // t = f - A u, the true residual, when the recurrence reports convergence; the
 // last block accepts convergence or schedules the replacement of r (twice at
 // most).  With force: unconditionally, the final relative residual.
-__global__ void k_true_residual(int32_t n, const int32_t *__restrict__ ptr, ColIdx ci,
-                                const double *__restrict__ val, const double *__restrict__ f,
-                                const double *__restrict__ u, double *__restrict__ t, double *__restrict__ partial,
-                                CgState *cg, int force) {
+template <class M>
+__global__ void __launch_bounds__(kCgThreads)
+k_true_residual(int32_t n, M A, const double *__restrict__ f, const double *__restrict__ u, double *__restrict__ t,
+                double *__restrict__ partial, CgState *cg, int force) {
     __shared__ int32_t s_off[kMaxColOffsets];
     pdl_wait();
     if (!force && (cg->done || !cg->need_true)) return;
-    stage_col_offsets(ci, s_off);
+    A.stage(s_off);
     double d = 0.0;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int32_t e = ptr[i]; e < ptr[i + 1]; ++e)
-            s = fma(val[e], u[col_at(ci, s_off, i, e)], s);
+        const double s = A.dot(s_off, i, 0, [&](int32_t j) { return u[j]; });
         const double ti = f[i] - s;
         t[i] = ti;
         d = fma(ti, ti, d);
@@ -1783,28 +1937,30 @@ __global__ void k_cg_update_p(int32_t n, CgState *cg, const double *__restrict__
 // device-resident control as CG: every kernel returns at once when the state
 // says done; scalars are formed by the last block of the producing kernel.
 
-// row i of y = A x for the scalar matrix (BS = 1) or the 4 x 4 block matrix
-// seen as 4 n scalar rows (BS = 4: node i / 4, component i % 4; entry order,
-// then component order)
-template <int BS>
-__device__ __forceinline__ double bi_row(int32_t i, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                                         const double *__restrict__ val, const double *__restrict__ x) {
-    double s = 0.0;
-    if (BS == 1) {
-        for (int32_t e = ptr[i]; e < ptr[i + 1]; ++e) s = fma(val[e], x[col[e]], s);
-    } else {
+// row policy of the 4 x 4 block matrix seen as 4 n scalar rows: node i / 4,
+// component i % 4; entry order, then component order
+struct BlockRows {
+    using value = double;
+    static constexpr int lanes = 1;
+    const int32_t *__restrict__ ptr;
+    const int32_t *__restrict__ col;
+    const double *__restrict__ val;
+    __device__ __forceinline__ void stage(int32_t *) const {}
+    template <class X>
+    __device__ __forceinline__ double dot(const int32_t *, int32_t i, int, X x) const {
+        double s = 0.0;
         const int32_t node = i >> 2, r = i & 3;
         for (int32_t e = ptr[node]; e < ptr[node + 1]; ++e) {
             const double *b = val + (int64_t)16 * e + 4 * r;
-            const double *xv = x + (int64_t)4 * col[e];
-            s = fma(b[0], xv[0], s);
-            s = fma(b[1], xv[1], s);
-            s = fma(b[2], xv[2], s);
-            s = fma(b[3], xv[3], s);
+            const int32_t j = 4 * col[e];
+            s = fma(b[0], x(j), s);
+            s = fma(b[1], x(j + 1), s);
+            s = fma(b[2], x(j + 2), s);
+            s = fma(b[3], x(j + 3), s);
         }
+        return s;
     }
-    return s;
-}
+};
 
 // two sums published together; the last block returns both totals
 __device__ bool bi_reduce2(double a, double b, double *pa, double *pb, unsigned *counter, double *ta, double *tb) {
@@ -1885,15 +2041,17 @@ __global__ void k_bi_p(int32_t n, const double *__restrict__ r, const double *__
 }
 
 // v = A p^, (r^, v); alpha = rho / (r^, v)
-template <int BS>
-__global__ void k_bi_spmv_rv(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                             const double *__restrict__ val, const double *__restrict__ ph, double *__restrict__ v,
-                             const double *__restrict__ rh, double *__restrict__ partial, BiState *st) {
+template <class M>
+__global__ void __launch_bounds__(kCgThreads)
+k_bi_spmv_rv(int32_t n, M A, const double *__restrict__ ph, double *__restrict__ v, const double *__restrict__ rh,
+             double *__restrict__ partial, BiState *st) {
+    __shared__ int32_t s_off[kMaxColOffsets];
     pdl_wait();
     if (st->done) return;
+    A.stage(s_off);
     double d = 0.0;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const double s = bi_row<BS>(i, ptr, col, val, ph);
+        const double s = A.dot(s_off, i, 0, [&](int32_t j) { return ph[j]; });
         v[i] = s;
         d = fma(rh[i], s, d);
     }
@@ -1944,16 +2102,17 @@ __global__ void k_bi_half(int32_t n, const double *__restrict__ ph, const double
 }
 
 // t = A s^, (t, s), (t, t); omega = (t, s) / (t, t)
-template <int BS>
-__global__ void k_bi_spmv_t(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                            const double *__restrict__ val, const double *__restrict__ sh,
-                            const double *__restrict__ sv, double *__restrict__ t, double *__restrict__ partial,
-                            BiState *st) {
+template <class M>
+__global__ void __launch_bounds__(kCgThreads)
+k_bi_spmv_t(int32_t n, M A, const double *__restrict__ sh, const double *__restrict__ sv, double *__restrict__ t,
+            double *__restrict__ partial, BiState *st) {
+    __shared__ int32_t s_off[kMaxColOffsets];
     pdl_wait();
     if (st->skip) return;
+    A.stage(s_off);
     double a = 0.0, b = 0.0;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const double s = bi_row<BS>(i, ptr, col, val, sh);
+        const double s = A.dot(s_off, i, 0, [&](int32_t j) { return sh[j]; });
         t[i] = s;
         a = fma(s, sv[i], a);
         b = fma(s, s, b);
@@ -1997,15 +2156,17 @@ __global__ void k_bi_xr(int32_t n, const double *__restrict__ ph, const double *
 // the true residual when the recurrence (or the half step) reports
 // convergence: accept, or replace r by it (twice at most); with force, the
 // final relative residual
-template <int BS>
-__global__ void k_bi_true(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                          const double *__restrict__ val, const double *__restrict__ f, const double *__restrict__ x,
-                          double *__restrict__ t, double *__restrict__ partial, BiState *st, int force) {
+template <class M>
+__global__ void __launch_bounds__(kCgThreads)
+k_bi_true(int32_t n, M A, const double *__restrict__ f, const double *__restrict__ x, double *__restrict__ t,
+          double *__restrict__ partial, BiState *st, int force) {
+    __shared__ int32_t s_off[kMaxColOffsets];
     pdl_wait();
     if (!force && (st->done || !st->need_true)) return;
+    A.stage(s_off);
     double d = 0.0;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const double s = bi_row<BS>(i, ptr, col, val, x);
+        const double s = A.dot(s_off, i, 0, [&](int32_t j) { return x[j]; });
         const double ti = f[i] - s;
         t[i] = ti;
         d = fma(ti, ti, d);
@@ -2108,6 +2269,35 @@ void launch_ingest_fine(int32_t row0, int32_t row1, const int32_t *ptr, const do
     k_ingest_fine<<<nblocks(row1 - row0), kThreads, 0, s>>>(row0, row1, ptr, val_in, dia, type, wj, val_out, valf_out,
                                                             m, mf, st);
 }
+void launch_ingest_stencil(int32_t row0, int32_t row1, const int32_t *ptr, const double *val_in, const Stencil &S,
+                           int type, double wj, double *sval, float *svalf, float *valf_out, double *m, float *mf,
+                           int *st, cudaStream_t s) {
+    if (row1 <= row0) return;
+    count_launch();
+    const int g = nblocks(row1 - row0, kIngestWarps * 32), t = kIngestWarps * 32;
+    if (S.noff == 5)
+        k_ingest_stencil<5><<<g, t, 0, s>>>(row0, row1, ptr, val_in, S, type, wj, sval, svalf, valf_out, m, mf, st);
+    else if (S.noff == 7)
+        k_ingest_stencil<7><<<g, t, 0, s>>>(row0, row1, ptr, val_in, S, type, wj, sval, svalf, valf_out, m, mf, st);
+    else
+        k_ingest_stencil<kMaxStencil>
+            <<<g, t, 0, s>>>(row0, row1, ptr, val_in, S, type, wj, sval, svalf, valf_out, m, mf, st);
+}
+void launch_stencil_mask(int32_t n, const int32_t *ptr, const int32_t *col, const Stencil &S, uint8_t *mask, int *st,
+                         cudaStream_t s) {
+    count_launch();
+    k_stencil_mask<<<nblocks(n), kThreads, 0, s>>>(n, ptr, col, S, mask, st);
+}
+void launch_csr_to_stencil(int32_t n, const int32_t *ptr, const double *val, const Stencil &S, double *sval,
+                           cudaStream_t s) {
+    count_launch();
+    k_csr_to_stencil<<<nblocks(((int64_t)n + 31) / 32 * 32), kThreads, 0, s>>>(n, ptr, val, S, sval);
+}
+void launch_stencil_to_csr(int32_t n, const int32_t *ptr, const double *sval, const Stencil &S, double *val,
+                           cudaStream_t s) {
+    count_launch();
+    k_stencil_to_csr<<<nblocks(n), kThreads, 0, s>>>(n, ptr, sval, S, val);
+}
 void launch_cast_f32(int64_t n, const double *in, float *out, cudaStream_t s) {
     int64_t b = nblocks(n);
     count_launch();
@@ -2191,29 +2381,70 @@ void launch_lu_inverse(int32_t n, const double *lu, const int32_t *piv, double *
         default: { constexpr int P_ = 32; KCALL; } break; \
     }
 
+// calls run(rows) with the row policy of a stencil (ord: the CSR lanes whose
+// order an FP32 sum keeps; FP64 rows are summed in column order)
+template <class V, int NOFF, class Run>
+void with_stencil(const Stencil &S, const V *val, int32_t n, int ord, Run run) {
+    if constexpr (sizeof(V) == 4) {
+        if (ord >= 8) return run(StencilRows<V, NOFF, 8>{S, val, n});
+        if (ord == 4) return run(StencilRows<V, NOFF, 4>{S, val, n});
+        if (ord == 2) return run(StencilRows<V, NOFF, 2>{S, val, n});
+    }
+    run(StencilRows<V, NOFF, 1>{S, val, n});
+}
+template <class V, class Run>
+void with_stencil(const Stencil &S, const V *val, int32_t n, int ord, Run run) {
+    if (S.noff == 5) with_stencil<V, 5>(S, val, n, ord, run);
+    else if (S.noff == 7) with_stencil<V, 7>(S, val, n, ord, run);
+    else with_stencil<V, kMaxStencil>(S, val, n, ord, run);
+}
+template <class V>
+const V *stencil_values(const Level &L) {
+    if constexpr (sizeof(V) == 4) return L.S_valf;
+    else return L.S_val;
+}
+// calls run(rows) with the row policy of a level's matrix
+template <class V, class Run>
+void with_level_rows(const Level &L, const V *val, Run run) {
+    if (L.sten.noff) return with_stencil<V>(L.sten, stencil_values<V>(L), L.n, L.lpr, run);
+    LPR_DISPATCH(L.lpr, (run(CsrRows<V, P_>{L.A_ptr, L.cols(), val})))
+}
+// ... and of the Krylov solver's system matrix (one lane per row)
+template <class Run>
+void with_fine_rows(const FineMat &A, int32_t n, Run run) {
+    if (A.sten.noff) return with_stencil<double>(A.sten, A.sval, n, 1, run);
+    run(CsrRows<double, 1>{A.ptr, A.col, A.val});
+}
+// lanes per row of a policy's launch
+template <class M>
+constexpr int64_t lanes_of(const M &) { return M::lanes; }
+
 template <class V, class TF>
 void launch_smooth0_residual(const Level &L, const V *val, const V *m, const TF *f, V *u, V *r, const int *skip,
                              cudaStream_t s) {
     count_launch();
-    const unsigned g = (unsigned)nblocks((int64_t)L.n * L.lpr);
-    LPR_DISPATCH(L.lpr, (launch_pdl(k_smooth0_residual<V, TF, P_>, g, kThreads, 0, s, L.n, L.A_ptr, L.cols(), val, m, f, u,
-                                                                              r, skip)))
+    with_level_rows<V>(L, val, [&](auto A) {
+        launch_pdl(k_smooth0_residual<decltype(A), TF>, nblocks(L.n * lanes_of(A)), kThreads, 0, s, L.n, A, m, f, u, r,
+                   skip);
+    });
 }
 template <class V, class TF, class TO>
 void launch_smooth_sweep(const Level &L, const V *val, const V *m, const TF *f, const V *u_in, TO *u_out,
                          const int *skip, cudaStream_t s) {
     count_launch();
-    const unsigned g = (unsigned)nblocks((int64_t)L.n * L.lpr);
-    LPR_DISPATCH(L.lpr, (launch_pdl(k_smooth_sweep<V, TF, TO, P_>, g, kThreads, 0, s, L.n, L.A_ptr, L.cols(), val, m, f,
-                                                                              u_in, u_out, skip)))
+    with_level_rows<V>(L, val, [&](auto A) {
+        launch_pdl(k_smooth_sweep<decltype(A), TF, TO>, nblocks(L.n * lanes_of(A)), kThreads, 0, s, L.n, A, m, f, u_in,
+                   u_out, skip);
+    });
 }
 template <class V>
 void launch_smooth_sweep_dot(const Level &L, const V *val, const V *m, const double *f, const V *u_in, double *z,
                              double *partial, CgState *cg, const int *skip, cudaStream_t s) {
     count_launch();
-    const unsigned g = (unsigned)cg_blocks(L.n);
-    LPR_DISPATCH(L.lpr, (launch_pdl(k_smooth_sweep_dot<V, P_>, g, cg_threads(L.n), 0, s, L.n, L.A_ptr, L.cols(), val, m, f, u_in,
-                                                                             z, partial, cg, skip)))
+    with_level_rows<V>(L, val, [&](auto A) {
+        launch_pdl(k_smooth_sweep_dot<decltype(A)>, cg_blocks(L.n * lanes_of(A)), kCgThreads, 0, s, L.n, A, m, f, u_in,
+                   z, partial, cg, skip);
+    });
 }
 template void launch_smooth_sweep_dot<double>(const Level &, const double *, const double *, const double *,
                                               const double *, double *, double *, CgState *, const int *,
@@ -2223,8 +2454,9 @@ template void launch_smooth_sweep_dot<float>(const Level &, const float *, const
 template <class V, class TF>
 void launch_residual(const Level &L, const V *val, const TF *f, const V *u, V *r, const int *skip, cudaStream_t s) {
     count_launch();
-    const unsigned g = (unsigned)nblocks((int64_t)L.n * L.lpr);
-    LPR_DISPATCH(L.lpr, (launch_pdl(k_residual<V, TF, P_>, g, kThreads, 0, s, L.n, L.A_ptr, L.cols(), val, f, u, r, skip)))
+    with_level_rows<V>(L, val, [&](auto A) {
+        launch_pdl(k_residual<decltype(A), TF>, nblocks(L.n * lanes_of(A)), kThreads, 0, s, L.n, A, f, u, r, skip);
+    });
 }
 template <class V>
 void launch_restrict(const Level &L, const V *Rval, const V *r, V *fc, const V *mc, V *uc, const int *skip,
@@ -2299,8 +2531,7 @@ template void launch_copy_cast<float, double>(int64_t, const float *, double *, 
 // blocks of 512 per SM (half the partials of eight blocks of 256, measured
 // faster at 128^3 and 192^3).
 int cg_blocks(int64_t n) {
-    const int t = cg_threads(n);
-    int64_t b = (n + t - 1) / t;
+    int64_t b = (n + kCgThreads - 1) / kCgThreads;
     const int64_t cap = n >= kCgLargeN ? kCgMaxBlocks : 152 * 2;
     if (b > cap) b = cap;
     return (int)(b < 1 ? 1 : b);
@@ -2308,27 +2539,29 @@ int cg_blocks(int64_t n) {
 void launch_cg_init(int32_t n, const double *f, double *u, double *r, double *partial, CgState *cg, double tol,
                     int maxiter, const Smooth0Out &z0, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_cg_init, cg_blocks(n), cg_threads(n), 0, s, n, f, u, r, partial, cg, tol, maxiter, z0);
+    launch_pdl(k_cg_init, cg_blocks(n), kCgThreads, 0, s, n, f, u, r, partial, cg, tol, maxiter, z0);
 }
 void launch_dot(int32_t n, const double *x, const double *y, double *partial, const int *skip, CgState *cg, int target,
                 cudaStream_t s) {
     count_launch();
-    launch_pdl(k_dot, cg_blocks(n), cg_threads(n), 0, s, n, x, y, partial, skip, cg, target);
+    launch_pdl(k_dot, cg_blocks(n), kCgThreads, 0, s, n, x, y, partial, skip, cg, target);
 }
 void launch_cg_set_rz_p(int32_t n, const double *z, double *p, CgState *cg, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_cg_set_rz_p, cg_blocks(n), cg_threads(n), 0, s, n, z, p, cg);
+    launch_pdl(k_cg_set_rz_p, cg_blocks(n), kCgThreads, 0, s, n, z, p, cg);
 }
-void launch_spmv_dot(int32_t n, const int32_t *ptr, const ColIdx &col, const double *val, const double *p,
-                     double *q, double *partial, CgState *cg, cudaStream_t s) {
+void launch_spmv_dot(int32_t n, const FineMat &A, const double *p, double *q, double *partial, CgState *cg,
+                     cudaStream_t s) {
     count_launch();
-    launch_pdl(k_spmv_dot, cg_blocks(n), cg_threads(n), 0, s, n, ptr, col, val, p, q, partial, cg);
+    with_fine_rows(A, n, [&](auto M) {
+        launch_pdl(k_spmv_dot<decltype(M)>, cg_blocks(n), kCgThreads, 0, s, n, M, p, q, partial, cg);
+    });
 }
 void launch_cg_update_ur(int32_t n, CgState *cg, const double *p, const double *q, double *u, double *r,
                          double *partial, const double *zo, double *part_zo, int use_h, cudaGraphConditionalHandle hb,
                          const Smooth0Out &z0, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_cg_update_ur, cg_blocks(n), cg_threads(n), 0, s, n, cg, p, q, u, r, partial, zo, part_zo, use_h, hb,
+    launch_pdl(k_cg_update_ur, cg_blocks(n), kCgThreads, 0, s, n, cg, p, q, u, r, partial, zo, part_zo, use_h, hb,
                z0);
 }
 void launch_col_delta16(int32_t n, const int32_t *ptr, const int32_t *col, float ratio, int16_t *c16, int *flag,
@@ -2346,71 +2579,82 @@ void launch_col_offsets_encode(int32_t n, const int32_t *ptr, const int32_t *col
     count_launch();
     k_col_offsets_encode<<<nblocks(n), kThreads, 0, s>>>(n, ptr, col, off, noff, cidx, st);
 }
-void launch_true_residual(int32_t n, const int32_t *ptr, const ColIdx &col, const double *val, const double *f,
-                          const double *u, double *t, double *partial, CgState *cg, int force, cudaStream_t s) {
+void launch_true_residual(int32_t n, const FineMat &A, const double *f, const double *u, double *t, double *partial,
+                          CgState *cg, int force, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_true_residual, cg_blocks(n), cg_threads(n), 0, s, n, ptr, col, val, f, u, t, partial, cg, force);
+    with_fine_rows(A, n, [&](auto M) {
+        launch_pdl(k_true_residual<decltype(M)>, cg_blocks(n), kCgThreads, 0, s, n, M, f, u, t, partial, cg, force);
+    });
 }
 void launch_replace_r(int32_t n, CgState *cg, const double *t, double *r, const double *zo, double *part_zo,
                       const Smooth0Out &z0, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_replace_r, cg_blocks(n), cg_threads(n), 0, s, n, cg, t, r, zo, part_zo, z0);
+    launch_pdl(k_replace_r, cg_blocks(n), kCgThreads, 0, s, n, cg, t, r, zo, part_zo, z0);
 }
 void launch_cg_update_p(int32_t n, CgState *cg, const double *z, double *p, int use_h, cudaGraphConditionalHandle h,
                         cudaStream_t s) {
     count_launch();
-    launch_pdl(k_cg_update_p, cg_blocks(n), cg_threads(n), 0, s, n, cg, z, p, use_h, h);
+    launch_pdl(k_cg_update_p, cg_blocks(n), kCgThreads, 0, s, n, cg, z, p, use_h, h);
 }
 
 
 void launch_bi_init(int32_t n, const double *f, double *x, double *r, double *rh, double *p, double *v,
                     double *partial, BiState *st, double tol, int maxiter, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_bi_init, cg_blocks(n), cg_threads(n), 0, s, n, f, x, r, rh, p, v, partial, st, tol, maxiter);
+    launch_pdl(k_bi_init, cg_blocks(n), kCgThreads, 0, s, n, f, x, r, rh, p, v, partial, st, tol, maxiter);
 }
 void launch_bi_rho(int32_t n, const double *rh, const double *r, double *partial, BiState *st, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_bi_rho, cg_blocks(n), cg_threads(n), 0, s, n, rh, r, partial, st);
+    launch_pdl(k_bi_rho, cg_blocks(n), kCgThreads, 0, s, n, rh, r, partial, st);
 }
 void launch_bi_p(int32_t n, const double *r, const double *v, double *p, BiState *st, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_bi_p, cg_blocks(n), cg_threads(n), 0, s, n, r, v, p, st);
+    launch_pdl(k_bi_p, cg_blocks(n), kCgThreads, 0, s, n, r, v, p, st);
 }
-void launch_bi_spmv_rv(int32_t n, int bs, const int32_t *ptr, const int32_t *col, const double *val,
-                       const double *ph, double *v, const double *rh, double *partial, BiState *st, cudaStream_t s) {
+void launch_bi_spmv_rv(int32_t n, int bs, const FineMat &A, const double *ph, double *v, const double *rh,
+                       double *partial, BiState *st, cudaStream_t s) {
     count_launch();
-    if (bs == 4) launch_pdl(k_bi_spmv_rv<4>, cg_blocks(n), cg_threads(n), 0, s, n, ptr, col, val, ph, v, rh, partial, st);
-    else launch_pdl(k_bi_spmv_rv<1>, cg_blocks(n), cg_threads(n), 0, s, n, ptr, col, val, ph, v, rh, partial, st);
+    const auto run = [&](auto M) {
+        launch_pdl(k_bi_spmv_rv<decltype(M)>, cg_blocks(n), kCgThreads, 0, s, n, M, ph, v, rh, partial, st);
+    };
+    if (bs == 4) run(BlockRows{A.ptr, A.col.col, A.val});
+    else with_fine_rows(A, n, run);
 }
 void launch_bi_s(int32_t n, const double *r, const double *v, double *sv, double *partial, BiState *st,
                  cudaStream_t s) {
     count_launch();
-    launch_pdl(k_bi_s, cg_blocks(n), cg_threads(n), 0, s, n, r, v, sv, partial, st);
+    launch_pdl(k_bi_s, cg_blocks(n), kCgThreads, 0, s, n, r, v, sv, partial, st);
 }
 void launch_bi_half(int32_t n, const double *ph, const double *sv, double *x, double *r, BiState *st, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_bi_half, cg_blocks(n), cg_threads(n), 0, s, n, ph, sv, x, r, st);
+    launch_pdl(k_bi_half, cg_blocks(n), kCgThreads, 0, s, n, ph, sv, x, r, st);
 }
-void launch_bi_spmv_t(int32_t n, int bs, const int32_t *ptr, const int32_t *col, const double *val,
-                      const double *sh, const double *sv, double *t, double *partial, BiState *st, cudaStream_t s) {
+void launch_bi_spmv_t(int32_t n, int bs, const FineMat &A, const double *sh, const double *sv, double *t,
+                      double *partial, BiState *st, cudaStream_t s) {
     count_launch();
-    if (bs == 4) launch_pdl(k_bi_spmv_t<4>, cg_blocks(n), cg_threads(n), 0, s, n, ptr, col, val, sh, sv, t, partial, st);
-    else launch_pdl(k_bi_spmv_t<1>, cg_blocks(n), cg_threads(n), 0, s, n, ptr, col, val, sh, sv, t, partial, st);
+    const auto run = [&](auto M) {
+        launch_pdl(k_bi_spmv_t<decltype(M)>, cg_blocks(n), kCgThreads, 0, s, n, M, sh, sv, t, partial, st);
+    };
+    if (bs == 4) run(BlockRows{A.ptr, A.col.col, A.val});
+    else with_fine_rows(A, n, run);
 }
 void launch_bi_xr(int32_t n, const double *ph, const double *sh, const double *sv, const double *t, double *x,
                   double *r, double *partial, BiState *st, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_bi_xr, cg_blocks(n), cg_threads(n), 0, s, n, ph, sh, sv, t, x, r, partial, st);
+    launch_pdl(k_bi_xr, cg_blocks(n), kCgThreads, 0, s, n, ph, sh, sv, t, x, r, partial, st);
 }
-void launch_bi_true(int32_t n, int bs, const int32_t *ptr, const int32_t *col, const double *val, const double *f,
-                    const double *x, double *t, double *partial, BiState *st, int force, cudaStream_t s) {
+void launch_bi_true(int32_t n, int bs, const FineMat &A, const double *f, const double *x, double *t, double *partial,
+                    BiState *st, int force, cudaStream_t s) {
     count_launch();
-    if (bs == 4) launch_pdl(k_bi_true<4>, cg_blocks(n), cg_threads(n), 0, s, n, ptr, col, val, f, x, t, partial, st, force);
-    else launch_pdl(k_bi_true<1>, cg_blocks(n), cg_threads(n), 0, s, n, ptr, col, val, f, x, t, partial, st, force);
+    const auto run = [&](auto M) {
+        launch_pdl(k_bi_true<decltype(M)>, cg_blocks(n), kCgThreads, 0, s, n, M, f, x, t, partial, st, force);
+    };
+    if (bs == 4) run(BlockRows{A.ptr, A.col.col, A.val});
+    else with_fine_rows(A, n, run);
 }
 void launch_bi_replace(int32_t n, const double *t, double *r, BiState *st, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_bi_replace, cg_blocks(n), cg_threads(n), 0, s, n, t, r, st);
+    launch_pdl(k_bi_replace, cg_blocks(n), kCgThreads, 0, s, n, t, r, st);
 }
 void launch_bi_end(BiState *st, int use_h, cudaGraphConditionalHandle h, cudaStream_t s) {
     count_launch();
