@@ -937,8 +937,8 @@ V *down_level(amg_ctx *ctx, int l, const TF *f, const int *skip, bool u0_ready) 
 
 // post-smoothing on the finest level; the last sweep writes z and, when
 // rz_partial is given, the per-block partials of r.z (r = f here)
-template <class V>
-void up_finest(amg_ctx *ctx, const double *f, V *u, double *out, double *rz_partial, const int *skip) {
+template <class V, class TZ>
+void up_finest(amg_ctx *ctx, const double *f, V *u, TZ *out, double *rz_partial, const int *skip) {
     Level &L = ctx->lev[0];
     VecSet<V> &v = Vops<V>::vec(L);
     const V *A = Vops<V>::A(L), *m = Vops<V>::m(L);
@@ -946,20 +946,23 @@ void up_finest(amg_ctx *ctx, const double *f, V *u, double *out, double *rz_part
     const int npost = ctx->prm.npost;
     for (int k = 0; k < npost; ++k) {
         if (k == npost - 1) {
-            if (rz_partial) {
-                ProfScope ps_(ctx, AMG_PROF_SWEEP_L0);
-                launch_smooth_sweep_dot<V>(L, A, m, f, u, out, rz_partial, ctx->cg, skip, ctx->s);
-            } else {
-                ProfScope ps_(ctx, AMG_PROF_SWEEP_L0);
+            ProfScope ps_(ctx, AMG_PROF_SWEEP_L0);
+            if constexpr (sizeof(TZ) == sizeof(V))
+                if (rz_partial) {
+                    launch_smooth_sweep_dot<V, TZ>(L, A, m, f, u, out, rz_partial, ctx->cg, skip, ctx->s);
+                    return;
+                }
+            if constexpr (sizeof(TZ) == sizeof(double))
                 launch_smooth_sweep<V, double, double>(L, A, m, f, u, out, skip, ctx->s);
-            }
             return;
         }
         launch_smooth_sweep<V, double, V>(L, A, m, f, u, t, skip, ctx->s);
         std::swap(u, t);
     }
-    launch_copy_cast<V, double>(L.n, u, out, skip, ctx->s);
-    if (rz_partial) launch_dot(ctx->n, f, out, rz_partial, skip, ctx->cg, 1, ctx->s);
+    if constexpr (sizeof(TZ) == sizeof(double)) {
+        launch_copy_cast<V, double>(L.n, u, out, skip, ctx->s);
+        if (rz_partial) launch_dot(ctx->n, f, out, rz_partial, skip, ctx->cg, 1, ctx->s);
+    }
 }
 
 // post-smoothing on level l; the last sweep writes `out` (type TO) when given
@@ -981,12 +984,14 @@ void up_level(amg_ctx *ctx, int l, const TF *f, V *u, TO *out, const int *skip) 
     if (out) launch_copy_cast<V, TO>(L.n, u, out, skip, ctx->s);
 }
 
-template <class V>
-void enqueue_vcycle(amg_ctx *ctx, const double *r, double *z, const int *skip, double *rz_partial, bool u0_ready) {
+template <class V, class TZ>
+void enqueue_vcycle(amg_ctx *ctx, const double *r, TZ *z, const int *skip, double *rz_partial, bool u0_ready) {
     const int nl = ctx->nlev;
     if (nl == 1) {
-        launch_coarse_solve<V, double, double>(ctx->lev[0].n, ctx->inv, r, z, skip, ctx->s);
-        if (rz_partial) launch_dot(ctx->n, r, z, rz_partial, skip, ctx->cg, 1, ctx->s);
+        if constexpr (sizeof(TZ) == sizeof(double)) {
+            launch_coarse_solve<V, double, double>(ctx->lev[0].n, ctx->inv, r, z, skip, ctx->s);
+            if (rz_partial) launch_dot(ctx->n, r, z, rz_partial, skip, ctx->cg, 1, ctx->s);
+        }
         return;
     }
     // the restriction into a smoothed level also writes that level's u0 = m o f
@@ -1024,7 +1029,7 @@ void enqueue_vcycle(amg_ctx *ctx, const double *r, double *z, const int *skip, d
     }
     Level &F = ctx->lev[0];
     { ProfScope ps_(ctx, AMG_PROF_PROLONG_L0, true); launch_prolong<V>(F, Vops<V>::P(F), cur[1], cur[0], skip, ctx->s); }
-    up_finest<V>(ctx, r, cur[0], z, rz_partial, skip);
+    up_finest<V, TZ>(ctx, r, cur[0], z, rz_partial, skip);
 }
 
 // Alg. 2 on the 4 x 4 block hierarchy (damped block Jacobi, zero initial
@@ -1080,8 +1085,8 @@ void enqueue_block_vcycle(amg_ctx *ctx, const double *r, double *z, const int *s
 void vcycle(amg_ctx *ctx, const double *r, double *z, const int *skip, double *rz_partial = nullptr,
             bool u0_ready = false) {
     if (blockmode(ctx)) enqueue_block_vcycle(ctx, r, z, skip);
-    else if (mixed(ctx)) enqueue_vcycle<float>(ctx, r, z, skip, rz_partial, u0_ready);
-    else enqueue_vcycle<double>(ctx, r, z, skip, rz_partial, u0_ready);
+    else if (mixed(ctx)) enqueue_vcycle<float, double>(ctx, r, z, skip, rz_partial, u0_ready);
+    else enqueue_vcycle<double, double>(ctx, r, z, skip, rz_partial, u0_ready);
 }
 
 // ---------------------------------------------------------------- CG
@@ -1098,17 +1103,29 @@ Smooth0Out cg_smooth0(amg_ctx *ctx) {
 }
 bool cg_u0(amg_ctx *ctx) { return ctx->nlev >= 2 && ctx->prm.npre >= 1 && !blockmode(ctx); }
 
+// CG holds z as the cycle makes it: in FP32 when the last sweep of a
+// mixed-precision cycle writes it (then in cg_z's memory as floats)
+bool cg_z32(const amg_ctx *ctx) { return mixed(ctx) && ctx->nlev >= 2 && ctx->prm.npost >= 1; }
+float *cg_zf(const amg_ctx *ctx) { return reinterpret_cast<float *>(ctx->cg_z); }
+void cg_vcycle(amg_ctx *ctx) {
+    if (cg_z32(ctx))
+        enqueue_vcycle<float, float>(ctx, ctx->cg_r, cg_zf(ctx), &ctx->cg->done, ctx->part_rz, cg_u0(ctx));
+    else
+        vcycle(ctx, ctx->cg_r, ctx->cg_z, &ctx->cg->done, ctx->part_rz, cg_u0(ctx));
+}
+
 void enqueue_cg_prologue(amg_ctx *ctx, const double *f, double *u, double tol) {
     const int32_t n = ctx->n;
     CgState *cg = ctx->cg;
     launch_cg_init(n, f, u, ctx->cg_r, ctx->part_rr, cg, tol, ctx->prm.maxiter, cg_smooth0(ctx), ctx->s);
-    vcycle(ctx, ctx->cg_r, ctx->cg_z, &cg->done, ctx->part_rz, cg_u0(ctx));
-    launch_cg_set_rz_p(n, ctx->cg_z, ctx->cg_p, cg, ctx->s);
+    cg_vcycle(ctx);
+    if (cg_z32(ctx)) launch_cg_set_rz_p<float>(n, cg_zf(ctx), ctx->cg_p, cg, ctx->s);
+    else launch_cg_set_rz_p<double>(n, ctx->cg_z, ctx->cg_p, cg, ctx->s);
 }
 
 // One CG iteration in three parts; every kernel returns at once when the
 // state says done.  A: q = A p, alpha, u and r, the recurrence residual check.
-void enqueue_cg_iter_a(amg_ctx *ctx, double *u, int use_h, cudaGraphConditionalHandle hb) {
+void enqueue_cg_iter_a(amg_ctx *ctx, int use_h, cudaGraphConditionalHandle hb) {
     const int32_t n = ctx->n;
     CgState *cg = ctx->cg;
     {
@@ -1118,31 +1135,39 @@ void enqueue_cg_iter_a(amg_ctx *ctx, double *u, int use_h, cudaGraphConditionalH
     {
         ProfScope ps_(ctx, AMG_PROF_CG_UPDATE, true);
         // flexible variant: r_new.z_old in the same pass (z still holds the last z)
-        const bool flex = mixed(ctx);
-        launch_cg_update_ur(n, cg, ctx->cg_p, ctx->cg_q, u, ctx->cg_r, ctx->part_rr, flex ? ctx->cg_z : nullptr,
-                            ctx->part_rzo, use_h, hb, cg_smooth0(ctx), ctx->s);
+        if (cg_z32(ctx))
+            launch_cg_update_r<float>(n, cg, ctx->cg_q, ctx->cg_r, ctx->part_rr, cg_zf(ctx), ctx->part_rzo, use_h, hb,
+                                      cg_smooth0(ctx), ctx->s);
+        else
+            launch_cg_update_r<double>(n, cg, ctx->cg_q, ctx->cg_r, ctx->part_rr, mixed(ctx) ? ctx->cg_z : nullptr,
+                                       ctx->part_rzo, use_h, hb, cg_smooth0(ctx), ctx->s);
     }
 }
 
-// B: only when the recurrence met the tolerance: the true residual, and r
-// replaced by it if it misses
+// B: only when the recurrence met the tolerance (or maxiter ended it): u, the
+// true residual, and r replaced by it if it misses
 void enqueue_cg_iter_b(amg_ctx *ctx, const double *f, double *u) {
     const int32_t n = ctx->n;
     CgState *cg = ctx->cg;
+    launch_cg_update_u(n, cg, ctx->cg_p, u, ctx->s);
     launch_true_residual(n, fine_mat(ctx), f, u, ctx->cg_t, ctx->part_tt, cg, 0, ctx->s);
-    launch_replace_r(n, cg, ctx->cg_t, ctx->cg_r, mixed(ctx) ? ctx->cg_z : nullptr, ctx->part_rzo, cg_smooth0(ctx),
-                     ctx->s);
+    if (cg_z32(ctx))
+        launch_replace_r<float>(n, cg, ctx->cg_t, ctx->cg_r, cg_zf(ctx), ctx->part_rzo, cg_smooth0(ctx), ctx->s);
+    else
+        launch_replace_r<double>(n, cg, ctx->cg_t, ctx->cg_r, mixed(ctx) ? ctx->cg_z : nullptr, ctx->part_rzo,
+                                 cg_smooth0(ctx), ctx->s);
 }
 
 // C: z = B r with the partials of r.z, beta and p (and the loop condition)
-void enqueue_cg_iter_c(amg_ctx *ctx, int use_h, cudaGraphConditionalHandle h) {
+void enqueue_cg_iter_c(amg_ctx *ctx, double *u, int use_h, cudaGraphConditionalHandle h) {
     const int32_t n = ctx->n;
     CgState *cg = ctx->cg;
     // (the flexible variant's r_new.z_old was formed by the u / r update)
-    vcycle(ctx, ctx->cg_r, ctx->cg_z, &cg->done, ctx->part_rz, cg_u0(ctx));
+    cg_vcycle(ctx);
     {
         ProfScope ps_(ctx, AMG_PROF_CG_P, true);
-        launch_cg_update_p(n, cg, ctx->cg_z, ctx->cg_p, use_h, h, ctx->s);
+        if (cg_z32(ctx)) launch_cg_update_p<float>(n, cg, cg_zf(ctx), ctx->cg_p, u, use_h, h, ctx->s);
+        else launch_cg_update_p<double>(n, cg, ctx->cg_z, ctx->cg_p, u, use_h, h, ctx->s);
     }
 }
 
@@ -1214,7 +1239,7 @@ amg_status build_solve_graph(amg_ctx *ctx, double tol) {
         // the IF handle belongs to the body graph; the check kernel sets it
         cudaError_t eh = cudaGraphConditionalHandleCreate(&h_true, body, 0, cudaGraphCondAssignDefault);
         if (eh == cudaSuccess) {
-            enqueue_cg_iter_a(ctx, u, 1, h_true);
+            enqueue_cg_iter_a(ctx, 1, h_true);
             cudaStreamCaptureStatus cs;
             cudaGraph_t g = nullptr;
             const cudaGraphNode_t *deps = nullptr;
@@ -1246,7 +1271,7 @@ amg_status build_solve_graph(amg_ctx *ctx, double tol) {
             if (eh == cudaSuccess)
                 eh = cudaStreamUpdateCaptureDependencies(ctx->s_cap, &if_node, nullptr, 1,
                                                          cudaStreamSetCaptureDependencies);
-            if (eh == cudaSuccess) enqueue_cg_iter_c(ctx, 1, h_loop);
+            if (eh == cudaSuccess) enqueue_cg_iter_c(ctx, u, 1, h_loop);
         }
         c2 = launch_total() - ctx->graph_branch;
         (void)ca;
@@ -1464,9 +1489,9 @@ amg_status solve_cg_profiled(amg_ctx *ctx, const double *f, double *u, double to
     for (int it = 1; it <= K; ++it) {
         if (it == K) ctx->prof.on = false;
         { ProfScope cal_(ctx, AMG_PROF_EMPTY, true); }  // two adjacent event nodes: the timing overhead
-        enqueue_cg_iter_a(ctx, u, 0, 0);
+        enqueue_cg_iter_a(ctx, 0, 0);
         enqueue_cg_iter_b(ctx, f, u);
-        enqueue_cg_iter_c(ctx, 0, 0);
+        enqueue_cg_iter_c(ctx, u, 0, 0);
     }
     ctx->prof.on = true;
     enqueue_cg_epilogue(ctx, f, u);
@@ -1498,16 +1523,17 @@ amg_status solve_impl(amg_ctx *ctx, const double *f, double *u, double tol, amg_
         // the true-residual branch ran in 1 + replacements bodies when it converged
         const CgState &hc = *ctx->h_cg;
         const int64_t bodies = (int64_t)hc.pad + 1;
-        const int64_t branches = (hc.status == AMG_OK && hc.iter > 0) ? 1 + hc.replacements : hc.replacements;
+        const int64_t branches =
+            (hc.status != AMG_ERR_BREAKDOWN && hc.iter > 0) ? 1 + hc.replacements : hc.replacements;
         add_launches(ctx->graph_pro + ctx->graph_epi + ctx->graph_body * bodies + ctx->graph_branch * branches);
         return st;
     }
     // eager path: the host checks the device state after every iteration
     enqueue_cg_prologue(ctx, f, u, tol);
     for (int it = 1; it <= ctx->prm.maxiter; ++it) {
-        enqueue_cg_iter_a(ctx, u, 0, 0);
+        enqueue_cg_iter_a(ctx, 0, 0);
         enqueue_cg_iter_b(ctx, f, u);
-        enqueue_cg_iter_c(ctx, 0, 0);
+        enqueue_cg_iter_c(ctx, u, 0, 0);
         CK(cudaMemcpyAsync(ctx->h_cg, ctx->cg, sizeof(CgState), cudaMemcpyDeviceToHost, ctx->s));
         CK(cudaStreamSynchronize(ctx->s));
         if (ctx->h_cg->done) break;

@@ -37,6 +37,7 @@ struct CgState {
     double rz, rz_next, rzo, pq, alpha, beta, rr, nf, res, tres, tol;
     unsigned ctr[CG_NCTR];  // arrival counters of the last-block reductions (zero between kernels)
     int iter, maxiter, done, status, replacements, need_true, copy_r;
+    int u_done;  // u += alpha p is left to k_cg_update_u in this iteration
     int pad;  // loop bodies executed (graph path)
 };
 
@@ -296,8 +297,8 @@ void launch_smooth_sweep(const Level &L, const V *val, const V *m, const TF *f, 
 template <class V, class TF>
 void launch_residual(const Level &L, const V *val, const TF *f, const V *u, V *r, const int *skip, cudaStream_t s);
 // last finest-level post-smoothing sweep fused with the CG product r.z (cg_blocks(n) partials)
-template <class V>
-void launch_smooth_sweep_dot(const Level &L, const V *val, const V *m, const double *f, const V *u_in, double *z,
+template <class V, class TZ>
+void launch_smooth_sweep_dot(const Level &L, const V *val, const V *m, const double *f, const V *u_in, TZ *z,
                              double *partial, CgState *cg, const int *skip, cudaStream_t s);
 template <class V>
 void launch_restrict(const Level &L, const V *Rval, const V *r, V *fc, const V *mc, V *uc, const int *skip,
@@ -336,7 +337,9 @@ void launch_cg_init(int32_t n, const double *f, double *u, double *r, double *pa
 // (target 1: the new r.z, target 2: r_new.z_old)
 void launch_dot(int32_t n, const double *x, const double *y, double *partial, const int *skip, CgState *cg, int target,
                 cudaStream_t s);
-void launch_cg_set_rz_p(int32_t n, const double *z, double *p, CgState *cg, cudaStream_t s);
+// (TZ: the type that z is kept in, FP32 for a mixed-precision cycle)
+template <class TZ>
+void launch_cg_set_rz_p(int32_t n, const TZ *z, double *p, CgState *cg, cudaStream_t s);
 void launch_spmv_dot(int32_t n, const FineMat &A, const double *p, double *q, double *partial, CgState *cg,
                      cudaStream_t s);
 // the compressed form of a pattern: collect the distinct offsets column - row
@@ -356,15 +359,19 @@ void launch_col_offsets_encode(int32_t n, const int32_t *ptr, const int32_t *col
                                uint8_t *cidx, int *st, cudaStream_t s);
 // zo (flexible variant, else null): the previous z; r_new.z_old goes to cg->rzo
 // through the partials part_zo
-void launch_cg_update_ur(int32_t n, CgState *cg, const double *p, const double *q, double *u, double *r,
-                         double *partial, const double *zo, double *part_zo, int use_h, cudaGraphConditionalHandle hb,
-                         const Smooth0Out &z0, cudaStream_t s);
+template <class TZ>
+void launch_cg_update_r(int32_t n, CgState *cg, const double *q, double *r, double *partial, const TZ *zo,
+                        double *part_zo, int use_h, cudaGraphConditionalHandle hb, const Smooth0Out &z0,
+                        cudaStream_t s);
+void launch_cg_update_u(int32_t n, const CgState *cg, const double *p, double *u, cudaStream_t s);
 void launch_true_residual(int32_t n, const FineMat &A, const double *f, const double *u, double *t, double *partial,
                           CgState *cg, int force, cudaStream_t s);
-void launch_replace_r(int32_t n, CgState *cg, const double *t, double *r, const double *zo, double *part_zo,
+template <class TZ>
+void launch_replace_r(int32_t n, CgState *cg, const double *t, double *r, const TZ *zo, double *part_zo,
                       const Smooth0Out &z0, cudaStream_t s);
-void launch_cg_update_p(int32_t n, CgState *cg, const double *z, double *p, int use_h, cudaGraphConditionalHandle h,
-                        cudaStream_t s);
+template <class TZ>
+void launch_cg_update_p(int32_t n, CgState *cg, const TZ *z, double *p, double *u, int use_h,
+                        cudaGraphConditionalHandle h, cudaStream_t s);
 
 // BiCGStab (FP64), right-preconditioned; partial: 3 * cg_blocks(n) doubles
 void launch_bi_init(int32_t n, const double *f, double *x, double *r, double *rh, double *p, double *v,

@@ -175,40 +175,33 @@ __device__ __forceinline__ bool finite_bits(double x) {
     return ((unsigned long long)__double_as_longlong(x) & 0x7ff0000000000000ull) != 0x7ff0000000000000ull;
 }
 
-// (float)x rounded to nearest, ties to even, from the IEEE 754 formats: on
-// this part the conversion instruction runs on the FP64 pipe (about as slow
-// as an FP64 add), these integer steps do not.  Worth it where the FP64 pipe
-// bounds a kernel (the finest level's copy-and-cast), not elsewhere (measured
-// slower in the V-cycle kernels).  The 52-bit significand drops
-// 29 bits (normal results) or more (subnormal results, shift 52 - (e + 149)
-// for an unbiased exponent e), rounded from the dropped bits; a carry out of
-// the significand moves to the next exponent (up to infinity).  Infinities
-// and NaNs use the conversion instruction.
+// Casts between FP64 and FP32 by integer steps on the IEEE 754 formats (the
+// bits of the conversion instructions), for normal results; zeros, subnormals,
+// infinities and NaNs use the instruction.  On this part it runs on the FP64
+// pipe at the rate of an FP64 add, and a predicated-off one still takes its
+// slot there, so the rare path is a function of its own (a real branch): with
+// the instruction inlined behind the test the r update at 192^3 took 85 us,
+// with the call 56.  Worth it where FP64 work bounds a kernel (the finest
+// level's copy-and-cast, the r and p updates); in kernels that hold many
+// loads in registers the call costs more than it saves (last sweep with r.z at
+// 192^3: 80 us against 61).
+static __device__ __noinline__ float f64_to_f32_instr(double x) { return (float)x; }
+static __device__ __noinline__ double f32_to_f64_instr(float x) { return (double)x; }
+
+// (float)x rounded to nearest, ties to even: the top 24 significand bits,
+// rounded by the other 29 (a carry moves on into the exponent)
 __device__ __forceinline__ float f64_to_f32_rn(double x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const unsigned sgn = (unsigned)(b >> 32) & 0x80000000u;
-    const int eb = (int)((b >> 52) & 0x7ff);
-    if (eb == 0x7ff) return (float)x;
-    const int e = eb - 1023;
-    if (e > 127) return __uint_as_float(sgn | 0x7f800000u);
-    const unsigned long long full = (b & 0x000fffffffffffffull) | (eb ? 0x0010000000000000ull : 0ull);
-    // result = round(full * 2^(e - 52)) in units of the float's last place:
-    // 2^(e - 23) for normal results, 2^-149 for subnormal ones
-    const int sh = e >= -126 ? 29 : 52 - (e + 149);
-    if (eb == 0 || sh > 63) return __uint_as_float(sgn);
-    unsigned long long q = full >> sh;
-    const unsigned long long rem = full & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
-    if (rem > half || (rem == half && (q & 1ull))) q += 1ull;
-    unsigned bits;
-    if (e >= -126) {
-        // q in [2^23, 2^24]: the hidden bit and 23 fraction bits (2^24: a carry)
-        bits = (unsigned)((unsigned long long)(e + 127) << 23) + (unsigned)(q - (1ull << 23));
-        if (bits >= 0x7f800000u) bits = 0x7f800000u;
-    } else {
-        bits = (unsigned)q;  // subnormal (2^23: the smallest normal)
-    }
-    return __uint_as_float(sgn | bits);
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), a = hi & 0x7fffffffu;
+    // exponents from -126 up to the last below FP32's largest value
+    if (a - 0x38100000u >= 0x0fdfffffu) return f64_to_f32_instr(x);
+    const unsigned t = __funnelshift_l(lo, a - 0x38000000u, 3), rest = lo & 0x1fffffffu;
+    return __uint_as_float((t + (rest + (t & 1u) > 0x10000000u ? 1u : 0u)) | (hi & 0x80000000u));
 }
 
+__device__ __forceinline__ double f32_to_f64(float x) {
+    const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+    if (e - 1u >= 254u) return f32_to_f64_instr(x);
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
 
 }  // namespace amgpr

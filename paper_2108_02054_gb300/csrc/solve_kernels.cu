@@ -1394,6 +1394,17 @@ __global__ void k_col_offsets_encode(int32_t n, const int32_t *__restrict__ ptr,
     }
 }
 
+// the value types of the cycle and of the CG vectors (FP64 or FP32), with the
+// integer-step casts (fdiv.cuh) where they pay: in the r and p updates
+__device__ __forceinline__ double to_f64(double x) { return x; }
+__device__ __forceinline__ double to_f64(float x) { return f32_to_f64(x); }
+template <class V>
+__device__ __forceinline__ V to_value(double x);
+template <>
+__device__ __forceinline__ double to_value<double>(double x) { return x; }
+template <>
+__device__ __forceinline__ float to_value<float>(double x) { return f64_to_f32_rn(x); }
+
 // u = A_L^-1 f, one warp per row
 template <class TF, class TO>
 __global__ void k_coarse_solve(int32_t n, const double *__restrict__ inv, const TF *__restrict__ f,
@@ -1534,10 +1545,10 @@ __global__ void k_smooth_sweep(int32_t n, M A, const typename M::value *__restri
 // z = u_in + m o (r - A u_in) and a per-block partial of r.z (block_sum order)
 __device__ double block_sum(double v);
 __device__ bool cg_reduce(double d, double *partial, unsigned *counter, double *total);
-template <class M>
+template <class M, class TZ>
 __global__ void __launch_bounds__(kCgThreads)
 k_smooth_sweep_dot(int32_t n, M A, const typename M::value *__restrict__ m, const double *__restrict__ f,
-                   const typename M::value *__restrict__ u_in, double *__restrict__ z, double *__restrict__ partial,
+                   const typename M::value *__restrict__ u_in, TZ *__restrict__ z, double *__restrict__ partial,
                    CgState *cg, const int *skip) {
     using V = typename M::value;
     constexpr int LPR = M::lanes;
@@ -1557,9 +1568,9 @@ k_smooth_sweep_dot(int32_t n, M A, const typename M::value *__restrict__ m, cons
         s = group_sum<LPR>(s);
         if (gt < total && sub == 0) {
             const double fi = f[i];
-            const double zi = (double)fma(m[i], (V)fi - s, u_in[i]);
-            z[i] = zi;
-            d = fma(fi, zi, d);
+            const V zi = fma(m[i], (V)fi - s, u_in[i]);
+            z[i] = (TZ)zi;
+            d = fma(fi, (double)zi, d);
         }
     }
     // the last block stores the new r.z in the CG state
@@ -1740,6 +1751,7 @@ __global__ void k_cg_init(int32_t n, const double *__restrict__ f, double *__res
         cg->replacements = 0;
         cg->need_true = 0;
         cg->copy_r = 0;
+        cg->u_done = 0;
         cg->pad = 0;
         cg->rz = cg->rz_next = cg->rzo = 0.0;
         cg->alpha = cg->beta = cg->pq = cg->rr = cg->res = cg->tres = 0.0;
@@ -1767,11 +1779,12 @@ __global__ void k_dot(int32_t n, const double *__restrict__ x, const double *__r
 }
 
 // after the first preconditioner application: p = z, r.z becomes current
-__global__ void k_cg_set_rz_p(int32_t n, const double *__restrict__ z, double *__restrict__ p, CgState *cg) {
+template <class TZ>
+__global__ void k_cg_set_rz_p(int32_t n, const TZ *__restrict__ z, double *__restrict__ p, CgState *cg) {
     pdl_wait();
     if (cg->done) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) cg->rz = cg->rz_next;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = z[i];
+    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = (double)z[i];
 }
 
 // q = A p; the last block forms p.q and alpha = r.z / p.q (breakdown: p.q <= 0)
@@ -1794,6 +1807,7 @@ k_spmv_dot(int32_t n, M A, const double *__restrict__ p, double *__restrict__ q,
     double pq = 0.0;
     if (cg_reduce(d, partial, &cg->ctr[CG_CTR_PQ], &pq) && threadIdx.x == 0) {
         cg->pq = pq;
+        cg->u_done = 0;
         if (!(pq > 0.0) || !isfinite(pq)) {
             cg->iter += 1;
             cg->status = AMG_ERR_BREAKDOWN;
@@ -1804,14 +1818,23 @@ k_spmv_dot(int32_t n, M A, const double *__restrict__ p, double *__restrict__ q,
     }
 }
 
-// u += alpha p, r -= alpha q; the last block checks the recurrence residual
-// (graph: opens the IF branch hb of the true-residual check when it meets tol).
-// With zo (the flexible variant), also r_new.z_old into cg->rzo, summed as the
-// separate dot kernel would sum it (same grid, same order).
-__global__ void k_cg_update_ur(int32_t n, CgState *cg, const double *__restrict__ p, const double *__restrict__ q,
-                               double *__restrict__ u, double *__restrict__ r, double *__restrict__ partial,
-                               const double *__restrict__ zo, double *__restrict__ part_zo, int use_h,
-                               cudaGraphConditionalHandle hb, Smooth0Out z0) {
+// r -= alpha q, u0 = m o r; the last block checks the recurrence residual
+// (graph: opens the IF branch hb of the true-residual check when it meets tol,
+// or when maxiter ends the iteration).  u += alpha p is left to the p update,
+// which reads p anyway; where the iteration ends, to k_cg_update_u in the
+// branch (cg->u_done then tells the p update).  With zo (the flexible variant),
+// also r_new.z_old into cg->rzo.
+// Two rows' loads are in flight per thread, before any store (the compiler may
+// not move a load across one), and the casts are integer steps.  192^3, mixed:
+// with u, p and an FP64 z in this kernel 97.5 us (64 bytes a row) and the p
+// update 21.6; now 56 (36 bytes a row, 4.6 TB/s; three FP64 operations a row)
+// and 31 (36 bytes, 8.2 TB/s with what L2 keeps).  With conversion
+// instructions the two took 83 and 40.
+template <class TZ, class V>
+__global__ void __launch_bounds__(kCgThreads, 4)
+k_cg_update_r(int32_t n, CgState *cg, const double *__restrict__ q, double *__restrict__ r,
+              double *__restrict__ partial, const TZ *__restrict__ zo, double *__restrict__ part_zo, int use_h,
+              cudaGraphConditionalHandle hb, const V *__restrict__ m, V *__restrict__ u0) {
     pdl_wait();
     if (cg->done) {
         if (use_h && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(hb, 0u);
@@ -1819,13 +1842,23 @@ __global__ void k_cg_update_ur(int32_t n, CgState *cg, const double *__restrict_
     }
     const double alpha = cg->alpha;
     double s = 0.0, so = 0.0;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        u[i] = fma(alpha, p[i], u[i]);
-        const double ri = fma(-alpha, q[i], r[i]);
+    const int32_t stride = gridDim.x * blockDim.x;
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 2 * (int64_t)stride) {
+        const int32_t i = (int32_t)i0, j = i0 + stride < n ? (int32_t)(i0 + stride) : i;
+        const double qi = q[i], ri0 = r[i], qj = q[j], rj0 = r[j];
+        const TZ zi = zo ? zo[i] : TZ(0), zj = zo ? zo[j] : TZ(0);
+        const V mi = u0 ? m[i] : V(0), mj = u0 ? m[j] : V(0);
+        const double ri = fma(-alpha, qi, ri0), rj = fma(-alpha, qj, rj0);
         r[i] = ri;
-        put_smooth0(z0, i, ri);
+        if (u0) u0[i] = mi * to_value<V>(ri);
         s = fma(ri, ri, s);
-        if (zo) so = fma(ri, zo[i], so);
+        if (zo) so = fma(ri, to_f64(zi), so);
+        if (j != i) {
+            r[j] = rj;
+            if (u0) u0[j] = mj * to_value<V>(rj);
+            s = fma(rj, rj, s);
+            if (zo) so = fma(rj, to_f64(zj), so);
+        }
     }
     double rr = 0.0, rzo = 0.0;
     const bool last = zo ? cg_reduce2(s, so, partial, part_zo, &cg->ctr[CG_CTR_RR], &rr, &rzo)
@@ -1840,8 +1873,18 @@ __global__ void k_cg_update_ur(int32_t n, CgState *cg, const double *__restrict_
             cg->done = 1;
             cg->status = AMG_NOT_CONVERGED;
         }
-        if (use_h) cudaGraphSetConditional(hb, (cg->need_true && !cg->done) ? 1u : 0u);
+        cg->u_done = cg->need_true || cg->done;
+        if (use_h) cudaGraphSetConditional(hb, cg->u_done ? 1u : 0u);
     }
+}
+
+// u += alpha p where the iteration ends (or may end: before the true residual)
+__global__ void k_cg_update_u(int32_t n, const CgState *cg, const double *__restrict__ p, double *__restrict__ u) {
+    pdl_wait();
+    if (!cg->u_done) return;
+    const double alpha = cg->alpha;
+    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        u[i] = fma(alpha, p[i], u[i]);
 }
 
 // t = f - A u, the true residual, when the recurrence reports convergence; the
@@ -1882,8 +1925,9 @@ k_true_residual(int32_t n, M A, const double *__restrict__ f, const double *__re
 
 // r = t when the true residual replaces the recurrence residual; with zo (the
 // flexible variant), r_new.z_old is formed again from the new r
+template <class TZ>
 __global__ void k_replace_r(int32_t n, CgState *cg, const double *__restrict__ t, double *__restrict__ r,
-                            const double *__restrict__ zo, double *__restrict__ part_zo, Smooth0Out z0) {
+                            const TZ *__restrict__ zo, double *__restrict__ part_zo, Smooth0Out z0) {
     pdl_wait();
     if (cg->done || !cg->copy_r) return;
     double so = 0.0;
@@ -1891,7 +1935,7 @@ __global__ void k_replace_r(int32_t n, CgState *cg, const double *__restrict__ t
         const double ti = t[i];
         r[i] = ti;
         put_smooth0(z0, i, ti);
-        if (zo) so = fma(ti, zo[i], so);
+        if (zo) so = fma(ti, (double)zo[i], so);
     }
     if (!zo) return;
     double rzo = 0.0;
@@ -1899,12 +1943,14 @@ __global__ void k_replace_r(int32_t n, CgState *cg, const double *__restrict__ t
 }
 
 // beta = (r.z_new - r.z_old) / (r.z)_old, the flexible form (r.z_old = 0 for
-// standard CG), p = z + beta p.  The new r.z becomes current in the next
+// standard CG), u += alpha p (unless u_done), p = z + beta p.  The new r.z becomes current in the next
 // iteration's first kernel.  In the graph this is the body's last kernel: it
 // keeps the while loop going while the iteration is not done, with a hard
 // cap of maxiter + 4 bodies.
-__global__ void k_cg_update_p(int32_t n, CgState *cg, const double *__restrict__ z, double *__restrict__ p,
-                              int use_h, cudaGraphConditionalHandle h) {
+template <class TZ>
+__global__ void __launch_bounds__(kCgThreads, 4)
+k_cg_update_p(int32_t n, CgState *cg, const TZ *__restrict__ z, double *__restrict__ p, double *__restrict__ u,
+              int use_h, cudaGraphConditionalHandle h) {
     pdl_wait();
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
     if (cg->done) {
@@ -1916,9 +1962,20 @@ __global__ void k_cg_update_p(int32_t n, CgState *cg, const double *__restrict__
     __shared__ double s_beta;
     if (threadIdx.x == 0) s_beta = (cg->rz_next - cg->rzo) / cg->rz;
     __syncthreads();
-    const double beta = s_beta;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        p[i] = fma(beta, p[i], z[i]);
+    const double beta = s_beta, alpha = cg->alpha;
+    const bool with_u = !cg->u_done;
+    const int32_t stride = gridDim.x * blockDim.x;
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 2 * (int64_t)stride) {
+        const int32_t i = (int32_t)i0, j = i0 + stride < n ? (int32_t)(i0 + stride) : i;
+        const double pi = p[i], ui = u[i], pj = p[j], uj = u[j];
+        const TZ zi = z[i], zj = z[j];
+        p[i] = fma(beta, pi, to_f64(zi));
+        if (with_u) u[i] = fma(alpha, pi, ui);
+        if (j != i) {
+            p[j] = fma(beta, pj, to_f64(zj));
+            if (with_u) u[j] = fma(alpha, pj, uj);
+        }
+    }
     if (lead) {
         cg->beta = beta;
         cg->copy_r = 0;
@@ -2437,20 +2494,21 @@ void launch_smooth_sweep(const Level &L, const V *val, const V *m, const TF *f, 
                    u_out, skip);
     });
 }
-template <class V>
-void launch_smooth_sweep_dot(const Level &L, const V *val, const V *m, const double *f, const V *u_in, double *z,
+template <class V, class TZ>
+void launch_smooth_sweep_dot(const Level &L, const V *val, const V *m, const double *f, const V *u_in, TZ *z,
                              double *partial, CgState *cg, const int *skip, cudaStream_t s) {
     count_launch();
     with_level_rows<V>(L, val, [&](auto A) {
-        launch_pdl(k_smooth_sweep_dot<decltype(A)>, cg_blocks(L.n * lanes_of(A)), kCgThreads, 0, s, L.n, A, m, f, u_in,
+        launch_pdl(k_smooth_sweep_dot<decltype(A), TZ>, cg_blocks(L.n * lanes_of(A)), kCgThreads, 0, s, L.n, A, m, f, u_in,
                    z, partial, cg, skip);
     });
 }
-template void launch_smooth_sweep_dot<double>(const Level &, const double *, const double *, const double *,
-                                              const double *, double *, double *, CgState *, const int *,
-                                              cudaStream_t);
-template void launch_smooth_sweep_dot<float>(const Level &, const float *, const float *, const double *,
-                                             const float *, double *, double *, CgState *, const int *, cudaStream_t);
+template void launch_smooth_sweep_dot<double, double>(const Level &, const double *, const double *, const double *,
+                                                      const double *, double *, double *, CgState *, const int *,
+                                                      cudaStream_t);
+template void launch_smooth_sweep_dot<float, float>(const Level &, const float *, const float *, const double *,
+                                                    const float *, float *, double *, CgState *, const int *,
+                                                    cudaStream_t);
 template <class V, class TF>
 void launch_residual(const Level &L, const V *val, const TF *f, const V *u, V *r, const int *skip, cudaStream_t s) {
     count_launch();
@@ -2546,9 +2604,10 @@ void launch_dot(int32_t n, const double *x, const double *y, double *partial, co
     count_launch();
     launch_pdl(k_dot, cg_blocks(n), kCgThreads, 0, s, n, x, y, partial, skip, cg, target);
 }
-void launch_cg_set_rz_p(int32_t n, const double *z, double *p, CgState *cg, cudaStream_t s) {
+template <class TZ>
+void launch_cg_set_rz_p(int32_t n, const TZ *z, double *p, CgState *cg, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_cg_set_rz_p, cg_blocks(n), kCgThreads, 0, s, n, z, p, cg);
+    launch_pdl(k_cg_set_rz_p<TZ>, cg_blocks(n), kCgThreads, 0, s, n, z, p, cg);
 }
 void launch_spmv_dot(int32_t n, const FineMat &A, const double *p, double *q, double *partial, CgState *cg,
                      cudaStream_t s) {
@@ -2557,12 +2616,21 @@ void launch_spmv_dot(int32_t n, const FineMat &A, const double *p, double *q, do
         launch_pdl(k_spmv_dot<decltype(M)>, cg_blocks(n), kCgThreads, 0, s, n, M, p, q, partial, cg);
     });
 }
-void launch_cg_update_ur(int32_t n, CgState *cg, const double *p, const double *q, double *u, double *r,
-                         double *partial, const double *zo, double *part_zo, int use_h, cudaGraphConditionalHandle hb,
-                         const Smooth0Out &z0, cudaStream_t s) {
+template <class TZ>
+void launch_cg_update_r(int32_t n, CgState *cg, const double *q, double *r, double *partial, const TZ *zo,
+                        double *part_zo, int use_h, cudaGraphConditionalHandle hb, const Smooth0Out &z0,
+                        cudaStream_t s) {
     count_launch();
-    launch_pdl(k_cg_update_ur, cg_blocks(n), kCgThreads, 0, s, n, cg, p, q, u, r, partial, zo, part_zo, use_h, hb,
-               z0);
+    if (z0.uf)
+        launch_pdl(k_cg_update_r<TZ, float>, cg_blocks(n), kCgThreads, 0, s, n, cg, q, r, partial, zo, part_zo, use_h,
+                   hb, z0.mf, z0.uf);
+    else
+        launch_pdl(k_cg_update_r<TZ, double>, cg_blocks(n), kCgThreads, 0, s, n, cg, q, r, partial, zo, part_zo, use_h,
+                   hb, z0.m, z0.u);
+}
+void launch_cg_update_u(int32_t n, const CgState *cg, const double *p, double *u, cudaStream_t s) {
+    count_launch();
+    launch_pdl(k_cg_update_u, cg_blocks(n), kCgThreads, 0, s, n, cg, p, u);
 }
 void launch_col_delta16(int32_t n, const int32_t *ptr, const int32_t *col, float ratio, int16_t *c16, int *flag,
                         cudaStream_t s) {
@@ -2586,17 +2654,30 @@ void launch_true_residual(int32_t n, const FineMat &A, const double *f, const do
         launch_pdl(k_true_residual<decltype(M)>, cg_blocks(n), kCgThreads, 0, s, n, M, f, u, t, partial, cg, force);
     });
 }
-void launch_replace_r(int32_t n, CgState *cg, const double *t, double *r, const double *zo, double *part_zo,
+template <class TZ>
+void launch_replace_r(int32_t n, CgState *cg, const double *t, double *r, const TZ *zo, double *part_zo,
                       const Smooth0Out &z0, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_replace_r, cg_blocks(n), kCgThreads, 0, s, n, cg, t, r, zo, part_zo, z0);
+    launch_pdl(k_replace_r<TZ>, cg_blocks(n), kCgThreads, 0, s, n, cg, t, r, zo, part_zo, z0);
 }
-void launch_cg_update_p(int32_t n, CgState *cg, const double *z, double *p, int use_h, cudaGraphConditionalHandle h,
-                        cudaStream_t s) {
+template <class TZ>
+void launch_cg_update_p(int32_t n, CgState *cg, const TZ *z, double *p, double *u, int use_h,
+                        cudaGraphConditionalHandle h, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_cg_update_p, cg_blocks(n), kCgThreads, 0, s, n, cg, z, p, use_h, h);
+    launch_pdl(k_cg_update_p<TZ>, cg_blocks(n), kCgThreads, 0, s, n, cg, z, p, u, use_h, h);
 }
-
+#define INST_CG(TZ)                                                                                                  \
+    template void launch_cg_set_rz_p<TZ>(int32_t, const TZ *, double *, CgState *, cudaStream_t);                    \
+    template void launch_cg_update_r<TZ>(int32_t, CgState *, const double *, double *, double *, const TZ *,         \
+                                         double *, int, cudaGraphConditionalHandle, const Smooth0Out &,              \
+                                         cudaStream_t);                                                              \
+    template void launch_replace_r<TZ>(int32_t, CgState *, const double *, double *, const TZ *, double *,           \
+                                       const Smooth0Out &, cudaStream_t);                                            \
+    template void launch_cg_update_p<TZ>(int32_t, CgState *, const TZ *, double *, double *, int,                    \
+                                         cudaGraphConditionalHandle, cudaStream_t);
+INST_CG(double)
+INST_CG(float)
+#undef INST_CG
 
 void launch_bi_init(int32_t n, const double *f, double *x, double *r, double *rh, double *p, double *v,
                     double *partial, BiState *st, double tol, int maxiter, cudaStream_t s) {

@@ -105,3 +105,22 @@ def test_stencil_bicgstab_and_full_reuse(noff):
         u, info = G.solve(cuda(f)[0], 1e-9)
         assert info.status == 0
         assert np.linalg.norm(f - scale * (A @ u.cpu().numpy())) <= 1.01e-9 * np.linalg.norm(f)
+
+
+@pytest.mark.parametrize("maxiter,precision,nlev1", [(1, 0, False), (2, 0, False), (7, 0, False), (1, 1, False),
+                                                     (6, 1, False), (1, 0, True), (1, 1, True)])
+def test_iterate_when_maxiter_ends_it(maxiter, precision, nlev1):
+    """u += alpha p is part of the p update except where the iteration ends:
+    the iterate left by maxiter against the oracle's, FP64 (1e-10) and with an
+    FP32 cycle (its rounding, 1e-4), with and without a coarse level."""
+    n = 1000
+    ptr, col, val = stencil_matrix(n, SYM[5], 1.0, seed=maxiter)
+    kw = dict(coarse_enough=n if nlev1 else 50)
+    f = np.random.default_rng(6).normal(size=n)
+    G = B.AMG(precision=precision, maxiter=maxiter, **kw)
+    G.full_setup(*cuda(ptr, col, val))
+    u, info = G.solve(cuda(f)[0], 1e-30)
+    H = O.Hierarchy(ptr, col, val, O.Params(**kw))
+    uo, it, rr, st = H.pcg(f, 1e-30, maxiter=maxiter)
+    assert info.iters == it and info.status != 0 and st != 0
+    assert np.linalg.norm(u.cpu().numpy() - uo) <= (1e-10 if precision == 0 else 1e-4) * np.linalg.norm(uo)
