@@ -1034,7 +1034,8 @@ void enqueue_vcycle(amg_ctx *ctx, const double *r, TZ *z, const int *skip, doubl
 
 // Alg. 2 on the 4 x 4 block hierarchy (damped block Jacobi, zero initial
 // guess on every level, dense inverse on the coarsest), z = B r
-void enqueue_block_vcycle(amg_ctx *ctx, const double *r, double *z, const int *skip) {
+// (u0_ready: the producer of r has written the finest level's first step)
+void enqueue_block_vcycle(amg_ctx *ctx, const double *r, double *z, const int *skip, bool u0_ready) {
     const int nl = ctx->nlev;
     const int npre = ctx->prm.npre, npost = ctx->prm.npost;
     if (nl == 1) {
@@ -1049,14 +1050,17 @@ void enqueue_block_vcycle(amg_ctx *ctx, const double *r, double *z, const int *s
         if (npre <= 0) {
             (void)(cudaMemsetAsync(u, 0, sizeof(double) * 4 * (size_t)L.n, ctx->s));
         } else {
-            { ProfScope ps_(ctx, AMG_PROF_SMOOTH0_L0, l == 0); launch_block_smooth0(L.n, L.Minv, f, u, skip, ctx->s); }
+            // the coarser levels' first step is written by the restriction
+            if (l == 0 && !u0_ready) { ProfScope ps_(ctx, AMG_PROF_SMOOTH0_L0); launch_block_smooth0(L.n, L.Minv, f, u, skip, ctx->s); }
             for (int k = 1; k < npre; ++k) {
                 launch_block_sweep(L.n, L.A_ptr, L.A_col, L.Ab, L.Minv, f, u, t, skip, ctx->s);
                 std::swap(u, t);
             }
         }
         launch_block_residual(L.n, L.A_ptr, L.A_col, L.Ab, f, u, L.vd.r, skip, ctx->s);
-        { ProfScope ps_(ctx, AMG_PROF_RESTRICT_L0, l == 0); launch_block_restrict(L.nc, L.R_ptr, L.R_col, L.R_val, L.vd.r, ctx->lev[l + 1].vd.f, skip, ctx->s); }
+        Level &C = ctx->lev[l + 1];
+        const bool smooth = npre > 0 && l + 1 < nl - 1;
+        { ProfScope ps_(ctx, AMG_PROF_RESTRICT_L0, l == 0); launch_block_restrict(L.nc, L.R_ptr, L.R_col, L.R_val, L.vd.r, C.vd.f, smooth ? C.Minv : nullptr, smooth ? C.vd.u : nullptr, skip, ctx->s); }
         cur[l] = u;
     }
     Level &Cst = ctx->lev[nl - 1];
@@ -1084,7 +1088,7 @@ void enqueue_block_vcycle(amg_ctx *ctx, const double *r, double *z, const int *s
 // u0_ready: the producer of r has written the finest level's u0 (cg_smooth0)
 void vcycle(amg_ctx *ctx, const double *r, double *z, const int *skip, double *rz_partial = nullptr,
             bool u0_ready = false) {
-    if (blockmode(ctx)) enqueue_block_vcycle(ctx, r, z, skip);
+    if (blockmode(ctx)) enqueue_block_vcycle(ctx, r, z, skip, u0_ready);
     else if (mixed(ctx)) enqueue_vcycle<float, double>(ctx, r, z, skip, rz_partial, u0_ready);
     else enqueue_vcycle<double, double>(ctx, r, z, skip, rz_partial, u0_ready);
 }
@@ -1093,16 +1097,16 @@ void vcycle(amg_ctx *ctx, const double *r, double *z, const int *skip, double *r
 // CG prologue: u = 0, r = f, z = B r, p = z, rz = r.z (device state in ctx->cg)
 // the CG kernels that produce r also write the V-cycle's first finest-level
 // smoothing step from zero, u0 = m o r (when the V-cycle has a smoothed level)
+bool cg_u0(const amg_ctx *ctx) { return ctx->nlev >= 2 && ctx->prm.npre >= 1; }
 Smooth0Out cg_smooth0(amg_ctx *ctx) {
     Smooth0Out z0;
-    if (ctx->nlev < 2 || ctx->prm.npre < 1 || blockmode(ctx)) return z0;
+    if (!cg_u0(ctx)) return z0;
     Level &F = ctx->lev[0];
-    if (mixed(ctx)) { z0.mf = F.mf; z0.uf = F.vf.u; }
+    if (blockmode(ctx)) { z0.minv = F.Minv; z0.u = F.vd.u; }
+    else if (mixed(ctx)) { z0.mf = F.mf; z0.uf = F.vf.u; }
     else { z0.m = F.m; z0.u = F.vd.u; }
     return z0;
 }
-bool cg_u0(amg_ctx *ctx) { return ctx->nlev >= 2 && ctx->prm.npre >= 1 && !blockmode(ctx); }
-
 // CG holds z as the cycle makes it: in FP32 when the last sweep of a
 // mixed-precision cycle writes it (then in cg_z's memory as floats)
 bool cg_z32(const amg_ctx *ctx) { return mixed(ctx) && ctx->nlev >= 2 && ctx->prm.npost >= 1; }
@@ -1345,18 +1349,16 @@ void enqueue_bi_iter(amg_ctx *ctx, const double *f, double *u, int use_h, cudaGr
     const int bs = ctx->prm.block_size;
     BiState *st = ctx->bi;
     double *part = ctx->partial;
-    launch_bi_rho(n, ctx->bi_rh, ctx->cg_r, part, st, ctx->s);
-    launch_bi_p(n, ctx->cg_r, ctx->cg_q, ctx->cg_p, st, ctx->s);
-    vcycle(ctx, ctx->cg_p, ctx->cg_z, &st->done);
+    // p and s come with the V-cycle's first smoothing step (cg_smooth0)
+    launch_bi_p(n, ctx->cg_r, ctx->cg_q, ctx->cg_p, st, cg_smooth0(ctx), ctx->s);
+    vcycle(ctx, ctx->cg_p, ctx->cg_z, &st->done, nullptr, cg_u0(ctx));
     launch_bi_spmv_rv(n, bs, fine_mat(ctx), ctx->cg_z, ctx->cg_q, ctx->bi_rh, part, st, ctx->s);
-    launch_bi_s(n, ctx->cg_r, ctx->cg_q, ctx->bi_s, part, st, ctx->s);
-    launch_bi_half(n, ctx->cg_z, ctx->bi_s, u, ctx->cg_r, st, ctx->s);
-    vcycle(ctx, ctx->bi_s, ctx->bi_sh, &st->skip);
+    launch_bi_s(n, ctx->cg_r, ctx->cg_q, ctx->bi_s, part, st, cg_smooth0(ctx), ctx->s);
+    vcycle(ctx, ctx->bi_s, ctx->bi_sh, &st->skip, nullptr, cg_u0(ctx));
     launch_bi_spmv_t(n, bs, fine_mat(ctx), ctx->bi_sh, ctx->bi_s, ctx->cg_t, part, st, ctx->s);
-    launch_bi_xr(n, ctx->cg_z, ctx->bi_sh, ctx->bi_s, ctx->cg_t, u, ctx->cg_r, part, st, ctx->s);
+    launch_bi_xr(n, ctx->cg_z, ctx->bi_sh, ctx->bi_s, ctx->cg_t, ctx->bi_rh, u, ctx->cg_r, part, st, ctx->s);
     launch_bi_true(n, bs, fine_mat(ctx), f, u, ctx->cg_t, part, st, 0, ctx->s);
-    launch_bi_replace(n, ctx->cg_t, ctx->cg_r, st, ctx->s);
-    launch_bi_end(st, use_h, h, ctx->s);
+    launch_bi_end(n, ctx->cg_t, ctx->bi_rh, ctx->cg_r, part, st, use_h, h, ctx->s);
 }
 
 void enqueue_bi_epilogue(amg_ctx *ctx, const double *f, double *u) {

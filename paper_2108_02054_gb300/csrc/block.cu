@@ -187,136 +187,98 @@ __global__ void k_block_to_dense(int32_t n, const int32_t *__restrict__ ptr, con
                 dense[(4 * (int64_t)i + r) * n4 + 4 * (int64_t)col[e] + c] = bv[(int64_t)16 * e + 4 * r + c];
 }
 
-// ------------------------------------------------------------------ V-cycle pieces (one thread per node)
-__device__ __forceinline__ void load4(const double *p, double v[4]) {
-    const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
-    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-}
-__device__ __forceinline__ void store4(double *p, const double v[4]) {
-    reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
-    reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
-}
-
-// (A x)_i, component r summing in entry order then component order (fma from 0)
-__device__ __forceinline__ void block_row(int32_t i, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                                          const double *__restrict__ bv, const double *__restrict__ x, double y[4]) {
-    y[0] = y[1] = y[2] = y[3] = 0.0;
-    for (int32_t e = ptr[i]; e < ptr[i + 1]; ++e) {
-        double xv[4];
-        load4(x + (int64_t)4 * col[e], xv);
-        const double2 *b = reinterpret_cast<const double2 *>(bv + (int64_t)16 * e);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const double2 lo = b[2 * r], hi = b[2 * r + 1];
-            y[r] = fma(lo.x, xv[0], y[r]);
-            y[r] = fma(lo.y, xv[1], y[r]);
-            y[r] = fma(hi.x, xv[2], y[r]);
-            y[r] = fma(hi.y, xv[3], y[r]);
-        }
-    }
-}
-
-// u_out = u_in + Minv_i t (fma from u_in, component order)
-__device__ __forceinline__ void apply_minv(const double *__restrict__ m, const double t[4], const double uin[4],
-                                           double uout[4]) {
-    const double2 *M = reinterpret_cast<const double2 *>(m);
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const double2 lo = M[2 * r], hi = M[2 * r + 1];
-        double s = uin[r];
-        s = fma(lo.x, t[0], s);
-        s = fma(lo.y, t[1], s);
-        s = fma(hi.x, t[2], s);
-        s = fma(hi.y, t[3], s);
-        uout[r] = s;
-    }
-}
+// ------------------------------------------------------------------ V-cycle pieces
+// One thread per unknown, the four of a node side by side: a quad reads a
+// block's 128 bytes as one line (32 bytes a lane) and a node's vector entries
+// as one sector, and a coarse level of a thousand nodes still gives 4000
+// threads with a fourth of the serial work.  (With one thread per node each
+// load of a warp touched 32 lines, and a coarse row's 16 fma an entry ran one
+// after the other.)  What is left on the
+// finest level is the FP64 pipe (16 fma a block, 25 us at 760,320 blocks), on
+// the coarse ones the serial sum.  Measured at 48^3 per launch, one thread per
+// node -> per unknown, levels of 110,592 / 15,216 / 1,000 nodes: residual 32.9
+// / 30.5 / 36.4 -> 28.4 / 13.5 / 13.3 us, sweep 36.1 / 22.0 / 24.6 -> 31.3 /
+// 11.8 / 8.6, restriction 10.6 / 14.2 / 16.6 -> 10.1 / 9.1 / 9.0.
 
 // first pre-smoothing step from u = 0: u = Minv f
-__global__ void k_block_smooth0(int32_t n, const double *__restrict__ minv, const double *__restrict__ f,
-                                double *__restrict__ u, const int *skip) {
+__global__ void __launch_bounds__(kBThreads)
+k_block_smooth0(int32_t n, const double *__restrict__ minv, const double *__restrict__ f, double *__restrict__ u,
+                const int *skip) {
     pdl_wait();
     if (skip && *skip) return;
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double t[4], z[4] = {0.0, 0.0, 0.0, 0.0}, o[4];
-    load4(f + (int64_t)4 * i, t);
-    apply_minv(minv + (int64_t)16 * i, t, z, o);
-    store4(u + (int64_t)4 * i, o);
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 4 * (int64_t)n) return;  // whole quads
+    u[t] = quad_minv(minv, t, f[t], 0.0);
 }
 
 // one damped block-Jacobi sweep: u_out = u_in + Minv (f - A u_in)
-__global__ void k_block_sweep(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                              const double *__restrict__ bv, const double *__restrict__ minv,
-                              const double *__restrict__ f, const double *__restrict__ uin, double *__restrict__ uout,
-                              const int *skip) {
+__global__ void __launch_bounds__(kBThreads)
+k_block_sweep(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
+              const double *__restrict__ bv, const double *__restrict__ minv, const double *__restrict__ f,
+              const double *__restrict__ uin, double *__restrict__ uout, const int *skip) {
     pdl_wait();
     if (skip && *skip) return;
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double y[4], fv[4], t[4], u0[4], o[4];
-    block_row(i, ptr, col, bv, uin, y);
-    load4(f + (int64_t)4 * i, fv);
-#pragma unroll
-    for (int r = 0; r < 4; ++r) t[r] = fv[r] - y[r];
-    load4(uin + (int64_t)4 * i, u0);
-    apply_minv(minv + (int64_t)16 * i, t, u0, o);
-    store4(uout + (int64_t)4 * i, o);
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 4 * (int64_t)n) return;
+    const double y = block_dot<true>(ptr, col, bv, uin, (int32_t)(t >> 2), (int)(t & 3));
+    uout[t] = quad_minv(minv, t, f[t] - y, uin[t]);
 }
 
 // r = f - A u
-__global__ void k_block_residual(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                                 const double *__restrict__ bv, const double *__restrict__ f,
-                                 const double *__restrict__ u, double *__restrict__ r, const int *skip) {
+__global__ void __launch_bounds__(kBThreads)
+k_block_residual(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
+                 const double *__restrict__ bv, const double *__restrict__ f, const double *__restrict__ u,
+                 double *__restrict__ r, const int *skip) {
     pdl_wait();
     if (skip && *skip) return;
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double y[4], fv[4];
-    block_row(i, ptr, col, bv, u, y);
-    load4(f + (int64_t)4 * i, fv);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) fv[k] = fv[k] - y[k];
-    store4(r + (int64_t)4 * i, fv);
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 4 * (int64_t)n) return;
+    r[t] = f[t] - block_dot<true>(ptr, col, bv, u, (int32_t)(t >> 2), (int)(t & 3));
 }
 
-// f_c = R r (scalar R, per component: fma from 0 in R's column order)
-__global__ void k_block_restrict(int32_t nc, const int32_t *__restrict__ Rptr, const int32_t *__restrict__ Rcol,
-                                 const double *__restrict__ Rval, const double *__restrict__ r,
-                                 double *__restrict__ fc, const int *skip) {
+// f_c = R r (scalar R, per component: fma from 0 in R's column order), four
+// entries' loads in flight; with minv also the coarse level's first smoothing
+// step from zero, u_c = Minv f_c
+__global__ void __launch_bounds__(kBThreads)
+k_block_restrict(int32_t nc, const int32_t *__restrict__ Rptr, const int32_t *__restrict__ Rcol,
+                 const double *__restrict__ Rval, const double *__restrict__ r, double *__restrict__ fc,
+                 const double *__restrict__ minv, double *__restrict__ uc, const int *skip) {
     pdl_wait();
     if (skip && *skip) return;
-    const int32_t I = blockIdx.x * blockDim.x + threadIdx.x;
-    if (I >= nc) return;
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int32_t p = Rptr[I]; p < Rptr[I + 1]; ++p) {
-        double v[4];
-        load4(r + (int64_t)4 * Rcol[p], v);
-        const double w = Rval[p];
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 4 * (int64_t)nc) return;
+    const int32_t I = (int32_t)(t >> 2), c = (int32_t)(t & 3);
+    double s = 0.0;
+    const int32_t p1 = Rptr[I + 1];
+    int32_t p = Rptr[I];
+    for (; p + 4 <= p1; p += 4) {
+        double w[4], v[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) s[c] = fma(w, v[c], s[c]);
+        for (int k = 0; k < 4; ++k) {
+            w[k] = Rval[p + k];
+            v[k] = r[(int64_t)4 * Rcol[p + k] + c];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s = fma(w[k], v[k], s);
     }
-    store4(fc + (int64_t)4 * I, s);
+    for (; p < p1; ++p) s = fma(Rval[p], r[(int64_t)4 * Rcol[p] + c], s);
+    fc[t] = s;
+    if (uc) uc[t] = quad_minv(minv, t, s, 0.0);
 }
 
 // u += P u_c
-__global__ void k_block_prolong(int32_t n, const int32_t *__restrict__ Pptr, const int32_t *__restrict__ Pcol,
-                                const double *__restrict__ Pval, const double *__restrict__ uc,
-                                double *__restrict__ u, const int *skip) {
+__global__ void __launch_bounds__(kBThreads)
+k_block_prolong(int32_t n, const int32_t *__restrict__ Pptr, const int32_t *__restrict__ Pcol,
+                const double *__restrict__ Pval, const double *__restrict__ uc, double *__restrict__ u,
+                const int *skip) {
     pdl_wait();
     if (skip && *skip) return;
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double s[4];
-    load4(u + (int64_t)4 * i, s);
-    for (int32_t p = Pptr[i]; p < Pptr[i + 1]; ++p) {
-        double v[4];
-        load4(uc + (int64_t)4 * Pcol[p], v);
-        const double w = Pval[p];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) s[c] = fma(w, v[c], s[c]);
-    }
-    store4(u + (int64_t)4 * i, s);
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 4 * (int64_t)n) return;
+    const int32_t i = (int32_t)(t >> 2), c = (int32_t)(t & 3);
+    double s = u[t];
+    for (int32_t p = Pptr[i]; p < Pptr[i + 1]; ++p) s = fma(Pval[p], uc[(int64_t)4 * Pcol[p] + c], s);
+    u[t] = s;
 }
 
 }  // namespace
@@ -350,27 +312,27 @@ void launch_block_to_dense(int32_t n, const int32_t *ptr, const int32_t *col, co
 void launch_block_smooth0(int32_t n, const double *minv, const double *f, double *u, const int *skip,
                           cudaStream_t s) {
     count_launch();
-    launch_pdl(k_block_smooth0, bblocks(n), kBThreads, 0, s, n, minv, f, u, skip);
+    launch_pdl(k_block_smooth0, bblocks(4 * (int64_t)n), kBThreads, 0, s, n, minv, f, u, skip);
 }
 void launch_block_sweep(int32_t n, const int32_t *ptr, const int32_t *col, const double *bv, const double *minv,
                         const double *f, const double *uin, double *uout, const int *skip, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_block_sweep, bblocks(n), kBThreads, 0, s, n, ptr, col, bv, minv, f, uin, uout, skip);
+    launch_pdl(k_block_sweep, bblocks(4 * (int64_t)n), kBThreads, 0, s, n, ptr, col, bv, minv, f, uin, uout, skip);
 }
 void launch_block_residual(int32_t n, const int32_t *ptr, const int32_t *col, const double *bv, const double *f,
                            const double *u, double *r, const int *skip, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_block_residual, bblocks(n), kBThreads, 0, s, n, ptr, col, bv, f, u, r, skip);
+    launch_pdl(k_block_residual, bblocks(4 * (int64_t)n), kBThreads, 0, s, n, ptr, col, bv, f, u, r, skip);
 }
 void launch_block_restrict(int32_t nc, const int32_t *Rptr, const int32_t *Rcol, const double *Rval, const double *r,
-                           double *fc, const int *skip, cudaStream_t s) {
+                           double *fc, const double *minv, double *uc, const int *skip, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_block_restrict, bblocks(nc), kBThreads, 0, s, nc, Rptr, Rcol, Rval, r, fc, skip);
+    launch_pdl(k_block_restrict, bblocks(4 * (int64_t)nc), kBThreads, 0, s, nc, Rptr, Rcol, Rval, r, fc, minv, uc, skip);
 }
 void launch_block_prolong(int32_t n, const int32_t *Pptr, const int32_t *Pcol, const double *Pval, const double *uc,
                           double *u, const int *skip, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_block_prolong, bblocks(n), kBThreads, 0, s, n, Pptr, Pcol, Pval, uc, u, skip);
+    launch_pdl(k_block_prolong, bblocks(4 * (int64_t)n), kBThreads, 0, s, n, Pptr, Pcol, Pval, uc, u, skip);
 }
 
 }  // namespace amgpr

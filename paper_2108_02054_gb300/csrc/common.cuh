@@ -44,7 +44,7 @@ struct CgState {
 // Device-resident state of the BiCGStab iteration (same scheme as CgState).
 enum { BI_CTR_INIT = 0, BI_CTR_RHO, BI_CTR_RV, BI_CTR_SS, BI_CTR_T, BI_CTR_RR, BI_CTR_TRUE, BI_NCTR = 8 };
 struct BiState {
-    double rho, rho_old, alpha, omega, beta, rv, ts, tt, nf, res, sres, tres, tol;
+    double rho, rho_old, rho_next, alpha, omega, beta, rv, ts, tt, nf, res, sres, tres, tol;
     unsigned ctr[BI_NCTR];
     int iter, maxiter, done, status, replacements, half, need_true, copy_r, skip, pad;
 };
@@ -173,6 +173,79 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     cfg.numAttrs = 1;
     // a launch error stays the runtime's last error, read by the status check
     (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+// four consecutive doubles from a 32-byte boundary in one load
+__device__ __forceinline__ void load32(const double *p, double (&v)[4]) {
+    asm("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p));
+}
+// 4 x 4 blocks, one thread per unknown t = 4 node + r, whole quads active:
+// component r of base + Minv_node v (fma from base, component order), where
+// this lane holds component r of v and of base
+__device__ __forceinline__ double quad_minv(const double *__restrict__ minv, int64_t t, double v, double base) {
+    double m[4];
+    load32(minv + 4 * t, m);
+    const unsigned quad = 0xfu << (threadIdx.x & 28u);
+    double s = base;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) s = fma(m[c], __shfl_sync(quad, v, c, 4), s);
+    return s;
+}
+// Component r of row `node` of a 4 x 4 block matrix times x, summing in entry
+// order then component order (fma from 0): the row's odd entry first, then
+// pairs, the next pair's blocks and vector entries in flight while a pair is
+// summed.  A predicated-off FP64 instruction takes its slot of the FP64 pipe
+// like an executed one, so what a row lacks is skipped by branches (the odd
+// entry's loop count is opaque to the compiler).  VEC: x is 32-byte aligned.
+template <bool VEC>
+__device__ __forceinline__ void block_entry(const double *__restrict__ val, const double *__restrict__ x, int32_t e,
+                                            int32_t c, int r, double (&a)[4], double (&v)[4]) {
+    load32(val + (int64_t)16 * e + 4 * r, a);
+    const double *xc = x + (int64_t)4 * c;
+    if (VEC) load32(xc, v);
+    else
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = xc[q];
+}
+template <bool VEC>
+__device__ __forceinline__ double block_dot(const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
+                                            const double *__restrict__ val, const double *__restrict__ x, int32_t node,
+                                            int r) {
+    const int32_t e0 = ptr[node], e1 = ptr[node + 1];
+    int odd;
+    asm volatile("mov.u32 %0, %1;" : "=r"(odd) : "r"((e1 - e0) & 1));
+    int32_t e = e0 + ((e1 - e0) & 1);
+    double y = 0.0, a[2][4] = {}, v[2][4] = {};
+    int32_t c0 = 0, c1 = 0;
+    if (e < e1) {
+        block_entry<VEC>(val, x, e, col[e], r, a[0], v[0]);
+        block_entry<VEC>(val, x, e + 1, col[e + 1], r, a[1], v[1]);
+        if (e + 2 < e1) { c0 = col[e + 2]; c1 = col[e + 3]; }
+    }
+#pragma unroll 1
+    for (int k = 0; k < odd; ++k) {
+        double b[4], w[4];
+        block_entry<VEC>(val, x, e0, col[e0], r, b, w);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) y = fma(b[q], w[q], y);
+    }
+#pragma unroll 1
+    for (; e < e1; e += 2) {
+        double na[2][4] = {}, nv[2][4] = {};
+        if (e + 2 < e1) {
+            block_entry<VEC>(val, x, e + 2, c0, r, na[0], nv[0]);
+            block_entry<VEC>(val, x, e + 3, c1, r, na[1], nv[1]);
+        }
+        if (e + 4 < e1) { c0 = col[e + 4]; c1 = col[e + 5]; }
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                y = fma(a[k][q], v[k][q], y);
+                a[k][q] = na[k][q];
+                v[k][q] = nv[k][q];
+            }
+    }
+    return y;
 }
 void add_launches(int64_t d);
 int64_t launch_total();
@@ -330,6 +403,7 @@ struct Smooth0Out {
     double *u = nullptr;
     const float *mf = nullptr;
     float *uf = nullptr;
+    const double *minv = nullptr;  // 4 x 4 blocks: u0 = Minv r (with u)
 };
 void launch_cg_init(int32_t n, const double *f, double *u, double *r, double *partial, CgState *cg, double tol,
                     int maxiter, const Smooth0Out &z0, cudaStream_t s);
@@ -376,21 +450,22 @@ void launch_cg_update_p(int32_t n, CgState *cg, const TZ *z, double *p, double *
 // BiCGStab (FP64), right-preconditioned; partial: 3 * cg_blocks(n) doubles
 void launch_bi_init(int32_t n, const double *f, double *x, double *r, double *rh, double *p, double *v,
                     double *partial, BiState *st, double tol, int maxiter, cudaStream_t s);
-void launch_bi_rho(int32_t n, const double *rh, const double *r, double *partial, BiState *st, cudaStream_t s);
-void launch_bi_p(int32_t n, const double *r, const double *v, double *p, BiState *st, cudaStream_t s);
+// z0: the V-cycle's first pre-smoothing step from u = 0 on the finest level for
+// the vector that the kernel makes (at most one of the pointer sets is set)
+void launch_bi_p(int32_t n, const double *r, const double *v, double *p, BiState *st, const Smooth0Out &z0,
+                 cudaStream_t s);
 void launch_bi_spmv_rv(int32_t n, int bs, const FineMat &A, const double *ph, double *v, const double *rh,
                        double *partial, BiState *st, cudaStream_t s);
 void launch_bi_s(int32_t n, const double *r, const double *v, double *sv, double *partial, BiState *st,
-                 cudaStream_t s);
-void launch_bi_half(int32_t n, const double *ph, const double *sv, double *x, double *r, BiState *st, cudaStream_t s);
+                 const Smooth0Out &z0, cudaStream_t s);
 void launch_bi_spmv_t(int32_t n, int bs, const FineMat &A, const double *sh, const double *sv, double *t,
                       double *partial, BiState *st, cudaStream_t s);
-void launch_bi_xr(int32_t n, const double *ph, const double *sh, const double *sv, const double *t, double *x,
-                  double *r, double *partial, BiState *st, cudaStream_t s);
+void launch_bi_xr(int32_t n, const double *ph, const double *sh, const double *sv, const double *t, const double *rh,
+                  double *x, double *r, double *partial, BiState *st, cudaStream_t s);
 void launch_bi_true(int32_t n, int bs, const FineMat &A, const double *f, const double *x, double *t, double *partial,
                     BiState *st, int force, cudaStream_t s);
-void launch_bi_replace(int32_t n, const double *t, double *r, BiState *st, cudaStream_t s);
-void launch_bi_end(BiState *st, int use_h, cudaGraphConditionalHandle h, cudaStream_t s);
+void launch_bi_end(int32_t n, const double *t, const double *rh, double *r, double *partial, BiState *st, int use_h,
+                   cudaGraphConditionalHandle h, cudaStream_t s);
 // (BiCGStab vectors have n = bs * nodes entries; bs = 4 for the block matrix)
 
 // 4 x 4 block-valued hierarchy (block.cu): block CSR, 16 doubles per entry
@@ -409,7 +484,7 @@ void launch_block_sweep(int32_t n, const int32_t *ptr, const int32_t *col, const
 void launch_block_residual(int32_t n, const int32_t *ptr, const int32_t *col, const double *bv, const double *f,
                            const double *u, double *r, const int *skip, cudaStream_t s);
 void launch_block_restrict(int32_t nc, const int32_t *Rptr, const int32_t *Rcol, const double *Rval, const double *r,
-                           double *fc, const int *skip, cudaStream_t s);
+                           double *fc, const double *minv, double *uc, const int *skip, cudaStream_t s);
 void launch_block_prolong(int32_t n, const int32_t *Pptr, const int32_t *Pcol, const double *Pval, const double *uc,
                           double *u, const int *skip, cudaStream_t s);
 

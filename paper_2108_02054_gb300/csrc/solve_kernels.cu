@@ -1995,27 +1995,20 @@ k_cg_update_p(int32_t n, CgState *cg, const TZ *__restrict__ z, double *__restri
 // says done; scalars are formed by the last block of the producing kernel.
 
 // row policy of the 4 x 4 block matrix seen as 4 n scalar rows: node i / 4,
-// component i % 4; entry order, then component order
+// component i % 4; entry order, then component order.  VEC: x is 32-byte
+// aligned (the context's own vectors; not a caller's).
+template <bool VEC>
 struct BlockRows {
     using value = double;
     static constexpr int lanes = 1;
     const int32_t *__restrict__ ptr;
     const int32_t *__restrict__ col;
     const double *__restrict__ val;
+    const double *__restrict__ xp;
     __device__ __forceinline__ void stage(int32_t *) const {}
     template <class X>
-    __device__ __forceinline__ double dot(const int32_t *, int32_t i, int, X x) const {
-        double s = 0.0;
-        const int32_t node = i >> 2, r = i & 3;
-        for (int32_t e = ptr[node]; e < ptr[node + 1]; ++e) {
-            const double *b = val + (int64_t)16 * e + 4 * r;
-            const int32_t j = 4 * col[e];
-            s = fma(b[0], x(j), s);
-            s = fma(b[1], x(j + 1), s);
-            s = fma(b[2], x(j + 2), s);
-            s = fma(b[3], x(j + 3), s);
-        }
-        return s;
+    __device__ __forceinline__ double dot(const int32_t *, int32_t i, int, X) const {
+        return block_dot<VEC>(ptr, col, val, xp, i >> 2, i & 3);
     }
 };
 
@@ -2036,6 +2029,23 @@ __device__ bool bi_reduce2(double a, double b, double *pa, double *pb, unsigned 
         *counter = 0u;
     }
     return true;
+}
+
+// the scalar step that begins an iteration (one thread): rho = (r^, r), which
+// the kernel that made r has summed; beta = (rho / rho_old)(alpha / omega)
+__device__ void bi_begin(BiState *st) {
+    if (!st->done) {
+        st->iter += 1;
+        const double rho = st->rho_next;
+        if (!(rho != 0.0) || !isfinite(rho)) {
+            st->status = AMG_ERR_BREAKDOWN;
+            st->done = 1;
+        } else {
+            st->rho = rho;
+            st->beta = (rho / st->rho_old) * (st->alpha / st->omega);
+        }
+    }
+    st->skip = st->done;
 }
 
 // x = 0, r = r^ = f, p = v = 0; the last block initialises the state from |f|
@@ -2061,40 +2071,31 @@ __global__ void k_bi_init(int32_t n, const double *__restrict__ f, double *__res
         st->done = (st->nf == 0.0) || maxiter <= 0;
         st->status = (maxiter <= 0 && st->nf != 0.0) ? AMG_NOT_CONVERGED : AMG_OK;
         st->rho_old = st->alpha = st->omega = 1.0;
+        st->rho_next = ff;  // (r^, r) of the first iteration
         st->rho = st->beta = st->rv = st->ts = st->tt = st->res = st->sres = st->tres = 0.0;
         st->iter = st->replacements = st->half = st->need_true = st->copy_r = st->pad = 0;
-        st->skip = st->done;
+        bi_begin(st);
     }
 }
 
-// rho = (r^, r); beta = (rho / rho_old)(alpha / omega)
-__global__ void k_bi_rho(int32_t n, const double *__restrict__ rh, const double *__restrict__ r,
-                         double *__restrict__ partial, BiState *st) {
-    pdl_wait();
-    if (st->done) return;
-    double d = 0.0;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) d = fma(rh[i], r[i], d);
-    double rho = 0.0;
-    if (cg_reduce(d, partial, &st->ctr[BI_CTR_RHO], &rho) && threadIdx.x == 0) {
-        st->iter += 1;
-        if (!(rho != 0.0) || !isfinite(rho)) {
-            st->status = AMG_ERR_BREAKDOWN;
-            st->done = st->skip = 1;
-        } else {
-            st->rho = rho;
-            st->beta = (rho / st->rho_old) * (st->alpha / st->omega);
-        }
-    }
+// the V-cycle's first smoothing step for a BiCGStab vector (whole quads of a
+// block system take part together: n is a multiple of 4 and quads never split)
+__device__ __forceinline__ void bi_smooth0(const Smooth0Out &z0, int32_t i, double v) {
+    if (z0.minv) z0.u[i] = quad_minv(z0.minv, i, v, 0.0);
+    else put_smooth0(z0, i, v);
 }
 
-// p = r + beta (p - omega v)
+// p = r + beta (p - omega v), and the first smoothing step for it
 __global__ void k_bi_p(int32_t n, const double *__restrict__ r, const double *__restrict__ v, double *__restrict__ p,
-                       const BiState *st) {
+                       const BiState *st, Smooth0Out z0) {
     pdl_wait();
     if (st->done) return;
     const double beta = st->beta, omega = st->omega;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        p[i] = fma(beta, fma(-omega, v[i], p[i]), r[i]);
+    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const double pi = fma(beta, fma(-omega, v[i], p[i]), r[i]);
+        p[i] = pi;
+        bi_smooth0(z0, i, pi);
+    }
 }
 
 // v = A p^, (r^, v); alpha = rho / (r^, v)
@@ -2125,9 +2126,10 @@ k_bi_spmv_rv(int32_t n, M A, const double *__restrict__ ph, double *__restrict__
     }
 }
 
-// s = r - alpha v and |s|: converged at the half step when |s|/|f| <= tol
+// s = r - alpha v (and the first smoothing step for it) and |s|: converged at
+// the half step when |s|/|f| <= tol
 __global__ void k_bi_s(int32_t n, const double *__restrict__ r, const double *__restrict__ v, double *__restrict__ sv,
-                       double *__restrict__ partial, BiState *st) {
+                       double *__restrict__ partial, BiState *st, Smooth0Out z0) {
     pdl_wait();
     if (st->done) return;
     const double alpha = st->alpha;
@@ -2135,6 +2137,7 @@ __global__ void k_bi_s(int32_t n, const double *__restrict__ r, const double *__
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const double si = fma(-alpha, v[i], r[i]);
         sv[i] = si;
+        bi_smooth0(z0, i, si);
         d = fma(si, si, d);
     }
     double ss = 0.0;
@@ -2143,18 +2146,6 @@ __global__ void k_bi_s(int32_t n, const double *__restrict__ r, const double *__
         st->half = st->sres <= st->tol;
         st->need_true = st->half;
         st->skip = st->half;
-    }
-}
-
-// half step: x += alpha p^, r = s
-__global__ void k_bi_half(int32_t n, const double *__restrict__ ph, const double *__restrict__ sv,
-                          double *__restrict__ x, double *__restrict__ r, const BiState *st) {
-    pdl_wait();
-    if (st->done || !st->half) return;
-    const double alpha = st->alpha;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        x[i] = fma(alpha, ph[i], x[i]);
-        r[i] = sv[i];
     }
 }
 
@@ -2189,24 +2180,35 @@ k_bi_spmv_t(int32_t n, M A, const double *__restrict__ sh, const double *__restr
     }
 }
 
-// x += alpha p^ + omega s^, r = s - omega t, |r|
+// x += alpha p^ + omega s^, r = s - omega t, |r| and the next (r^, r); after a
+// half step instead x += alpha p^, r = s (the true residual decides then)
 __global__ void k_bi_xr(int32_t n, const double *__restrict__ ph, const double *__restrict__ sh,
-                        const double *__restrict__ sv, const double *__restrict__ t, double *__restrict__ x,
-                        double *__restrict__ r, double *__restrict__ partial, BiState *st) {
+                        const double *__restrict__ sv, const double *__restrict__ t, const double *__restrict__ rh,
+                        double *__restrict__ x, double *__restrict__ r, double *__restrict__ partial, BiState *st) {
     pdl_wait();
-    if (st->skip) return;
+    if (st->done) return;
     const double alpha = st->alpha, omega = st->omega;
-    double d = 0.0;
+    if (st->half) {
+        for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+            x[i] = fma(alpha, ph[i], x[i]);
+            r[i] = sv[i];
+        }
+        return;
+    }
+    double d = 0.0, dh = 0.0;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        x[i] = fma(omega, sh[i], fma(alpha, ph[i], x[i]));
-        const double ri = fma(-omega, t[i], sv[i]);
+        const double xi = x[i], phi = ph[i], shi = sh[i], si = sv[i], ti = t[i], rhi = rh[i];
+        const double ri = fma(-omega, ti, si);
+        x[i] = fma(omega, shi, fma(alpha, phi, xi));
         r[i] = ri;
         d = fma(ri, ri, d);
+        dh = fma(rhi, ri, dh);
     }
-    double rr = 0.0;
-    if (cg_reduce(d, partial, &st->ctr[BI_CTR_RR], &rr) && threadIdx.x == 0) {
+    double rr = 0.0, rho = 0.0;
+    if (bi_reduce2(d, dh, partial, partial + gridDim.x, &st->ctr[BI_CTR_RR], &rr, &rho) && threadIdx.x == 0) {
         st->res = sqrt(rr) / st->nf;
         st->need_true = st->res <= st->tol;
+        st->rho_next = rho;
     }
 }
 
@@ -2246,18 +2248,29 @@ k_bi_true(int32_t n, M A, const double *__restrict__ f, const double *__restrict
     }
 }
 
-__global__ void k_bi_replace(int32_t n, const double *__restrict__ t, double *__restrict__ r, const BiState *st) {
+// end of an iteration: r = t where the true residual replaces it (and its
+// (r^, r)); count it, clear the per-iteration flags, stop at maxiter (and, in
+// the graph, keep the while loop going; hard cap maxiter + 4 bodies), and take
+// the scalar step that begins the next one
+__global__ void k_bi_end(int32_t n, const double *__restrict__ t, const double *__restrict__ rh,
+                         double *__restrict__ r, double *__restrict__ partial, BiState *st, int use_h,
+                         cudaGraphConditionalHandle h) {
     pdl_wait();
-    if (st->done || !st->copy_r) return;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) r[i] = t[i];
-}
-
-// end of an iteration: count it, clear the per-iteration flags, stop at
-// maxiter (and, in the graph, keep the while loop going; hard cap maxiter + 4
-// bodies)
-__global__ void k_bi_end(BiState *st, int use_h, cudaGraphConditionalHandle h) {
-    pdl_wait();
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    // only a replacement has work for the other blocks (the flag is not
+    // cleared before every block has read it)
+    if (!st->done && st->copy_r) {
+        double d = 0.0;
+        for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+            const double ti = t[i];
+            r[i] = ti;
+            d = fma(rh[i], ti, d);
+        }
+        double rho = 0.0;
+        if (!cg_reduce(d, partial, &st->ctr[BI_CTR_RHO], &rho) || threadIdx.x != 0) return;
+        st->rho_next = rho;
+    } else if (blockIdx.x != 0 || threadIdx.x != 0) {
+        return;
+    }
     st->pad += 1;  // bodies run (the graph's launch count)
     if (!st->done) {
         if (st->iter >= st->maxiter || st->pad > st->maxiter + 4) {
@@ -2266,7 +2279,7 @@ __global__ void k_bi_end(BiState *st, int use_h, cudaGraphConditionalHandle h) {
         }
     }
     st->half = st->need_true = st->copy_r = 0;
-    st->skip = st->done;
+    bi_begin(st);
     if (use_h) cudaGraphSetConditional(h, st->done ? 0u : 1u);
 }
 
@@ -2684,13 +2697,10 @@ void launch_bi_init(int32_t n, const double *f, double *x, double *r, double *rh
     count_launch();
     launch_pdl(k_bi_init, cg_blocks(n), kCgThreads, 0, s, n, f, x, r, rh, p, v, partial, st, tol, maxiter);
 }
-void launch_bi_rho(int32_t n, const double *rh, const double *r, double *partial, BiState *st, cudaStream_t s) {
+void launch_bi_p(int32_t n, const double *r, const double *v, double *p, BiState *st, const Smooth0Out &z0,
+                 cudaStream_t s) {
     count_launch();
-    launch_pdl(k_bi_rho, cg_blocks(n), kCgThreads, 0, s, n, rh, r, partial, st);
-}
-void launch_bi_p(int32_t n, const double *r, const double *v, double *p, BiState *st, cudaStream_t s) {
-    count_launch();
-    launch_pdl(k_bi_p, cg_blocks(n), kCgThreads, 0, s, n, r, v, p, st);
+    launch_pdl(k_bi_p, cg_blocks(n), kCgThreads, 0, s, n, r, v, p, st, z0);
 }
 void launch_bi_spmv_rv(int32_t n, int bs, const FineMat &A, const double *ph, double *v, const double *rh,
                        double *partial, BiState *st, cudaStream_t s) {
@@ -2698,17 +2708,13 @@ void launch_bi_spmv_rv(int32_t n, int bs, const FineMat &A, const double *ph, do
     const auto run = [&](auto M) {
         launch_pdl(k_bi_spmv_rv<decltype(M)>, cg_blocks(n), kCgThreads, 0, s, n, M, ph, v, rh, partial, st);
     };
-    if (bs == 4) run(BlockRows{A.ptr, A.col.col, A.val});
+    if (bs == 4) run(BlockRows<true>{A.ptr, A.col.col, A.val, ph});
     else with_fine_rows(A, n, run);
 }
 void launch_bi_s(int32_t n, const double *r, const double *v, double *sv, double *partial, BiState *st,
-                 cudaStream_t s) {
+                 const Smooth0Out &z0, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_bi_s, cg_blocks(n), kCgThreads, 0, s, n, r, v, sv, partial, st);
-}
-void launch_bi_half(int32_t n, const double *ph, const double *sv, double *x, double *r, BiState *st, cudaStream_t s) {
-    count_launch();
-    launch_pdl(k_bi_half, cg_blocks(n), kCgThreads, 0, s, n, ph, sv, x, r, st);
+    launch_pdl(k_bi_s, cg_blocks(n), kCgThreads, 0, s, n, r, v, sv, partial, st, z0);
 }
 void launch_bi_spmv_t(int32_t n, int bs, const FineMat &A, const double *sh, const double *sv, double *t,
                       double *partial, BiState *st, cudaStream_t s) {
@@ -2716,13 +2722,13 @@ void launch_bi_spmv_t(int32_t n, int bs, const FineMat &A, const double *sh, con
     const auto run = [&](auto M) {
         launch_pdl(k_bi_spmv_t<decltype(M)>, cg_blocks(n), kCgThreads, 0, s, n, M, sh, sv, t, partial, st);
     };
-    if (bs == 4) run(BlockRows{A.ptr, A.col.col, A.val});
+    if (bs == 4) run(BlockRows<true>{A.ptr, A.col.col, A.val, sh});
     else with_fine_rows(A, n, run);
 }
-void launch_bi_xr(int32_t n, const double *ph, const double *sh, const double *sv, const double *t, double *x,
-                  double *r, double *partial, BiState *st, cudaStream_t s) {
+void launch_bi_xr(int32_t n, const double *ph, const double *sh, const double *sv, const double *t, const double *rh,
+                  double *x, double *r, double *partial, BiState *st, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_bi_xr, cg_blocks(n), kCgThreads, 0, s, n, ph, sh, sv, t, x, r, partial, st);
+    launch_pdl(k_bi_xr, cg_blocks(n), kCgThreads, 0, s, n, ph, sh, sv, t, rh, x, r, partial, st);
 }
 void launch_bi_true(int32_t n, int bs, const FineMat &A, const double *f, const double *x, double *t, double *partial,
                     BiState *st, int force, cudaStream_t s) {
@@ -2730,16 +2736,13 @@ void launch_bi_true(int32_t n, int bs, const FineMat &A, const double *f, const 
     const auto run = [&](auto M) {
         launch_pdl(k_bi_true<decltype(M)>, cg_blocks(n), kCgThreads, 0, s, n, M, f, x, t, partial, st, force);
     };
-    if (bs == 4) run(BlockRows{A.ptr, A.col.col, A.val});
+    if (bs == 4) run(BlockRows<false>{A.ptr, A.col.col, A.val, x});
     else with_fine_rows(A, n, run);
 }
-void launch_bi_replace(int32_t n, const double *t, double *r, BiState *st, cudaStream_t s) {
+void launch_bi_end(int32_t n, const double *t, const double *rh, double *r, double *partial, BiState *st, int use_h,
+                   cudaGraphConditionalHandle h, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_bi_replace, cg_blocks(n), kCgThreads, 0, s, n, t, r, st);
-}
-void launch_bi_end(BiState *st, int use_h, cudaGraphConditionalHandle h, cudaStream_t s) {
-    count_launch();
-    launch_pdl(k_bi_end, 1, 32, 0, s, st, use_h, h);
+    launch_pdl(k_bi_end, cg_blocks(n), kCgThreads, 0, s, n, t, rh, r, partial, st, use_h, h);
 }
 
 }  // namespace amgpr
