@@ -714,12 +714,26 @@ k_dense_lu_cluster(int32_t n, double *__restrict__ g, double *__restrict__ gT, i
 // Every wait is bounded by a clock budget; on expiry the CTA sets
 // DEV_ERR_TIMEOUT, waits no more and goes to the final cluster barrier, which
 // every CTA then reaches.
-constexpr int kLuPipeN = 128;
+//
+// Message rows are kept in a ring of R > C B slots.  When step k is sent, every
+// other CTA has begun its latest block, at most C - 1 blocks back, since the
+// owner of k waited for that block's steps; it has then consumed and applied
+// every step before that block but the last, all of them in the CTA's program
+// order, and every CTA has received them (each consumed them before a block of
+// its own that step k waited for).  So slot k % R, last used by step k - R,
+// is free: k - R < b_q B - 1 for every b_q >= k / B - C + 1.
+constexpr int kLuPipeN = 256;
 constexpr int kLuPipeMinN = 48;  // below: the one-CTA kernel is faster (fewer steps to pipeline)
-constexpr int kLuPipeWarps = 4;                           // compute warps, one row per lane
-constexpr int kLuPipeThreads = (kLuPipeWarps + 1) * 32;   // and the sender warp
-constexpr int kLuPipeC = 8;                               // CTAs of the cluster
-constexpr int kLuPipeB = 4;                               // columns per ownership block
+constexpr int kLuPipeB = 4;      // columns per ownership block
+// CTAs and warps: eight CTAs at every size; eight compute warps for 128 < n <=
+// 256.  n = 153 / 212 / 255: 226 / 332 / 430 us (sixteen CTAs, a non-portable
+// cluster: 235 / 324 / 393), where the one-CTA kernel took 569 at 153 and the
+// row-cyclic cluster kernel 722 / 876; n = 87 with four warps 103.  The owner's
+// step (about 2,000 cycles) bounds it, and at 255 the trailing updates too.
+constexpr int kLuPipeWideC = 8;
+// W compute warps, one row per lane (and the sender warp); C CTAs
+__host__ __device__ constexpr int lu_pipe_threads(int W) { return (W + 1) * 32; }
+__host__ __device__ constexpr int lu_pipe_ring(int C, int B) { return C * B + 8; }
 constexpr long long kLuPipeWaitClocks = 2000000000ll;
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -762,13 +776,15 @@ __device__ __forceinline__ void bulk_to_peer(uint32_t dst, uint32_t src, uint32_
                  : "memory");
 }
 // barrier of the compute warps only (named barrier 1)
-__device__ __forceinline__ void lu_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kLuPipeWarps * 32) : "memory"); }
+template <int W>
+__device__ __forceinline__ void lu_sync() { asm volatile("bar.sync 1, %0;" ::"n"(W * 32) : "memory"); }
+template <int W>
 __device__ __forceinline__ int lu_sync_or(int pred) {
     int r;
     asm volatile(
         "{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.s32 %0, 1, 0, q;\n}\n"
         : "=r"(r)
-        : "r"(pred), "n"(kLuPipeWarps * 32)
+        : "r"(pred), "n"(W * 32)
         : "memory");
     return r;
 }
@@ -800,20 +816,21 @@ struct LuPipeMap {
     __device__ int32_t ncols(int32_t q) const { return q < nblk ? local(last_col(q)) + 1 : 0; }
 };
 
-// shared memory: n_even mbarriers, n - 1 message rows of lu_pipe_row(n)
+// shared memory: n_even mbarriers, the ring of message rows of lu_pipe_row(n)
 // doubles (multipliers, then the header at n_even), the own columns
 __host__ __device__ inline int32_t lu_pipe_even(int32_t n) { return (n + 1) & ~1; }
 __host__ __device__ inline int32_t lu_pipe_row(int32_t n) { return lu_pipe_even(n) + 2; }
 size_t lu_pipe_smem(int32_t n, int C, int B) {
     const size_t nblk = (size_t)(n + B - 1) / B, per = (nblk + C - 1) / C * B;
-    return ((size_t)lu_pipe_even(n) + (size_t)(n > 0 ? n - 1 : 0) * lu_pipe_row(n) + per * n) * 8;
+    return ((size_t)lu_pipe_even(n) + (size_t)lu_pipe_ring(C, B) * lu_pipe_row(n) + per * n) * 8;
 }
 
-template <int C, int B>
-__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kLuPipeThreads)
+template <int C, int B, int W>
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(lu_pipe_threads(W))
 k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int32_t *__restrict__ piv, int *st) {
+    constexpr int R = lu_pipe_ring(C, B);
     extern __shared__ __align__(16) unsigned long long sm_pipe[];
-    __shared__ PivCand<B> cand_buf[2][kLuPipeWarps];  // by step parity: a fast warp may write step k+1's
+    __shared__ PivCand<B> cand_buf[2][W];  // by step parity: a fast warp may write step k+1's
     __shared__ int s_quit;
     cgr::cluster_group cluster = cgr::this_cluster();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -821,26 +838,27 @@ k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int3
     const LuPipeMap<C, B> M{n, (n + B - 1) / B};
     const int32_t nmine = M.ncols(rank), ne = lu_pipe_even(n), row = lu_pipe_row(n);
     unsigned long long *bar = sm_pipe;                       // one mbarrier per step
-    double *msg = (double *)(sm_pipe + ne);                  // message rows, [step][row]
-    double *col = msg + (size_t)(n > 0 ? n - 1 : 0) * row;   // own columns, [local column][row]
+    double *msg = (double *)(sm_pipe + ne);                  // message rows, [step % R][row]
+    double *col = msg + (size_t)R * row;                     // own columns, [local column][row]
+    auto slot = [&](int32_t s) { return msg + (size_t)(s % R) * row; };
     const uint32_t off_msg = 8u * (uint32_t)ne, row_bytes = 8u * (uint32_t)row;
 
     // setup: barriers (own steps: the compute warps arrive; others: one
     // arrival with the message's byte count), the own columns
-    for (int32_t s = tid; s < n; s += kLuPipeThreads)
-        mbar_init(smem_addr(bar + s), M.owner(s) == rank ? (uint32_t)kLuPipeWarps : 1u);
+    for (int32_t s = tid; s < n; s += lu_pipe_threads(W))
+        mbar_init(smem_addr(bar + s), M.owner(s) == rank ? (uint32_t)W : 1u);
     if (tid == 0) s_quit = 0;
     __syncthreads();
     if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    for (int32_t s = tid; s < n - 1; s += kLuPipeThreads)
+    for (int32_t s = tid; s < n - 1; s += lu_pipe_threads(W))
         if (M.owner(s) != rank) mbar_arrive_expect(smem_addr(bar + s), row_bytes);
-    for (int32_t e = tid; e < nmine * n; e += kLuPipeThreads) {
+    for (int32_t e = tid; e < nmine * n; e += lu_pipe_threads(W)) {
         const int32_t lc = e / n, r = e % n;
         col[e] = g[(int64_t)r * n + M.global(rank, lc)];
     }
     cluster.sync();
 
-    if (warp == kLuPipeWarps) {
+    if (warp == W) {
         // the sender: each own step's message row to every other CTA
         const uint32_t base = smem_addr(sm_pipe);
         bool stop = false;
@@ -869,11 +887,11 @@ k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int3
                     for (int q = 0; q < C; ++q)
                         if (q != rank) {
                             const uint32_t pb = peer_addr(base, (uint32_t)q);
-                            bulk_to_peer(pb + off_msg + row_bytes * (uint32_t)k, smem_addr(msg + (size_t)k * row),
+                            bulk_to_peer(pb + off_msg + row_bytes * (uint32_t)(k % R), smem_addr(slot(k)),
                                          row_bytes, pb + 8u * (uint32_t)k);
                         }
                 }
-                const unsigned long long h = (unsigned long long)__double_as_longlong(msg[(size_t)k * row + ne]);
+                const unsigned long long h = (unsigned long long)__double_as_longlong(slot(k)[ne]);
                 if ((h >> 32) & 1ull) stop = true;
             }
     } else {
@@ -886,12 +904,12 @@ k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int3
         // read the header of a received step: wait, then update the row bookkeeping
         auto consume = [&](int32_t s) -> bool {
             const int late = mbar_wait(smem_addr(bar + s)) ? 0 : 1;
-            if (lu_sync_or(late)) {
+            if (lu_sync_or<W>(late)) {
                 if (tid == 0) atomicOr(st, DEV_ERR_TIMEOUT);
                 abort = true;
                 return false;
             }
-            const unsigned long long h = (unsigned long long)__double_as_longlong(msg[(size_t)s * row + ne]);
+            const unsigned long long h = (unsigned long long)__double_as_longlong(slot(s)[ne]);
             if ((h >> 32) & 1ull) {
                 kstop = s;
                 return false;
@@ -906,7 +924,7 @@ k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int3
             if (lo >= hi) return;
             const bool act = valid && pstep > s;
             if (!__any_sync(0xffffffffu, act)) return;
-            const double *m = msg + (size_t)s * row;
+            const double *m = slot(s);
             const int32_t pr = (int32_t)(((unsigned long long)__double_as_longlong(m[ne]) >> 16) & 0xffffu);
             const double l = act ? m[r] : 0.0;
             int32_t lc = lo;
@@ -950,7 +968,7 @@ k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int3
 #pragma unroll
             for (int t = 0; t < B; ++t) vb[t] = valid && t < nb ? col[(size_t)(lb + t) * n + r] : 0.0;
             if (have_last) {
-                const double *m = msg + (size_t)(k0 - 1) * row;
+                const double *m = slot(k0 - 1);
                 const int32_t pr = (int32_t)(((unsigned long long)__double_as_longlong(m[ne]) >> 16) & 0xffffu);
                 const bool act = valid && pstep > k0 - 1;
                 const double l = act ? m[r] : 0.0;
@@ -993,13 +1011,13 @@ k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int3
                     for (int q = 0; q < B; ++q) c.vals[q] = vb[q];
                     c.rc = rc;
                 }
-                lu_sync();
+                lu_sync<W>();
                 int bw = 0;
                 {
                     unsigned long long bk_ = cand[0].key;
                     int32_t bpos = cand[0].pos;
 #pragma unroll
-                    for (int w = 1; w < kLuPipeWarps; ++w) {
+                    for (int w = 1; w < W; ++w) {
                         const unsigned long long kw = cand[w].key;
                         const int32_t pw = cand[w].pos;
                         if (kw > bk_ || (kw == bk_ && pw < bpos)) { bk_ = kw; bpos = pw; bw = w; }
@@ -1008,7 +1026,7 @@ k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int3
                 const PivCand<B> &best = cand[bw];
                 const int32_t brow = best.row, bpos = best.pos;
                 const bool sing = best.key == 0ull || brow < 0;
-                double *m = msg + (size_t)k * row;
+                double *m = slot(k);
                 if (sing) {
                     // the receivers see the flag in the header; no multipliers
                     // follow (the last step has no message row)
@@ -1068,10 +1086,10 @@ k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int3
                 for (int t = 0; t < B; ++t)
                     if (t < nb) col[(size_t)(lb + t) * n + r] = vb[t];
             const int32_t kend = kstop != n ? kstop : k1;
-            lu_sync();
+            lu_sync<W>();
             for (int32_t s = deferred ? k0 - 1 : k0; s < kend; ++s) {
                 apply(s, lb1, nmine);
-                lu_sync();
+                lu_sync<W>();
             }
             s_all = k1;
         }
@@ -1087,7 +1105,7 @@ k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int3
                 if (gT) gT[(int64_t)j * n + pos] = v;
             }
         // every arrival is made: let the sender stop waiting
-        lu_sync();
+        lu_sync<W>();
         if (tid == 0) {
             __threadfence_block();
             *(volatile int *)&s_quit = 1;
@@ -1268,25 +1286,22 @@ k_lu_inverse_rows(int32_t n, const double *__restrict__ lu_g, const int32_t *__r
     if (valid) inv[(int64_t)r * n + j] = x;
 }
 
-// explicit inverse from column-major factors (n > kLuSmemN): the factors stay
-// in global memory (L2) and every step's loads are contiguous across lanes;
-// the pivots, the reciprocals of U's diagonal and each warp's column live in
-// shared memory
-__global__ void __launch_bounds__(kInvWarps * 32)
+// explicit inverse from column-major factors (kLuSmemN < n <= kLuClusterN): one
+// block per column of A^-1 with one row per thread, as k_lu_inverse_rows, the
+// factors read from L2 (contiguous across the threads) a batch of steps ahead,
+// since no factor depends on a step.  n = 212 / 255: 84 / 111 us (one warp per
+// column: 267 / 364); a step is one barrier and one fma over all warps.
+constexpr int kInvAhead = 8;
+__global__ void __launch_bounds__((kLuClusterN + 31) / 32 * 32)
 k_lu_inverse_t(int32_t n, const double *__restrict__ luT, const int32_t *__restrict__ piv, double *__restrict__ inv) {
-    extern __shared__ double sm_it[];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    double *xs = sm_it;                                   // kInvWarps columns
-    double *rd = xs + (int64_t)kInvWarps * n;             // 1 / u_kk
-    int32_t *pv = (int32_t *)(rd + n);
-    for (int32_t e = threadIdx.x; e < n; e += blockDim.x) {
-        rd[e] = 1.0 / luT[(int64_t)e * n + e];
-        pv[e] = piv[e];
-    }
+    __shared__ double xs[kLuClusterN];     // x_k as each step finalises it
+    __shared__ int32_t pv[kLuClusterN];
+    const int32_t j = blockIdx.x, r = threadIdx.x;
+    const bool valid = r < n;
+    if (valid) pv[r] = piv[r];
+    const double rd = valid ? 1.0 / luT[(int64_t)r * n + r] : 0.0;
+    const int32_t rc = valid ? r : 0;
     __syncthreads();
-    const int32_t j = blockIdx.x * kInvWarps + w;
-    if (j >= n) return;  // warp-uniform; no block barrier follows
-    double *x = xs + (int64_t)w * n;
     int32_t pos = j;
     for (int32_t k = 0; k < n; ++k) {
         const int32_t p = pv[k];
@@ -1294,23 +1309,49 @@ k_lu_inverse_t(int32_t n, const double *__restrict__ luT, const int32_t *__restr
         if (pos == k) pos = p;
         else if (pos == p) pos = k;
     }
-    for (int32_t r = lane; r < n; r += 32) x[r] = (r == pos) ? 1.0 : 0.0;
-    __syncwarp();
-    for (int32_t k = pos; k < n - 1; ++k) {
-        const double xk = x[k];
-        const double *colk = luT + (int64_t)k * n;
-        for (int32_t r = k + 1 + lane; r < n; r += 32) x[r] = fma(-colk[r], xk, x[r]);
-        __syncwarp();
+    double x = valid && r == pos ? 1.0 : 0.0;
+    // L y = P e_j (unit lower triangular); entries before pos stay zero
+    double l[kInvAhead];
+#pragma unroll
+    for (int q = 0; q < kInvAhead; ++q) l[q] = luT[(int64_t)min(pos + q, n - 1) * n + rc];
+    for (int32_t k0 = pos; k0 < n - 1; k0 += kInvAhead) {
+        double nl[kInvAhead];
+#pragma unroll
+        for (int q = 0; q < kInvAhead; ++q) nl[q] = luT[(int64_t)min(k0 + kInvAhead + q, n - 1) * n + rc];
+#pragma unroll
+        for (int q = 0; q < kInvAhead; ++q) {
+            const int32_t k = k0 + q;
+            if (k >= n - 1) break;  // block-uniform
+            if (r == k) xs[k] = x;
+            __syncthreads();
+            if (valid && r > k) x = fma(-l[q], xs[k], x);
+        }
+#pragma unroll
+        for (int q = 0; q < kInvAhead; ++q) l[q] = nl[q];
     }
-    for (int32_t k = n - 1; k >= 0; --k) {
-        if (lane == 0) x[k] = x[k] * rd[k];
-        __syncwarp();
-        const double xk = x[k];
-        const double *colk = luT + (int64_t)k * n;
-        for (int32_t r = lane; r < k; r += 32) x[r] = fma(-colk[r], xk, x[r]);
-        __syncwarp();
+    // U x = y
+#pragma unroll
+    for (int q = 0; q < kInvAhead; ++q) l[q] = luT[(int64_t)max(n - 1 - q, 0) * n + rc];
+    __syncthreads();
+    for (int32_t k0 = n - 1; k0 >= 0; k0 -= kInvAhead) {
+        double nl[kInvAhead];
+#pragma unroll
+        for (int q = 0; q < kInvAhead; ++q) nl[q] = luT[(int64_t)max(k0 - kInvAhead - q, 0) * n + rc];
+#pragma unroll
+        for (int q = 0; q < kInvAhead; ++q) {
+            const int32_t k = k0 - q;
+            if (k < 0) break;  // block-uniform
+            if (r == k) {
+                x = x * rd;
+                xs[k] = x;
+            }
+            __syncthreads();
+            if (valid && r < k) x = fma(-l[q], xs[k], x);
+        }
+#pragma unroll
+        for (int q = 0; q < kInvAhead; ++q) l[q] = nl[q];
     }
-    for (int32_t r = lane; r < n; r += 32) inv[(int64_t)r * n + j] = x[r];
+    if (valid) inv[(int64_t)r * n + j] = x;
 }
 
 // ---- two-byte column offsets (built once per pattern)
@@ -2389,23 +2430,25 @@ void launch_dense_lu(int32_t n, double *a, int32_t *piv, int *st, cudaStream_t s
     static bool attr = false;
     const int max_bytes = kLuSmemN * kLuSmemN * (int)sizeof(double);
     if (!attr) {
-        cudaFuncSetAttribute(k_dense_lu_pipe<kLuPipeC, kLuPipeB>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_pipe_smem(kLuPipeN, kLuPipeC, kLuPipeB));
-        if (kLuPipeC > 8)
-            cudaFuncSetAttribute(k_dense_lu_pipe<kLuPipeC, kLuPipeB>,
+        cudaFuncSetAttribute(k_dense_lu_pipe<8, kLuPipeB, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)lu_pipe_smem(128, 8, kLuPipeB));
+        cudaFuncSetAttribute(k_dense_lu_pipe<kLuPipeWideC, kLuPipeB, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)lu_pipe_smem(kLuPipeN, kLuPipeWideC, kLuPipeB));
+        if (kLuPipeWideC > 8)
+            cudaFuncSetAttribute(k_dense_lu_pipe<kLuPipeWideC, kLuPipeB, 8>,
                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cudaFuncSetAttribute(k_dense_lu_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
         cudaFuncSetAttribute(k_dense_lu_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)lu_cluster_smem(kLuClusterN));
-        cudaFuncSetAttribute(k_lu_inverse_t, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(((size_t)(kInvWarps + 1) * kLuClusterN) * sizeof(double) +
-                                   (size_t)kLuClusterN * sizeof(int32_t)));
         attr = true;
     }
     count_launch();
-    if (n > kLuPipeMinN && n <= kLuPipeN)
-        k_dense_lu_pipe<kLuPipeC, kLuPipeB>
-            <<<kLuPipeC, kLuPipeThreads, lu_pipe_smem(n, kLuPipeC, kLuPipeB), s>>>(n, a, aT, piv, st);
+    if (n > kLuPipeMinN && n <= 128)
+        k_dense_lu_pipe<8, kLuPipeB, 4>
+            <<<8, lu_pipe_threads(4), lu_pipe_smem(n, 8, kLuPipeB), s>>>(n, a, aT, piv, st);
+    else if (n > 128 && n <= kLuPipeN)
+        k_dense_lu_pipe<kLuPipeWideC, kLuPipeB, 8>
+            <<<kLuPipeWideC, lu_pipe_threads(8), lu_pipe_smem(n, kLuPipeWideC, kLuPipeB), s>>>(n, a, aT, piv, st);
     else if (n <= kLuSmemN)
         k_dense_lu_smem<<<1, kLuThreads, (size_t)n * n * sizeof(double), s>>>(n, a, piv, st);
     else if (n <= kLuClusterN)
@@ -2417,8 +2460,7 @@ void launch_lu_inverse(int32_t n, const double *lu, const int32_t *piv, double *
                        const double *luT) {
     if (luT && n > kLuSmemN && n <= kLuClusterN) {
         count_launch();
-        const size_t bytes = ((size_t)(kInvWarps + 1) * n) * sizeof(double) + (size_t)n * sizeof(int32_t);
-        k_lu_inverse_t<<<(unsigned)((n + kInvWarps - 1) / kInvWarps), kInvWarps * 32, bytes, s>>>(n, luT, piv, inv);
+        k_lu_inverse_t<<<(unsigned)n, (unsigned)((n + 31) / 32 * 32), 0, s>>>(n, luT, piv, inv);
         return;
     }
     static bool attr = false;
