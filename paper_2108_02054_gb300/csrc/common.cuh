@@ -442,10 +442,10 @@ void launch_true_residual(int32_t n, const FineMat &A, const double *f, const do
                           CgState *cg, int force, cudaStream_t s);
 template <class TZ>
 void launch_replace_r(int32_t n, CgState *cg, const double *t, double *r, const TZ *zo, double *part_zo,
-                      const Smooth0Out &z0, cudaStream_t s);
+                      const Smooth0Out &z0, int use_h, cudaGraphConditionalHandle h_in,
+                      cudaGraphConditionalHandle h_out, cudaStream_t s);
 template <class TZ>
-void launch_cg_update_p(int32_t n, CgState *cg, const TZ *z, double *p, double *u, int use_h,
-                        cudaGraphConditionalHandle h, cudaStream_t s);
+void launch_cg_update_p(int32_t n, CgState *cg, const TZ *z, double *p, double *u, cudaStream_t s);
 
 // BiCGStab (FP64), right-preconditioned; partial: 3 * cg_blocks(n) doubles
 void launch_bi_init(int32_t n, const double *f, double *x, double *r, double *rh, double *p, double *v,

@@ -1860,8 +1860,7 @@ k_spmv_dot(int32_t n, M A, const double *__restrict__ p, double *__restrict__ q,
 }
 
 // r -= alpha q, u0 = m o r; the last block checks the recurrence residual
-// (graph: opens the IF branch hb of the true-residual check when it meets tol,
-// or when maxiter ends the iteration).  u += alpha p is left to the p update,
+// (graph: the inner loop hb goes on unless it meets tol or maxiter ends it).  u += alpha p is left to the p update,
 // which reads p anyway; where the iteration ends, to k_cg_update_u in the
 // branch (cg->u_done then tells the p update).  With zo (the flexible variant),
 // also r_new.z_old into cg->rzo.
@@ -1915,7 +1914,7 @@ k_cg_update_r(int32_t n, CgState *cg, const double *__restrict__ q, double *__re
             cg->status = AMG_NOT_CONVERGED;
         }
         cg->u_done = cg->need_true || cg->done;
-        if (use_h) cudaGraphSetConditional(hb, cg->u_done ? 1u : 0u);
+        if (use_h) cudaGraphSetConditional(hb, cg->u_done ? 0u : 1u);
     }
 }
 
@@ -1968,8 +1967,14 @@ k_true_residual(int32_t n, M A, const double *__restrict__ f, const double *__re
 // flexible variant), r_new.z_old is formed again from the new r
 template <class TZ>
 __global__ void k_replace_r(int32_t n, CgState *cg, const double *__restrict__ t, double *__restrict__ r,
-                            const TZ *__restrict__ zo, double *__restrict__ part_zo, Smooth0Out z0) {
+                            const TZ *__restrict__ zo, double *__restrict__ part_zo, Smooth0Out z0, int use_h,
+                            cudaGraphConditionalHandle h_in, cudaGraphConditionalHandle h_out) {
     pdl_wait();
+    if (use_h && blockIdx.x == 0 && threadIdx.x == 0) {
+        // both loops go on while the solve is not done
+        cudaGraphSetConditional(h_in, cg->done ? 0u : 1u);
+        cudaGraphSetConditional(h_out, cg->done ? 0u : 1u);
+    }
     if (cg->done || !cg->copy_r) return;
     double so = 0.0;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -1984,20 +1989,15 @@ __global__ void k_replace_r(int32_t n, CgState *cg, const double *__restrict__ t
 }
 
 // beta = (r.z_new - r.z_old) / (r.z)_old, the flexible form (r.z_old = 0 for
-// standard CG), u += alpha p (unless u_done), p = z + beta p.  The new r.z becomes current in the next
-// iteration's first kernel.  In the graph this is the body's last kernel: it
-// keeps the while loop going while the iteration is not done, with a hard
-// cap of maxiter + 4 bodies.
+// standard CG), u += alpha p (unless u_done), p = z + beta p.  The new r.z becomes
+// current in the next iteration's first kernel.  At most maxiter + 4 of these
+// run.
 template <class TZ>
 __global__ void __launch_bounds__(kCgThreads, 4)
-k_cg_update_p(int32_t n, CgState *cg, const TZ *__restrict__ z, double *__restrict__ p, double *__restrict__ u,
-              int use_h, cudaGraphConditionalHandle h) {
+k_cg_update_p(int32_t n, CgState *cg, const TZ *__restrict__ z, double *__restrict__ p, double *__restrict__ u) {
     pdl_wait();
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
-    if (cg->done) {
-        if (lead && use_h) cudaGraphSetConditional(h, 0u);
-        return;
-    }
+    if (cg->done) return;
     // one FP64 division per block, not per thread (FP64 runs at a small
     // fraction of the FP32 rate on this part)
     __shared__ double s_beta;
@@ -2026,7 +2026,6 @@ k_cg_update_p(int32_t n, CgState *cg, const TZ *__restrict__ z, double *__restri
             cg->done = 1;
             cg->status = AMG_NOT_CONVERGED;
         }
-        if (use_h) cudaGraphSetConditional(h, cg->done ? 0u : 1u);
     }
 }
 
@@ -2711,15 +2710,15 @@ void launch_true_residual(int32_t n, const FineMat &A, const double *f, const do
 }
 template <class TZ>
 void launch_replace_r(int32_t n, CgState *cg, const double *t, double *r, const TZ *zo, double *part_zo,
-                      const Smooth0Out &z0, cudaStream_t s) {
+                      const Smooth0Out &z0, int use_h, cudaGraphConditionalHandle h_in,
+                      cudaGraphConditionalHandle h_out, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_replace_r<TZ>, cg_blocks(n), kCgThreads, 0, s, n, cg, t, r, zo, part_zo, z0);
+    launch_pdl(k_replace_r<TZ>, cg_blocks(n), kCgThreads, 0, s, n, cg, t, r, zo, part_zo, z0, use_h, h_in, h_out);
 }
 template <class TZ>
-void launch_cg_update_p(int32_t n, CgState *cg, const TZ *z, double *p, double *u, int use_h,
-                        cudaGraphConditionalHandle h, cudaStream_t s) {
+void launch_cg_update_p(int32_t n, CgState *cg, const TZ *z, double *p, double *u, cudaStream_t s) {
     count_launch();
-    launch_pdl(k_cg_update_p<TZ>, cg_blocks(n), kCgThreads, 0, s, n, cg, z, p, u, use_h, h);
+    launch_pdl(k_cg_update_p<TZ>, cg_blocks(n), kCgThreads, 0, s, n, cg, z, p, u);
 }
 #define INST_CG(TZ)                                                                                                  \
     template void launch_cg_set_rz_p<TZ>(int32_t, const TZ *, double *, CgState *, cudaStream_t);                    \
@@ -2727,9 +2726,9 @@ void launch_cg_update_p(int32_t n, CgState *cg, const TZ *z, double *p, double *
                                          double *, int, cudaGraphConditionalHandle, const Smooth0Out &,              \
                                          cudaStream_t);                                                              \
     template void launch_replace_r<TZ>(int32_t, CgState *, const double *, double *, const TZ *, double *,           \
-                                       const Smooth0Out &, cudaStream_t);                                            \
-    template void launch_cg_update_p<TZ>(int32_t, CgState *, const TZ *, double *, double *, int,                    \
-                                         cudaGraphConditionalHandle, cudaStream_t);
+                                       const Smooth0Out &, int, cudaGraphConditionalHandle,                          \
+                                       cudaGraphConditionalHandle, cudaStream_t);                                    \
+    template void launch_cg_update_p<TZ>(int32_t, CgState *, const TZ *, double *, double *, cudaStream_t);
 INST_CG(double)
 INST_CG(float)
 #undef INST_CG
