@@ -344,6 +344,21 @@ int choose_lpr(int64_t rows, int64_t nnz) {
     return p;
 }
 
+// Lanes per row for the correction and sweep through A P: as above, but with at
+// least four entries a lane, since every doubling adds a step to two FP64
+// shuffle sums.  FP64, us per launch with this rule / two entries a lane / the
+// rule above: 64^3 levels 1 and 2 (16 and 17 entries a row) 7.0 + 5.1 / 8.1 +
+// 4.7 / 8.0 + 5.4; plain aggregation 71^3 (4.4) 4.9 + 4.5 / 6.1 + 4.4 / 9.6 +
+// 5.7; a mesh (24 and 16) 5.7 + 5.6 / 7.5 + 4.6 / 12.3 + 4.6.
+int choose_lpr_ap(int64_t rows, int64_t nnz) {
+    if (rows <= 0) return 1;
+    const double avg = (double)nnz / (double)rows;
+    int p = 1;
+    while (p < 32 && 16.0 * p < avg) p *= 2;
+    while (p < 32 && rows * p < 152LL * 1024 && 4.0 * p <= avg) p *= 2;
+    return p;
+}
+
 // the coarsest direct solver: dense LU (FP64) and its explicit inverse
 amg_status coarse_factor(amg_ctx *ctx) {
     Level &C = ctx->lev[ctx->nlev - 1];
@@ -504,9 +519,9 @@ amg_status numeric_rebuild(amg_ctx *ctx, const double *d_val, bool galerkin, con
 amg_status build_delta16(amg_ctx *ctx) {
     if (blockmode(ctx)) return AMG_OK;
     int *flags = nullptr;
-    TRY(alloc(ctx, &flags, (size_t)(2 * kMaxLevels)));
-    CK(cudaMemsetAsync(flags, 0, sizeof(int) * 2 * kMaxLevels, ctx->s));
-    int16_t *buf[kMaxLevels] = {}, *pbuf[kMaxLevels] = {};
+    TRY(alloc(ctx, &flags, (size_t)(3 * kMaxLevels)));
+    CK(cudaMemsetAsync(flags, 0, sizeof(int) * 3 * kMaxLevels, ctx->s));
+    int16_t *buf[kMaxLevels] = {}, *pbuf[kMaxLevels] = {}, *apbuf[kMaxLevels] = {};
     float ratio[kMaxLevels] = {};
     for (int l = 0; l < ctx->nlev; ++l) {
         Level &L = ctx->lev[l];
@@ -520,15 +535,23 @@ amg_status build_delta16(amg_ctx *ctx) {
             ratio[l] = (float)L.nc / (float)L.n;
             TRY(alloc(ctx, &pbuf[l], (size_t)L.nnzP));
             launch_col_delta16(L.n, L.P_ptr, L.P_col, ratio[l], pbuf[l], flags + kMaxLevels + l, ctx->s);
+            if (l > 0) {
+                TRY(alloc(ctx, &apbuf[l], (size_t)L.nnzAP));
+                launch_col_delta16(L.n, L.AP_ptr, L.AP_col, ratio[l], apbuf[l], flags + 2 * kMaxLevels + l, ctx->s);
+            }
         }
     }
-    int h[2 * kMaxLevels] = {};
+    int h[3 * kMaxLevels] = {};
     CK(cudaMemcpyAsync(h, flags, sizeof(h), cudaMemcpyDeviceToHost, ctx->s));
     CK(cudaStreamSynchronize(ctx->s));
     for (int l = 0; l < ctx->nlev; ++l) {
         if (buf[l] && h[l] == 0) ctx->lev[l].A_c16 = buf[l];
         if (pbuf[l] && h[kMaxLevels + l] == 0) {
             ctx->lev[l].P_c16 = pbuf[l];
+            ctx->lev[l].P_ratio = ratio[l];
+        }
+        if (apbuf[l] && h[2 * kMaxLevels + l] == 0) {
+            ctx->lev[l].AP_c16 = apbuf[l];
             ctx->lev[l].P_ratio = ratio[l];
         }
     }
@@ -638,6 +661,7 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         TRY(symbolic_product(ctx, L.n, nagg, L.A_ptr, L.A_col, L.P_ptr, L.P_col, 0, &L.AP_ptr, &L.AP_col,
                              &L.nnzAP));
         TRY(alloc(ctx, &L.AP_val, (size_t)L.nnzAP));
+        L.lpr_ap = choose_lpr_ap(L.n, L.nnzAP);
         Level &C = ctx->lev[ctx->nlev];
         C.n = nagg;
         TRY(symbolic_product(ctx, nagg, nagg, L.R_ptr, L.R_col, L.AP_ptr, L.AP_col, 1, &C.A_ptr, &C.A_col, &C.nnz));
@@ -706,7 +730,12 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
     ctx->luT = nullptr;
     if (lu_wants_transpose((int32_t)nL)) TRY(alloc(ctx, &ctx->luT, (size_t)(nL * nL)));
     if (mixed(ctx))
-        for (int l = 1; l < ctx->nlev; ++l) launch_cast_f32(ctx->lev[l].nnz, ctx->lev[l].A_val, ctx->lev[l].A_valf, ctx->s);
+        for (int l = 1; l < ctx->nlev; ++l) {
+            const Level &L = ctx->lev[l];
+            launch_cast_f32(L.nnz, L.A_val, L.A_valf, ctx->s);
+            // (the coarser levels' post-smoothing reads A P)
+            if (l + 1 < ctx->nlev) launch_cast_f32(L.nnzAP, L.AP_val, L.AP_valf, ctx->s);
+        }
     TRY(build_delta16(ctx));
     TRY(numeric_rebuild(ctx, blockmode(ctx) ? ctx->lev[0].Ab : ctx->lev[0].A_val, false));
     TRY(check_device(ctx, "full setup"));
@@ -891,6 +920,7 @@ struct Vops<double> {
     static const double *m(const Level &L) { return L.m; }
     static const double *P(const Level &L) { return L.P_val; }
     static const double *R(const Level &L) { return L.R_val; }
+    static const double *AP(const Level &L) { return L.AP_val; }
 };
 template <>
 struct Vops<float> {
@@ -899,6 +929,7 @@ struct Vops<float> {
     static const float *m(const Level &L) { return L.mf; }
     static const float *P(const Level &L) { return L.P_valf; }
     static const float *R(const Level &L) { return L.R_valf; }
+    static const float *AP(const Level &L) { return L.AP_valf; }
 };
 
 // pre-smoothing from a zero guess and the residual on level l (input f of type TF);
@@ -1016,12 +1047,16 @@ void enqueue_vcycle(amg_ctx *ctx, const double *r, TZ *z, const int *skip, doubl
     cur[nl - 1] = Vops<V>::vec(Cst).u;
     for (int l = nl - 2; l >= 1; --l) {
         Level &L = ctx->lev[l];
-        launch_prolong<V>(L, Vops<V>::P(L), cur[l + 1], cur[l], skip, ctx->s);
-        // the post-smoothed iterate stays in this level's buffers
+        // the post-smoothed iterate stays in this level's buffers; the first
+        // sweep comes with the correction (v.r: the residual before it)
         V *u = cur[l];
         VecSet<V> &v = Vops<V>::vec(L);
         V *t = (u == v.u) ? v.t : v.u;
-        for (int k = 0; k < ctx->prm.npost; ++k) {
+        if (ctx->prm.npost > 0)
+            launch_correct_sweep<V>(L, Vops<V>::P(L), Vops<V>::AP(L), Vops<V>::m(L), v.r, cur[l + 1], u, skip, ctx->s);
+        else
+            launch_prolong<V>(L, Vops<V>::P(L), cur[l + 1], u, skip, ctx->s);
+        for (int k = 1; k < ctx->prm.npost; ++k) {
             launch_smooth_sweep<V, V, V>(L, Vops<V>::A(L), Vops<V>::m(L), v.f, u, t, skip, ctx->s);
             std::swap(u, t);
         }

@@ -112,6 +112,7 @@ struct Level {
     // P's columns as two-byte offsets from (int)(row * P_ratio), when they fit
     int16_t *P_c16 = nullptr;
     float P_ratio = 0.0f;
+    int16_t *AP_c16 = nullptr;  // A P's columns likewise (the coarser levels)
     double *P_val = nullptr;
     float *P_valf = nullptr;
     int32_t *R_ptr = nullptr, *R_col = nullptr;
@@ -126,7 +127,7 @@ struct Level {
     uint16_t *slot1 = nullptr, *slot2 = nullptr;
     int32_t max_ap_row = 0, max_ac_row = 0;
     // lanes per row of the matrix-vector pieces on this level (A rows, R rows)
-    int lpr = 1, lpr_r = 8;
+    int lpr = 1, lpr_r = 8, lpr_ap = 8;
     // the same products as fixed gather operators, built at the first partial rebuild
     bool gather_ready = false;
     int32_t *g1_ptr = nullptr, *g1_idx = nullptr, *g2_ptr = nullptr, *g2_idx = nullptr;
@@ -378,6 +379,10 @@ void launch_restrict(const Level &L, const V *Rval, const V *r, V *fc, const V *
                      cudaStream_t s);
 template <class V>
 void launch_prolong(const Level &L, const V *Pval, const V *uc, V *u, const int *skip, cudaStream_t s);
+// u += P u_c and the first post-smoothing sweep, through A P (r: the residual before)
+template <class V>
+void launch_correct_sweep(const Level &L, const V *Pval, const V *APval, const V *m, const V *r, const V *uc, V *u,
+                          const int *skip, cudaStream_t s);
 template <class V, class TF, class TO>
 void launch_coarse_solve(int32_t n, const double *inv, const TF *f, TO *u, const int *skip, cudaStream_t s);
 template <class TI, class TO>
