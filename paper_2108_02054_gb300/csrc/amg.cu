@@ -579,7 +579,7 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
     }
     TRY(alloc(ctx, &F.A_val, (size_t)nnz));
     TRY(alloc(ctx, &F.dia, (size_t)n));
-    launch_check_pattern(n, F.A_ptr, F.A_col, F.dia, ctx->d_st, ctx->s);
+    launch_check_pattern(n, nnz, F.A_ptr, F.A_col, F.dia, ctx->d_st, ctx->s);
     launch_check_finite((int64_t)nvals(ctx), d_val, ctx->d_st, ctx->s);
     if (blockmode(ctx)) {
         // the node graph carries the block norms
@@ -616,8 +616,8 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         TRY(alloc(ctx, &r1, (size_t)L.n));
         TRY(alloc(ctx, &counter, 1));
         TRY(alloc(ctx, &scan_tmp, (size_t)scan_tmp_elems(L.n)));
-        launch_strength(L.n, L.A_ptr, L.A_col, L.A_val, L.dia, theta * theta, L.strong, deg, ctx->s);
-        int32_t nagg = run_aggregation(L.n, L.A_ptr, L.A_col, L.A_val, L.strong, deg, L.agg, state, m1, r1, root_id,
+        launch_strength(L.n, L.nnz, L.A_ptr, L.A_col, L.A_val, L.dia, theta * theta, L.strong, deg, ctx->s);
+        int32_t nagg = run_aggregation(L.n, L.nnz, L.A_ptr, L.A_col, L.A_val, L.strong, deg, L.agg, state, m1, r1, root_id,
                                        agg1, root_of, counter, ctx->d_st, scan_tmp, ctx->s);
         if (nagg < 0) {
             CK(cudaGetLastError());
@@ -635,12 +635,12 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         int32_t *plen = nullptr;
         TRY(alloc(ctx, &plen, (size_t)L.n));
         TRY(alloc(ctx, &L.P_ptr, (size_t)L.n + 1));
-        launch_p_count(L.n, L.A_ptr, L.A_col, L.strong, L.agg, p.smoothed, plen, ctx->s);
+        launch_p_count(L.n, L.nnz, L.A_ptr, L.A_col, L.strong, L.agg, p.smoothed, plen, ctx->s);
         TRY(scan(ctx, plen, L.P_ptr, L.n));
         TRY(read_scalar(ctx, L.P_ptr + L.n, &L.nnzP));
         TRY(alloc(ctx, &L.P_col, (size_t)L.nnzP));
         TRY(alloc(ctx, &L.P_val, (size_t)L.nnzP));
-        launch_p_fill(L.n, L.A_ptr, L.A_col, L.A_val, L.strong, L.dia, L.agg, p.omega, p.smoothed, L.P_ptr, L.P_col,
+        launch_p_fill(L.n, L.nnz, L.A_ptr, L.A_col, L.A_val, L.strong, L.dia, L.agg, p.omega, p.smoothed, L.P_ptr, L.P_col,
                       L.P_val, ctx->s);
         // R = P^T
         int32_t *cnt = nullptr, *cursor = nullptr;
@@ -667,7 +667,7 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         TRY(symbolic_product(ctx, nagg, nagg, L.R_ptr, L.R_col, L.AP_ptr, L.AP_col, 1, &C.A_ptr, &C.A_col, &C.nnz));
         TRY(alloc(ctx, &C.A_val, (size_t)C.nnz));
         TRY(alloc(ctx, &C.dia, (size_t)C.n));
-        launch_check_pattern(C.n, C.A_ptr, C.A_col, C.dia, ctx->d_st, ctx->s);
+        launch_check_pattern(C.n, C.nnz, C.A_ptr, C.A_col, C.dia, ctx->d_st, ctx->s);
         TRY(max_row(ctx, L.n, L.AP_ptr, &L.max_ap_row));
         TRY(max_row(ctx, C.n, C.A_ptr, &L.max_ac_row));
         if (L.max_ap_row > 65535 || L.max_ac_row > 65535)
@@ -683,7 +683,7 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         TRY(read_scalar(ctx, L.t1ptr + L.n, &nt1));
         L.nt1 = nt1;
         TRY(alloc(ctx, &L.slot1, (size_t)nt1));
-        launch_t1_fill(L.n, L.A_ptr, L.A_col, L.P_ptr, L.P_col, L.AP_ptr, L.AP_col, L.t1ptr, L.slot1, ctx->d_st,
+        launch_t1_fill(L.n, L.nnz, L.A_ptr, L.A_col, L.P_ptr, L.P_col, L.AP_ptr, L.AP_col, L.t1ptr, L.slot1, ctx->d_st,
                        ctx->s);
         TRY(alloc(ctx, &L.t2ptr, (size_t)nagg + 1));
         launch_t2_count(nagg, L.R_ptr, L.R_col, L.AP_ptr, tc, ctx->s);

@@ -265,19 +265,20 @@ void launch_levelset_vals(int dim, int N, const double *fx, const double *fy, co
 
 // a caller's row pointers (ptr[0] = 0, non-decreasing, ptr[n] = nnz): DEV_ERR_PATTERN otherwise
 void launch_check_rowptr(int32_t n, int32_t nnz, const int32_t *ptr, int *st, cudaStream_t s);
-void launch_check_pattern(int32_t n, const int32_t *ptr, const int32_t *col, int32_t *dia, int *st,
+// (nnz picks the lanes per row)
+void launch_check_pattern(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, int32_t *dia, int *st,
                           cudaStream_t s);
 void launch_check_finite(int64_t nnz, const double *val, int *st, cudaStream_t s);
-void launch_strength(int32_t n, const int32_t *ptr, const int32_t *col, const double *val, const int32_t *dia,
+void launch_strength(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const double *val, const int32_t *dia,
                      double eps2, uint8_t *strong, int32_t *deg, cudaStream_t s);
 // aggregation; returns the number of aggregates (host sync inside), or -1 on error
-int32_t run_aggregation(int32_t n, const int32_t *ptr, const int32_t *col, const double *val,
+int32_t run_aggregation(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const double *val,
                         const uint8_t *strong, const int32_t *deg, int32_t *agg, int8_t *state, int64_t *m1,
                         uint8_t *r1, int32_t *root_id, int32_t *agg1, int32_t *root_of, int *counter, int *st,
                         int64_t *scan_tmp, cudaStream_t s);
-void launch_p_count(int32_t n, const int32_t *ptr, const int32_t *col, const uint8_t *strong, const int32_t *agg,
+void launch_p_count(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const uint8_t *strong, const int32_t *agg,
                     int smoothed, int32_t *plen, cudaStream_t s);
-void launch_p_fill(int32_t n, const int32_t *ptr, const int32_t *col, const double *val, const uint8_t *strong,
+void launch_p_fill(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const double *val, const uint8_t *strong,
                    const int32_t *dia, const int32_t *agg, double omega, int smoothed, const int32_t *P_ptr,
                    int32_t *P_col, double *P_val, cudaStream_t s);
 void launch_count_cols(int64_t nnz, const int32_t *col, int32_t *cnt, cudaStream_t s);
@@ -297,7 +298,7 @@ void launch_spgemm_symbolic(int32_t nrows, int32_t ncols, const int32_t *X_ptr, 
                             int32_t *len, const int32_t *C_ptr, int32_t *C_col, int *st, cudaStream_t s);
 void launch_t1_count(int32_t n, const int32_t *A_ptr, const int32_t *A_col, const int32_t *P_ptr, int32_t *cnt,
                      cudaStream_t s);
-void launch_t1_fill(int32_t n, const int32_t *A_ptr, const int32_t *A_col, const int32_t *P_ptr,
+void launch_t1_fill(int32_t n, int32_t nnz, const int32_t *A_ptr, const int32_t *A_col, const int32_t *P_ptr,
                     const int32_t *P_col, const int32_t *AP_ptr, const int32_t *AP_col, const int32_t *t1ptr,
                     uint16_t *slot1, int *st, cudaStream_t s);
 void launch_t2_count(int32_t nc, const int32_t *R_ptr, const int32_t *R_col, const int32_t *AP_ptr, int32_t *cnt,

@@ -286,19 +286,47 @@ __global__ void k_check_rowptr(int32_t n, int32_t nnz, const int32_t *__restrict
     }
 }
 
+// The setup's row kernels take G lanes per row: one on grids' finest levels
+// (5 to 7 entries a row), a warp where rows hold more than eight on average
+// (the launchers' row_lanes), since a coarse level of a thousand rows of 50 to
+// 100 entries leaves one thread per row with a long serial chain on an idle
+// chip.  What a row's lanes find is combined without regard to their order, or
+// in the row's column order where that decides the result, so both forms give
+// the same bits.  At 64^3 (levels of 24,028 and 1,289 rows) with one thread per
+// row: P's pattern 125 + 333 us, its values 129 + 218, the slots of A P 142 +
+// 267, A P 128 + 225, strength 95 + 144, a round of the independent set 42 + 59;
+// the step with a full setup went from 9.18 to 6.01 ms.
+template <int G>
+__device__ __forceinline__ int32_t row_of_thread(int &sub) {
+    const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    sub = (int)(gt % G);
+    return (int32_t)(gt / G);
+}
+template <int G>
+__device__ __forceinline__ bool row_any(bool x) {
+    return G == 1 ? x : __any_sync(0xffffffffu, x) != 0;
+}
+
+template <int G>
 __global__ void k_check_pattern(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
                                 int32_t *__restrict__ dia, int *st) {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0 && ptr[0] != 0) atomicOr(st, DEV_ERR_PATTERN);
-    if (i >= n) return;
-    int32_t b = ptr[i], e = ptr[i + 1];
+    int sub;
+    const int32_t i = row_of_thread<G>(sub);
+    if (i == 0 && sub == 0 && ptr[0] != 0) atomicOr(st, DEV_ERR_PATTERN);
+    if (i >= n) return;  // (a warp's lanes share the row)
+    const int32_t b = ptr[i], e = ptr[i + 1];
     int32_t d = -1;
     bool bad = e < b;
-    for (int32_t p = b; p < e && !bad; ++p) {
-        int32_t c = col[p];
+    for (int32_t p = b + sub; p < e && !bad; p += G) {
+        const int32_t c = col[p];
         if (c < 0 || c >= n || (p > b && c <= col[p - 1])) bad = true;
         if (c == i) d = p;
     }
+    if (G > 1) {
+        bad = row_any<G>(bad);
+        d = __reduce_max_sync(0xffffffffu, d);
+    }
+    if (sub != 0) return;
     if (bad || d < 0) atomicOr(st, DEV_ERR_PATTERN);
     dia[i] = d < 0 ? b : d;
 }
@@ -311,14 +339,16 @@ __global__ void k_check_finite(int64_t n, const double *__restrict__ v, int *st)
 // ------------------------------------------------------------------ strength
 // (i,j), j != i, is strong iff a_ij^2 > eps^2 |a_ii a_jj| holds in row i's
 // direction or in row j's; each product separately rounded.
+template <int G>
 __global__ void k_strength(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
                            const double *__restrict__ val, const int32_t *__restrict__ dia, double eps2,
                            uint8_t *__restrict__ strong, int32_t *__restrict__ deg) {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    int sub;
+    const int32_t i = row_of_thread<G>(sub);
     if (i >= n) return;
     const double aii = val[dia[i]];
     int32_t cnt = 0;
-    for (int32_t p = ptr[i]; p < ptr[i + 1]; ++p) {
+    for (int32_t p = ptr[i] + sub; p < ptr[i + 1]; p += G) {
         int32_t j = col[p];
         uint8_t s = 0;
         if (j != i) {
@@ -337,7 +367,8 @@ __global__ void k_strength(int32_t n, const int32_t *__restrict__ ptr, const int
         strong[p] = s;
         cnt += s;
     }
-    deg[i] = cnt;
+    if (G > 1) cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (sub == 0) deg[i] = cnt;
 }
 
 // ------------------------------------------------------------------ aggregation
@@ -348,59 +379,79 @@ __global__ void k_mis_init(int32_t n, const int32_t *__restrict__ deg, int8_t *_
 }
 
 // m1[i] = largest priority among undecided nodes of {i} + strong(i), -1 if none
+template <int G>
 __global__ void k_mis_m1(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
                          const uint8_t *__restrict__ strong, const int8_t *__restrict__ state,
                          int64_t *__restrict__ m1) {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    int sub;
+    const int32_t i = row_of_thread<G>(sub);
     if (i >= n) return;
-    if (state[i] == 3) { m1[i] = -1; return; }
-    int64_t m = state[i] == 0 ? (int64_t)node_priority((uint32_t)i) : -1;
-    for (int32_t p = ptr[i]; p < ptr[i + 1]; ++p) {
+    const int8_t si = state[i];
+    if (si == 3) {
+        if (sub == 0) m1[i] = -1;
+        return;
+    }
+    bool has = si == 0;
+    uint32_t m = has ? node_priority((uint32_t)i) : 0u;
+    for (int32_t p = ptr[i] + sub; p < ptr[i + 1]; p += G) {
         if (!strong[p]) continue;
-        int32_t j = col[p];
+        const int32_t j = col[p];
         if (state[j] == 0) {
-            int64_t q = (int64_t)node_priority((uint32_t)j);
-            m = q > m ? q : m;
+            m = max(m, node_priority((uint32_t)j));
+            has = true;
         }
     }
-    m1[i] = m;
+    if (G > 1) {
+        m = __reduce_max_sync(0xffffffffu, m);
+        has = row_any<G>(has);
+    }
+    if (sub == 0) m1[i] = has ? (int64_t)m : -1;
 }
 
 // an undecided node whose priority is the largest among undecided nodes
 // within strong distance 2 becomes a root
+template <int G>
 __global__ void k_mis_select(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
                              const uint8_t *__restrict__ strong, int8_t *__restrict__ state,
                              const int64_t *__restrict__ m1) {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    int sub;
+    const int32_t i = row_of_thread<G>(sub);
     if (i >= n || state[i] != 0) return;
-    int64_t m = m1[i];
-    for (int32_t p = ptr[i]; p < ptr[i + 1]; ++p)
-        if (strong[p]) {
-            int64_t q = m1[col[p]];
-            m = q > m ? q : m;
-        }
-    if (m == (int64_t)node_priority((uint32_t)i)) state[i] = 1;
+    const int64_t own = (int64_t)node_priority((uint32_t)i);
+    bool larger = m1[i] > own;
+    for (int32_t p = ptr[i] + sub; p < ptr[i + 1]; p += G)
+        if (strong[p]) larger = larger || m1[col[p]] > own;
+    larger = row_any<G>(larger);
+    // (m1[i] is at least the node's own priority)
+    if (sub == 0 && !larger) state[i] = 1;
 }
 
+template <int G>
 __global__ void k_mis_r1(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
                          const uint8_t *__restrict__ strong, const int8_t *__restrict__ state,
                          uint8_t *__restrict__ r1) {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    int sub;
+    const int32_t i = row_of_thread<G>(sub);
     if (i >= n) return;
-    uint8_t r = state[i] == 1;
-    for (int32_t p = ptr[i]; p < ptr[i + 1] && !r; ++p)
-        if (strong[p] && state[col[p]] == 1) r = 1;
-    r1[i] = r;
+    bool r = state[i] == 1;
+    for (int32_t p = ptr[i] + sub; p < ptr[i + 1] && !r; p += G)
+        if (strong[p] && state[col[p]] == 1) r = true;
+    r = row_any<G>(r);
+    if (sub == 0) r1[i] = r;
 }
 
+template <int G>
 __global__ void k_mis_exclude(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
                               const uint8_t *__restrict__ strong, int8_t *__restrict__ state,
                               const uint8_t *__restrict__ r1, int *__restrict__ undecided) {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    int sub;
+    const int32_t i = row_of_thread<G>(sub);
     if (i >= n || state[i] != 0) return;
     bool ex = r1[i];
-    for (int32_t p = ptr[i]; p < ptr[i + 1] && !ex; ++p)
+    for (int32_t p = ptr[i] + sub; p < ptr[i + 1] && !ex; p += G)
         if (strong[p] && r1[col[p]]) ex = true;
+    ex = row_any<G>(ex);
+    if (sub != 0) return;
     if (ex) state[i] = 2;
     else atomicAdd(undecided, 1);
 }
@@ -410,60 +461,76 @@ __global__ void k_root_flags(int32_t n, const int8_t *__restrict__ state, int32_
     if (i < n) flag[i] = state[i] == 1;
 }
 
-// phase 1: a root and its strong neighbours form aggregate root_id[root]
+// phase 1: a root and its strong neighbours form aggregate root_id[root] (the
+// first root in column order, should a one-sided pattern offer several)
+template <int G>
 __global__ void k_agg_phase1(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
                              const uint8_t *__restrict__ strong, const int8_t *__restrict__ state,
                              const int32_t *__restrict__ root_id, int32_t *__restrict__ agg1,
                              int32_t *__restrict__ root_of) {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    int sub;
+    const int32_t i = row_of_thread<G>(sub);
     if (i >= n) return;
+    const int8_t si = state[i];
     int32_t a = -1;
-    if (state[i] == 1) {
+    if (si == 1) {
         a = root_id[i];
-        root_of[a] = i;
-    } else if (state[i] != 3) {
-        for (int32_t p = ptr[i]; p < ptr[i + 1]; ++p)
-            if (strong[p] && state[col[p]] == 1) { a = root_id[col[p]]; break; }
+        if (sub == 0) root_of[a] = i;
+    } else if (si != 3) {
+        int32_t first = INT_MAX;
+        for (int32_t p = ptr[i] + sub; p < ptr[i + 1]; p += G)
+            if (strong[p] && state[col[p]] == 1) {
+                first = p;
+                break;
+            }
+        if (G > 1) first = __reduce_min_sync(0xffffffffu, first);
+        if (first != INT_MAX) a = root_id[col[first]];
     }
-    agg1[i] = a;
+    if (sub == 0) agg1[i] = a;
 }
 
 // phase 2: a remaining non-isolated node joins the phase-1 aggregate of its
-// strong neighbour with the largest |a_ij| (ties: larger root priority)
+// strong neighbour with the largest |a_ij| (ties: larger root priority; equal
+// priorities are one root)
+template <int G>
 __global__ void k_agg_phase2(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
                              const double *__restrict__ val, const uint8_t *__restrict__ strong,
                              const int8_t *__restrict__ state, const int32_t *__restrict__ agg1,
                              const int32_t *__restrict__ root_of, int32_t *__restrict__ agg, int *st) {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    int sub;
+    const int32_t i = row_of_thread<G>(sub);
     if (i >= n) return;
     int32_t a = agg1[i];
     if (state[i] != 3 && a < 0) {
         double bestv = -1.0;
         uint32_t bestk = 0;
-        for (int32_t p = ptr[i]; p < ptr[i + 1]; ++p) {
+        for (int32_t p = ptr[i] + sub; p < ptr[i + 1]; p += G) {
             if (!strong[p]) continue;
-            int32_t aj = agg1[col[p]];
+            const int32_t aj = agg1[col[p]];
             if (aj < 0) continue;
-            double v = fabs(val[p]);
-            uint32_t k = node_priority((uint32_t)root_of[aj]);
+            const double v = fabs(val[p]);
+            const uint32_t k = node_priority((uint32_t)root_of[aj]);
             if (a < 0 || v > bestv || (v == bestv && k > bestk)) { a = aj; bestv = v; bestk = k; }
         }
-        if (a < 0) atomicOr(st, DEV_ERR_STATE);
+        if (G > 1) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const int32_t ao = __shfl_xor_sync(0xffffffffu, a, o);
+                const double vo = __shfl_xor_sync(0xffffffffu, bestv, o);
+                const uint32_t ko = __shfl_xor_sync(0xffffffffu, bestk, o);
+                if (ao >= 0 && (a < 0 || vo > bestv || (vo == bestv && ko > bestk))) { a = ao; bestv = vo; bestk = ko; }
+            }
+        }
+        if (a < 0 && sub == 0) atomicOr(st, DEV_ERR_STATE);
     }
-    agg[i] = a;
+    if (sub == 0) agg[i] = a;
 }
 
 // ------------------------------------------------------------------ prolongation
 // row i of smoothed P has one column per distinct aggregate among {i} + strong(i)
-__global__ void k_p_count(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                          const uint8_t *__restrict__ strong, const int32_t *__restrict__ agg, int smoothed,
-                          int32_t *__restrict__ plen) {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (agg[i] < 0) { plen[i] = 0; return; }
-    if (!smoothed) { plen[i] = 1; return; }
+__device__ __forceinline__ int32_t p_row_count(int32_t i, int32_t b, int32_t e, const int32_t *__restrict__ col,
+                                               const uint8_t *__restrict__ strong, const int32_t *__restrict__ agg) {
     int32_t cnt = 0;
-    const int32_t b = ptr[i], e = ptr[i + 1];
     for (int32_t p = b; p < e; ++p) {
         int32_t j = col[p];
         if (j != i && !strong[p]) continue;
@@ -477,28 +544,26 @@ __global__ void k_p_count(int32_t n, const int32_t *__restrict__ ptr, const int3
         }
         cnt += !dup;
     }
-    plen[i] = cnt;
+    return cnt;
+}
+__global__ void k_p_count(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
+                          const uint8_t *__restrict__ strong, const int32_t *__restrict__ agg, int smoothed,
+                          int32_t *__restrict__ plen) {
+    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    if (agg[i] < 0) { plen[i] = 0; return; }
+    if (!smoothed) { plen[i] = 1; return; }
+    plen[i] = p_row_count(i, ptr[i], ptr[i + 1], col, strong, agg);
 }
 
 // P = (I - w D_F^-1 A_F) P_tent: d_i = a_ii + weak off-diagonals (column order);
 // P[i,c] = [c == agg(i)] - sum_{j in {i}+strong(i), agg(j) = c} (w * A_F[i,j]) / d_i
 // in column order, A_F[i,i] = d_i.
-__global__ void k_p_fill(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
-                         const double *__restrict__ val, const uint8_t *__restrict__ strong,
-                         const int32_t *__restrict__ dia, const int32_t *__restrict__ agg, double omega,
-                         int smoothed, const int32_t *__restrict__ P_ptr, int32_t *__restrict__ P_col,
-                         double *__restrict__ P_val) {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int32_t ai = agg[i];
-    if (ai < 0) return;
-    const int32_t base = P_ptr[i];
-    if (!smoothed) {
-        P_col[base] = ai;
-        P_val[base] = 1.0;
-        return;
-    }
-    const int32_t b = ptr[i], e = ptr[i + 1];
+__device__ __forceinline__ void p_row_fill(int32_t i, int32_t b, int32_t e, int32_t ai, int32_t base,
+                                           const int32_t *__restrict__ col, const double *__restrict__ val,
+                                           const uint8_t *__restrict__ strong, const int32_t *__restrict__ dia,
+                                           const int32_t *__restrict__ agg, double omega,
+                                           int32_t *__restrict__ P_col, double *__restrict__ P_val) {
     int32_t nc = 0;
     for (int32_t p = b; p < e; ++p) {
         int32_t j = col[p];
@@ -532,6 +597,119 @@ __global__ void k_p_fill(int32_t n, const int32_t *__restrict__ ptr, const int32
         P_val[base + s] = v;
     }
 }
+__global__ void k_p_fill(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
+                         const double *__restrict__ val, const uint8_t *__restrict__ strong,
+                         const int32_t *__restrict__ dia, const int32_t *__restrict__ agg, double omega,
+                         int smoothed, const int32_t *__restrict__ P_ptr, int32_t *__restrict__ P_col,
+                         double *__restrict__ P_val) {
+    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int32_t ai = agg[i];
+    if (ai < 0) return;
+    const int32_t base = P_ptr[i];
+    if (!smoothed) {
+        P_col[base] = ai;
+        P_val[base] = 1.0;
+        return;
+    }
+    p_row_fill(i, ptr[i], ptr[i + 1], ai, base, col, val, strong, dia, agg, omega, P_col, P_val);
+}
+
+// The same two passes with a warp per row: the row's aggregates (-1: none, -2:
+// a weak off-diagonal) and its quotients staged in shared memory, the lanes
+// over the entries.  The diagonal sum and each entry's sum over its terms run in
+// column order as above.  Rows longer than kPRow are taken by one lane as above.
+constexpr int kPWarps = 4, kPRow = 512;
+__device__ __forceinline__ int32_t stage_row_aggs(int32_t i, int32_t b, int32_t len, int lane,
+                                                  const int32_t *__restrict__ col,
+                                                  const uint8_t *__restrict__ strong,
+                                                  const int32_t *__restrict__ agg, int32_t *c) {
+    for (int32_t e = lane; e < len; e += 32) {
+        const int32_t j = col[b + e];
+        c[e] = j == i || strong[b + e] ? max(agg[j], -1) : -2;
+    }
+    __syncwarp();
+    return len;
+}
+__device__ __forceinline__ bool first_of_its_agg(const int32_t *c, int32_t e) {
+    if (c[e] < 0) return false;
+    for (int32_t q = 0; q < e; ++q)
+        if (c[q] == c[e]) return false;
+    return true;
+}
+__global__ void __launch_bounds__(kPWarps * 32)
+k_p_count_warp(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
+               const uint8_t *__restrict__ strong, const int32_t *__restrict__ agg, int32_t *__restrict__ plen) {
+    __shared__ int32_t s_c[kPWarps][kPRow];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int32_t i = blockIdx.x * kPWarps + w;
+    if (i >= n) return;  // warp-uniform
+    if (agg[i] < 0) {
+        if (lane == 0) plen[i] = 0;
+        return;
+    }
+    const int32_t b = ptr[i], len = ptr[i + 1] - b;
+    if (len > kPRow) {
+        if (lane == 0) plen[i] = p_row_count(i, b, b + len, col, strong, agg);
+        return;
+    }
+    stage_row_aggs(i, b, len, lane, col, strong, agg, s_c[w]);
+    int32_t cnt = 0;
+    for (int32_t e = lane; e < len; e += 32) cnt += first_of_its_agg(s_c[w], e);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) plen[i] = cnt;
+}
+__global__ void __launch_bounds__(kPWarps * 32)
+k_p_fill_warp(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
+              const double *__restrict__ val, const uint8_t *__restrict__ strong, const int32_t *__restrict__ dia,
+              const int32_t *__restrict__ agg, double omega, const int32_t *__restrict__ P_ptr,
+              int32_t *__restrict__ P_col, double *__restrict__ P_val) {
+    __shared__ int32_t s_c[kPWarps][kPRow], s_list[kPWarps][kPRow];
+    __shared__ double s_t[kPWarps][kPRow];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int32_t i = blockIdx.x * kPWarps + w;
+    if (i >= n) return;  // warp-uniform
+    const int32_t ai = agg[i];
+    if (ai < 0) return;
+    const int32_t b = ptr[i], len = ptr[i + 1] - b, base = P_ptr[i];
+    if (len > kPRow) {
+        if (lane == 0) p_row_fill(i, b, b + len, ai, base, col, val, strong, dia, agg, omega, P_col, P_val);
+        return;
+    }
+    int32_t *c = s_c[w], *list = s_list[w];
+    double *t = s_t[w];
+    for (int32_t e = lane; e < len; e += 32) t[e] = val[b + e];
+    stage_row_aggs(i, b, len, lane, col, strong, agg, c);
+    const int32_t ed = dia[i] - b;
+    double d = t[ed];
+    for (int32_t e = 0; e < len; ++e)
+        if (c[e] == -2) d = __dadd_rn(d, t[e]);  // every lane forms the same sum
+    __syncwarp();
+    const DivRecip rd = div_recip(d);
+    int32_t nd = 0;
+    for (int32_t e0 = 0; e0 < len; e0 += 32) {
+        const int32_t e = e0 + lane;
+        bool first = false;
+        if (e < len) {
+            first = first_of_its_agg(c, e);
+            if (c[e] >= 0) t[e] = div_rn(__dmul_rn(omega, e == ed ? d : t[e]), rd);
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, first);
+        if (first) list[nd + __popc(m & ((1u << lane) - 1u))] = e;
+        nd += __popc(m);
+    }
+    __syncwarp();
+    for (int32_t k = lane; k < nd; k += 32) {
+        const int32_t e0 = list[k], ck = c[e0];
+        int32_t rank = 0;
+        for (int32_t q = 0; q < nd; ++q) rank += c[list[q]] < ck;
+        double v = ck == ai ? 1.0 : 0.0;
+        for (int32_t e = e0; e < len; ++e)
+            if (c[e] == ck) v = __dsub_rn(v, t[e]);
+        P_col[base + rank] = ck;
+        P_val[base + rank] = v;
+    }
+}
 
 __global__ void k_count_cols(int64_t nnz, const int32_t *__restrict__ col, int32_t *__restrict__ cnt) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x)
@@ -553,9 +731,10 @@ __global__ void k_transpose_scatter(int32_t n, const int32_t *__restrict__ P_ptr
 }
 
 // Sort each row of a CSR matrix by column (columns distinct within a row),
-// one warp per row.  Rows of up to 128 entries are sorted in registers by a
+// one warp per row.  Rows of up to 512 entries are sorted in registers by a
 // bitonic network over the warp (entry e = 32 j + lane in slot j; padding
-// sorts last); longer rows by an insertion sort in place.
+// sorts last); longer rows by an insertion sort in place.  (With the network up
+// to 128 entries only, the few longer rows of a coarse R took 567 us at 64^3.)
 template <int E>
 __device__ __forceinline__ void warp_bitonic(int32_t (&key)[E], double (&val)[E], int lane) {
 #pragma unroll
@@ -616,15 +795,20 @@ __device__ __forceinline__ void warp_sort_row(int32_t b, int32_t len, int32_t *_
     }
 }
 constexpr int kSortWarps = 4;
+// rows of more than `above` entries (the others are left to another launch)
+template <int EMAX>
 __global__ void __launch_bounds__(kSortWarps * 32)
-k_sort_rows(int32_t nrows, const int32_t *__restrict__ ptr, int32_t *__restrict__ col, double *__restrict__ val) {
+k_sort_rows(int32_t nrows, int32_t above, const int32_t *__restrict__ ptr, int32_t *__restrict__ col,
+            double *__restrict__ val) {
     const int lane = threadIdx.x & 31;
     const int32_t r = blockIdx.x * kSortWarps + (threadIdx.x >> 5);
     if (r >= nrows) return;  // warp-uniform
     const int32_t b = ptr[r], e = ptr[r + 1], len = e - b;
-    if (len <= 1) return;
+    if (len <= 1 || len <= above || (EMAX == 4 && len > 128)) return;
     if (len <= 64) warp_sort_row<2>(b, len, col, val, lane);
     else if (len <= 128) warp_sort_row<4>(b, len, col, val, lane);
+    else if (EMAX > 4 && len <= 256) warp_sort_row<8>(b, len, col, val, lane);
+    else if (EMAX > 4 && len <= 512) warp_sort_row<16>(b, len, col, val, lane);
     else if (lane == 0)
         for (int32_t a = b + 1; a < e; ++a) {
             int32_t c = col[a];
@@ -1012,23 +1196,31 @@ void launch_check_rowptr(int32_t n, int32_t nnz, const int32_t *ptr, int *st, cu
     count_launch();
     k_check_rowptr<<<(unsigned)(b > 4096 ? 4096 : b), kThreads, 0, s>>>(n, nnz, ptr, st);
 }
-void launch_check_pattern(int32_t n, const int32_t *ptr, const int32_t *col, int32_t *dia, int *st,
+namespace {
+// lanes per row of the setup's row kernels: a warp above eight entries a row
+// on average (grids' finest levels have 5 to 7, coarse levels 30 and more)
+bool warp_rows(int32_t n, int32_t nnz) { return (int64_t)nnz > 8 * (int64_t)n; }
+}  // namespace
+#define ROW_LANES(KERNEL, ...)                                                                     \
+    do {                                                                                           \
+        count_launch();                                                                            \
+        if (warp_rows(n, nnz)) KERNEL<32><<<nblocks((int64_t)n * 32), kThreads, 0, s>>>(__VA_ARGS__); \
+        else KERNEL<1><<<nblocks(n), kThreads, 0, s>>>(__VA_ARGS__);                               \
+    } while (0)
+void launch_check_pattern(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, int32_t *dia, int *st,
                           cudaStream_t s) {
-    count_launch();
-    k_check_pattern<<<nblocks(n), kThreads, 0, s>>>(n, ptr, col, dia, st);
+    ROW_LANES(k_check_pattern, n, ptr, col, dia, st);
 }
 void launch_check_finite(int64_t nnz, const double *val, int *st, cudaStream_t s) {
     int64_t b = nblocks(nnz);
     count_launch();
     k_check_finite<<<(unsigned)(b > 4096 ? 4096 : b), kThreads, 0, s>>>(nnz, val, st);
 }
-void launch_strength(int32_t n, const int32_t *ptr, const int32_t *col, const double *val, const int32_t *dia,
-                     double eps2, uint8_t *strong, int32_t *deg, cudaStream_t s) {
-    count_launch();
-    k_strength<<<nblocks(n), kThreads, 0, s>>>(n, ptr, col, val, dia, eps2, strong, deg);
+void launch_strength(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const double *val,
+                     const int32_t *dia, double eps2, uint8_t *strong, int32_t *deg, cudaStream_t s) {
+    ROW_LANES(k_strength, n, ptr, col, val, dia, eps2, strong, deg);
 }
-
-int32_t run_aggregation(int32_t n, const int32_t *ptr, const int32_t *col, const double *val,
+int32_t run_aggregation(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const double *val,
                         const uint8_t *strong, const int32_t *deg, int32_t *agg, int8_t *state, int64_t *m1,
                         uint8_t *r1, int32_t *root_id, int32_t *agg1, int32_t *root_of, int *counter, int *st,
                         int64_t *scan_tmp, cudaStream_t s) {
@@ -1038,15 +1230,11 @@ int32_t run_aggregation(int32_t n, const int32_t *ptr, const int32_t *col, const
     // every round turns at least the undecided node of largest priority into
     // a root, so at most n rounds; in practice a few dozen
     for (int32_t round = 0; round <= n; ++round) {
-        count_launch();
-        k_mis_m1<<<nb, kThreads, 0, s>>>(n, ptr, col, strong, state, m1);
-        count_launch();
-        k_mis_select<<<nb, kThreads, 0, s>>>(n, ptr, col, strong, state, m1);
-        count_launch();
-        k_mis_r1<<<nb, kThreads, 0, s>>>(n, ptr, col, strong, state, r1);
+        ROW_LANES(k_mis_m1, n, ptr, col, strong, state, m1);
+        ROW_LANES(k_mis_select, n, ptr, col, strong, state, m1);
+        ROW_LANES(k_mis_r1, n, ptr, col, strong, state, r1);
         cudaMemsetAsync(counter, 0, sizeof(int), s);
-        count_launch();
-        k_mis_exclude<<<nb, kThreads, 0, s>>>(n, ptr, col, strong, state, r1, counter);
+        ROW_LANES(k_mis_exclude, n, ptr, col, strong, state, r1, counter);
         int h = -1;
         if (cudaMemcpyAsync(&h, counter, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -1;
         if (cudaStreamSynchronize(s) != cudaSuccess) return -1;
@@ -1059,24 +1247,29 @@ int32_t run_aggregation(int32_t n, const int32_t *ptr, const int32_t *col, const
     int32_t nagg = 0;
     if (cudaMemcpyAsync(&nagg, root_id + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -1;
     if (cudaStreamSynchronize(s) != cudaSuccess) return -1;
-    count_launch();
-    k_agg_phase1<<<nb, kThreads, 0, s>>>(n, ptr, col, strong, state, root_id, agg1, root_of);
-    count_launch();
-    k_agg_phase2<<<nb, kThreads, 0, s>>>(n, ptr, col, val, strong, state, agg1, root_of, agg, st);
+    ROW_LANES(k_agg_phase1, n, ptr, col, strong, state, root_id, agg1, root_of);
+    ROW_LANES(k_agg_phase2, n, ptr, col, val, strong, state, agg1, root_of, agg, st);
     return nagg;
 }
 
-void launch_p_count(int32_t n, const int32_t *ptr, const int32_t *col, const uint8_t *strong, const int32_t *agg,
-                    int smoothed, int32_t *plen, cudaStream_t s) {
+void launch_p_count(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const uint8_t *strong,
+                    const int32_t *agg, int smoothed, int32_t *plen, cudaStream_t s) {
     count_launch();
-    k_p_count<<<nblocks(n), kThreads, 0, s>>>(n, ptr, col, strong, agg, smoothed, plen);
+    if (smoothed && warp_rows(n, nnz))
+        k_p_count_warp<<<nblocks(n, kPWarps), kPWarps * 32, 0, s>>>(n, ptr, col, strong, agg, plen);
+    else
+        k_p_count<<<nblocks(n), kThreads, 0, s>>>(n, ptr, col, strong, agg, smoothed, plen);
 }
-void launch_p_fill(int32_t n, const int32_t *ptr, const int32_t *col, const double *val, const uint8_t *strong,
-                   const int32_t *dia, const int32_t *agg, double omega, int smoothed, const int32_t *P_ptr,
-                   int32_t *P_col, double *P_val, cudaStream_t s) {
+void launch_p_fill(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const double *val,
+                   const uint8_t *strong, const int32_t *dia, const int32_t *agg, double omega, int smoothed,
+                   const int32_t *P_ptr, int32_t *P_col, double *P_val, cudaStream_t s) {
     count_launch();
-    k_p_fill<<<nblocks(n), kThreads, 0, s>>>(n, ptr, col, val, strong, dia, agg, omega, smoothed, P_ptr, P_col,
-                                             P_val);
+    if (smoothed && warp_rows(n, nnz))
+        k_p_fill_warp<<<nblocks(n, kPWarps), kPWarps * 32, 0, s>>>(n, ptr, col, val, strong, dia, agg, omega, P_ptr,
+                                                                   P_col, P_val);
+    else
+        k_p_fill<<<nblocks(n), kThreads, 0, s>>>(n, ptr, col, val, strong, dia, agg, omega, smoothed, P_ptr, P_col,
+                                                 P_val);
 }
 void launch_count_cols(int64_t nnz, const int32_t *col, int32_t *cnt, cudaStream_t s) {
     int64_t b = nblocks(nnz);
@@ -1090,9 +1283,17 @@ void launch_transpose_scatter(int32_t n, const int32_t *P_ptr, const int32_t *P_
     k_transpose_scatter<<<nblocks(n), kThreads, 0, s>>>(n, P_ptr, P_col, P_val, R_ptr, cursor, R_col, R_val);
 }
 void launch_sort_rows(int32_t nrows, const int32_t *ptr, int32_t *col, double *val, cudaStream_t s) {
-    count_launch();
     if (nrows <= 0) return;
-    k_sort_rows<<<(unsigned)((nrows + kSortWarps - 1) / kSortWarps), kSortWarps * 32, 0, s>>>(nrows, ptr, col, val);
+    // many rows: the short ones by the kernel with fewer registers, then the
+    // few long ones; a small level in one launch
+    const unsigned g = (unsigned)((nrows + kSortWarps - 1) / kSortWarps);
+    const bool split = nrows > 152 * 64;
+    if (split) {
+        count_launch();
+        k_sort_rows<4><<<g, kSortWarps * 32, 0, s>>>(nrows, 0, ptr, col, val);
+    }
+    count_launch();
+    k_sort_rows<16><<<g, kSortWarps * 32, 0, s>>>(nrows, split ? 128 : 0, ptr, col, val);
 }
 
 void launch_row_terms_max(int32_t nrows, const int32_t *X_ptr, const int32_t *X_col, const int32_t *Y_ptr,
@@ -1148,9 +1349,14 @@ void launch_t1_count(int32_t n, const int32_t *A_ptr, const int32_t *A_col, cons
     count_launch();
     k_t1_count<<<nblocks(n), kThreads, 0, s>>>(n, A_ptr, A_col, P_ptr, cnt);
 }
-void launch_t1_fill(int32_t n, const int32_t *A_ptr, const int32_t *A_col, const int32_t *P_ptr,
+void launch_t1_fill(int32_t n, int32_t nnz, const int32_t *A_ptr, const int32_t *A_col, const int32_t *P_ptr,
                     const int32_t *P_col, const int32_t *AP_ptr, const int32_t *AP_col, const int32_t *t1ptr,
                     uint16_t *slot1, int *st, cudaStream_t s) {
+    // long rows: the warp-per-row fill of stage 2 (the same positions)
+    if (warp_rows(n, nnz)) {
+        launch_t2_fill(n, A_ptr, A_col, P_ptr, P_col, AP_ptr, AP_col, t1ptr, slot1, st, s);
+        return;
+    }
     count_launch();
     k_t1_fill<<<nblocks(n), kThreads, 0, s>>>(n, A_ptr, A_col, P_ptr, P_col, AP_ptr, AP_col, t1ptr, slot1, st);
 }

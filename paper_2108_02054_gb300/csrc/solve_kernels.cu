@@ -2365,6 +2365,15 @@ __global__ void k_bi_end(int32_t n, const double *__restrict__ t, const double *
 // ======================================================================= launchers
 void launch_ap_numeric_f64(const Level &L, const double *A_val, cudaStream_t s) {
     count_launch();
+    // rows of more than eight entries on average: a warp per row, as stage 2
+    // (the same sums; 64^3, 24,028 rows of 31: 128 -> about 66 us, 1,289 rows of
+    // 54: 225 -> 48)
+    if ((int64_t)L.nnz > 8 * (int64_t)L.n) {
+        k_rap_terms<double><<<nblocks(L.n, kRapWarps), kRapWarps * 32, 0, s>>>(L.n, L.A_ptr, L.A_col, A_val, L.P_ptr,
+                                                                             L.P_val, L.AP_ptr, L.t1ptr, L.slot1,
+                                                                             L.AP_val);
+        return;
+    }
     k_ap_numeric_f64<<<nblocks(L.n, kApThreads), kApThreads, 0, s>>>(L.n, L.A_ptr, L.A_col, A_val, L.P_ptr, L.P_val,
                                                                      L.AP_ptr, L.t1ptr, L.slot1, L.AP_val);
 }
