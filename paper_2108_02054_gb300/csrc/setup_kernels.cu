@@ -170,37 +170,144 @@ __device__ __forceinline__ double cell_rho(const double *__restrict__ in, int64_
     return logd ? exp(x) : x;
 }
 
+// 2 / s, correctly rounded, in integer arithmetic (the FP64 division bounds the
+// assembly on this part), formed once while s stays the same: in a two-fluid
+// field all faces of a cell away from the interface have one sum
+struct TwoOver {
+    unsigned long long bits = 0ull;  // s = +0: an infinite quotient
+    double q = __builtin_huge_val();
+    __device__ __forceinline__ double operator()(double s) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(s);
+        if (b != bits) {
+            bits = b;
+            q = div_rn(2.0, div_recip(s));
+        }
+        return q;
+    }
+};
+
+// A cell's faces in ascending neighbour order: z-, y-, x-, x+, y+, z+
+struct CellFaces {
+    bool has[6];
+    __device__ __forceinline__ CellFaces(int dim, int N, int32_t x, int32_t y, int32_t z)
+        : has{dim == 3 && z > 0, y > 0, x > 0, x < N - 1, y < N - 1, dim == 3 && z < N - 1} {}
+    __device__ __forceinline__ int count() const { return has[0] + has[1] + has[2] + has[3] + has[4] + has[5]; }
+};
+
 // Row c: neighbours in ascending index order, off-diagonal -2/(rho_c + rho_nb),
 // diagonal = running sum of the face coefficients in that order, then the
 // ghost-cell Dirichlet term 2/rho_c on the top face.
-__global__ void k_poisson_vals(int dim, int N, int64_t n, int top, const double *__restrict__ rho, int logd,
-                               const int32_t *__restrict__ ptr, double *__restrict__ val) {
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    int64_t x, y, z;
-    cell_coords(dim, N, c, x, y, z);
-    const int64_t s2 = N, s3 = (int64_t)N * N;
-    int64_t nb[7];
-    int nnb = 0;
-    if (dim == 3 && z > 0) nb[nnb++] = c - s3;
-    if (y > 0) nb[nnb++] = c - s2;
-    if (x > 0) nb[nnb++] = c - 1;
-    nb[nnb++] = -1;
-    if (x < N - 1) nb[nnb++] = c + 1;
-    if (y < N - 1) nb[nnb++] = c + s2;
-    if (dim == 3 && z < N - 1) nb[nnb++] = c + s3;
-    const double rc = cell_rho(rho, c, logd);
+template <class R>
+__device__ __forceinline__ void poisson_row(const CellFaces &F, bool top, double rc, R rho_nb, double *out) {
+    TwoOver two;
     double diag = 0.0;
-    int32_t p = ptr[c], dpos = p;
-    for (int t = 0; t < nnb; ++t, ++p) {
-        if (nb[t] < 0) { dpos = p; continue; }
-        double k = 2.0 / (rc + cell_rho(rho, nb[t], logd));
-        diag = diag + k;
-        val[p] = -k;
+    int p = 0, dpos = 0;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        if (q == 3) dpos = p++;
+        if (F.has[q]) {
+            const double k = two(rc + rho_nb(q));
+            diag = diag + k;
+            out[p++] = -k;
+        }
     }
-    int is_top = dim == 2 ? (y == N - 1) : (z == N - 1);
-    if (top && is_top) diag = diag + 2.0 / rc;
-    val[dpos] = diag;
+    if (top) diag = diag + two(rc);
+    out[dpos] = diag;
+}
+
+// A warp's 32 consecutive rows are one contiguous range of values, written
+// through shared memory with whole-line stores (one row per thread stored 8
+// bytes of each line at a time).  192^3: 885 us with FP64 divisions and those
+// stores, 290 now; 64^3: 47 -> 18.
+constexpr int kAsmWarps = 8;
+template <class R>
+__device__ __forceinline__ void store_poisson_rows(const int32_t *__restrict__ ptr, double *__restrict__ val,
+                                                   double *buf, int64_t c, bool in, const CellFaces &F, bool top,
+                                                   double rc, R rho_nb) {
+    const int lane = threadIdx.x & 31;
+    const int len = in ? F.count() + 1 : 0;
+    int off = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, off, o);
+        if (lane >= o) off += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, off, 31);
+    off -= len;
+    if (in) poisson_row(F, top, rc, rho_nb, buf + off);
+    __syncwarp();
+    const int32_t p = in ? ptr[c] : 0, p0 = __shfl_sync(0xffffffffu, p, 0);
+    if (__all_sync(0xffffffffu, !in || p == p0 + off)) {
+        for (int e = lane; e < total; e += 32) val[p0 + e] = buf[e];
+    } else {  // rows with gaps between them
+        for (int e = 0; e < len; ++e) val[p + e] = buf[off + e];
+    }
+    __syncwarp();
+}
+
+__global__ void __launch_bounds__(kAsmWarps * 32)
+k_poisson_vals(int dim, int N, int64_t n, int top, const double *__restrict__ rho, int logd,
+               const int32_t *__restrict__ ptr, double *__restrict__ val) {
+    __shared__ double s_row[kAsmWarps][32 * 7];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, c0 = c - lane;
+    if (c0 >= n) return;  // warp-uniform
+    const bool in = c < n;
+    const int64_t cc = in ? c : c0;
+    int64_t x, y, z;
+    cell_coords(dim, N, cc, x, y, z);
+    const int64_t s3 = (int64_t)N * N;
+    const int64_t nb[6] = {cc - s3, cc - N, cc - 1, cc + 1, cc + N, cc + s3};
+    store_poisson_rows(ptr, val, s_row[w], cc, in, CellFaces(dim, N, (int32_t)x, (int32_t)y, (int32_t)z),
+                       top && (dim == 2 ? y : z) == N - 1, cell_rho(rho, cc, logd),
+                       [&](int q) { return cell_rho(rho, nb[q], logd); });
+}
+
+// The log-density forms march in z: a block takes 256 consecutive cells of a
+// plane through kLogPlanes planes, a cell's density exp(theta) kept in
+// registers for its own plane and the next, the plane's tile (with N cells on
+// either side for the y neighbours) in shared memory.  An FP64 exponential is
+// some 25 instructions of the slow pipe and a cell's seven densities bounded the
+// kernels; this forms about 1 + 2 N / 256 + 1/4 per cell.  Used while a tile
+// fits (kLogTile cells), else the direct kernels above and below.
+constexpr int kLogPlanes = 8, kLogTile = 4096;
+template <class Cell>
+__device__ __forceinline__ void march_log(int dim, int N, const double *__restrict__ theta, Cell cell) {
+    extern __shared__ double s_tile[];  // 256 + 2 N densities: cell t of the tile at t + N
+    const int64_t P = (int64_t)N * N;
+    const int64_t t0 = (int64_t)blockIdx.x * 256, t = t0 + threadIdx.x;  // in-plane index
+    const int nz = dim == 3 ? N : 1, z0 = blockIdx.y * kLogPlanes, z1 = min(nz, z0 + kLogPlanes);
+    const bool in = t < P;
+    const int32_t x = (int32_t)(t % N), y = (int32_t)(t / N);
+    double prev = in && z0 > 0 ? exp(theta[(z0 - 1) * P + t]) : 0.0;
+    double cur = in ? exp(theta[z0 * P + t]) : 0.0;
+    for (int z = z0; z < z1; ++z) {
+        const double *plane = theta + (int64_t)z * P;
+        const double next = in && z + 1 < nz ? exp(plane[P + t]) : 0.0;
+        s_tile[N + threadIdx.x] = cur;
+        for (int h = threadIdx.x; h < 2 * N; h += 256) {
+            const int64_t k = h < N ? t0 - N + h : t0 + 256 + (h - N);
+            s_tile[h < N ? h : 256 + h] = k >= 0 && k < P ? exp(plane[k]) : 0.0;
+        }
+        __syncthreads();
+        const double *me = s_tile + N + threadIdx.x;
+        const double nb[6] = {prev, me[-N], me[-1], me[1], me[N], next};
+        cell(in, (int64_t)z * P + t, CellFaces(dim, N, x, y, z), (dim == 2 ? y : z) == N - 1, cur, nb);
+        __syncthreads();
+        prev = cur;
+        cur = next;
+    }
+}
+
+__global__ void __launch_bounds__(256)
+k_poisson_vals_log(int dim, int N, int64_t n, int top, const double *__restrict__ theta,
+                   const int32_t *__restrict__ ptr, double *__restrict__ val) {
+    __shared__ double s_row[kAsmWarps][32 * 7];
+    march_log(dim, N, theta, [&](bool in, int64_t c, const CellFaces &F, bool is_top, double rc, const double(&nb)[6]) {
+        if (!__any_sync(0xffffffffu, in)) return;  // (a warp's cells in the plane are its first lanes)
+        store_poisson_rows(ptr, val, s_row[threadIdx.x >> 5], c, in, F, top && is_top, rc,
+                           [&](int q) { return nb[q]; });
+    });
 }
 
 // Level-set transport stand-in (Sec. 4, eq. 5): implicit upwind
@@ -243,33 +350,55 @@ __global__ void k_levelset_vals(int dim, int N, int64_t n, const double *__restr
 // of cell c contributes dL/dk_f * dk_f/dtheta_c with
 // dL/dk_f = -(lam_c - lam_j)(u_c - u_j), dk_f/dtheta_c = -2 rho_c/(rho_c + rho_j)^2;
 // the Dirichlet term contributes (-lam_c u_c) * (-2/rho_c).
+// (Faces in ascending neighbour order; rho_c / s^2 through the IEEE division.)
+template <class R>
+__device__ __forceinline__ double poisson_grad_cell(const CellFaces &F, bool top, int64_t c, const int64_t (&nb)[6],
+                                                    double rc, R rho_nb, const double *__restrict__ u,
+                                                    const double *__restrict__ lam) {
+    const double lc = lam[c], uc = u[c];
+    double g = 0.0;
+    // the last face's sum and its factor: formed again only when it changes
+    unsigned long long bits = 0ull;
+    double fac = 0.0;
+    bool have = false;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        if (!F.has[q]) continue;
+        const double dLdk = -(lc - lam[nb[q]]) * (uc - u[nb[q]]);
+        const double s = rc + rho_nb(q);
+        const unsigned long long b = (unsigned long long)__double_as_longlong(s);
+        if (!have || b != bits) {
+            have = true;
+            bits = b;
+            fac = div_rn(-2.0 * rc, div_recip(s * s));
+        }
+        g += dLdk * fac;
+    }
+    if (top) g += (-lc * uc) * div_rn(-2.0, div_recip(rc));
+    return g;
+}
 __global__ void k_poisson_grad(int dim, int N, int64_t n, int top, const double *__restrict__ rho, int logd,
                                const double *__restrict__ u, const double *__restrict__ lam,
                                double *__restrict__ grad) {
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n) return;
     int64_t x, y, z;
     cell_coords(dim, N, c, x, y, z);
-    const int64_t s2 = N, s3 = (int64_t)N * N;
-    int64_t nb[6];
-    int nnb = 0;
-    if (dim == 3 && z > 0) nb[nnb++] = c - s3;
-    if (y > 0) nb[nnb++] = c - s2;
-    if (x > 0) nb[nnb++] = c - 1;
-    if (x < N - 1) nb[nnb++] = c + 1;
-    if (y < N - 1) nb[nnb++] = c + s2;
-    if (dim == 3 && z < N - 1) nb[nnb++] = c + s3;
-    const double rc = cell_rho(rho, c, logd), lc = lam[c], uc = u[c];
-    double g = 0.0;
-    for (int t = 0; t < nnb; ++t) {
-        int64_t j = nb[t];
-        double dLdk = -(lc - lam[j]) * (uc - u[j]);
-        double s = rc + cell_rho(rho, j, logd);
-        g += dLdk * (-2.0 * rc / (s * s));
-    }
-    int is_top = dim == 2 ? (y == N - 1) : (z == N - 1);
-    if (top && is_top) g += (-lc * uc) * (-2.0 / rc);
-    grad[c] = g;
+    const int64_t s3 = (int64_t)N * N;
+    const int64_t nb[6] = {c - s3, c - N, c - 1, c + 1, c + N, c + s3};
+    grad[c] = poisson_grad_cell(CellFaces(dim, N, (int32_t)x, (int32_t)y, (int32_t)z),
+                                top && (dim == 2 ? y : z) == N - 1, c, nb, cell_rho(rho, c, logd),
+                                [&](int q) { return cell_rho(rho, nb[q], logd); }, u, lam);
+}
+__global__ void __launch_bounds__(256)
+k_poisson_grad_log(int dim, int N, int64_t n, int top, const double *__restrict__ theta,
+                   const double *__restrict__ u, const double *__restrict__ lam, double *__restrict__ grad) {
+    const int64_t s3 = (int64_t)N * N;
+    march_log(dim, N, theta, [&](bool in, int64_t c, const CellFaces &F, bool is_top, double rc, const double(&r)[6]) {
+        if (!in) return;
+        const int64_t nb[6] = {c - s3, c - N, c - 1, c + 1, c + N, c + s3};
+        grad[c] = poisson_grad_cell(F, top && is_top, c, nb, rc, [&](int q) { return r[q]; }, u, lam);
+    });
 }
 
 // ------------------------------------------------------------------ checks
@@ -1171,17 +1300,33 @@ void launch_poisson_cols(int dim, int N, const int32_t *ptr, int32_t *col, cudaS
     count_launch();
     k_poisson_cols<<<nblocks(n), kThreads, 0, s>>>(dim, N, n, ptr, col);
 }
+namespace {
+// the marching kernels' grid (tiles of a plane, chunks of planes), when a tile fits
+bool log_grid(int dim, int N, dim3 &g, size_t &smem) {
+    if (256 + 2 * N > kLogTile) return false;
+    const int64_t P = (int64_t)N * N;
+    g = dim3((unsigned)((P + 255) / 256), (unsigned)((dim == 3 ? N + kLogPlanes - 1 : kLogPlanes) / kLogPlanes));
+    smem = sizeof(double) * (size_t)(256 + 2 * N);
+    return g.y <= 65535;
+}
+}  // namespace
 void launch_poisson_vals(int dim, int N, int top, const double *rho, int logd, const int32_t *ptr, double *val,
                          cudaStream_t s) {
     int64_t n = dim == 2 ? (int64_t)N * N : (int64_t)N * N * N;
     count_launch();
-    k_poisson_vals<<<nblocks(n), kThreads, 0, s>>>(dim, N, n, top, rho, logd, ptr, val);
+    dim3 g;
+    size_t smem = 0;
+    if (logd && log_grid(dim, N, g, smem)) k_poisson_vals_log<<<g, 256, smem, s>>>(dim, N, n, top, rho, ptr, val);
+    else k_poisson_vals<<<nblocks(n, kAsmWarps * 32), kAsmWarps * 32, 0, s>>>(dim, N, n, top, rho, logd, ptr, val);
 }
 void launch_poisson_grad(int dim, int N, int top, const double *rho, int logd, const double *u, const double *lam,
                          double *grad, cudaStream_t s) {
     int64_t n = dim == 2 ? (int64_t)N * N : (int64_t)N * N * N;
     count_launch();
-    k_poisson_grad<<<nblocks(n), kThreads, 0, s>>>(dim, N, n, top, rho, logd, u, lam, grad);
+    dim3 g;
+    size_t smem = 0;
+    if (logd && log_grid(dim, N, g, smem)) k_poisson_grad_log<<<g, 256, smem, s>>>(dim, N, n, top, rho, u, lam, grad);
+    else k_poisson_grad<<<nblocks(n), kThreads, 0, s>>>(dim, N, n, top, rho, logd, u, lam, grad);
 }
 
 void launch_levelset_vals(int dim, int N, const double *fx, const double *fy, const double *fz, const int32_t *ptr,
