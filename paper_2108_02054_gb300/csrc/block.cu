@@ -198,7 +198,7 @@ __global__ void k_block_to_dense(int32_t n, const int32_t *__restrict__ ptr, con
 // the coarse ones the serial sum.  Measured at 48^3 per launch, one thread per
 // node -> per unknown, levels of 110,592 / 15,216 / 1,000 nodes: residual 32.9
 // / 30.5 / 36.4 -> 28.4 / 13.5 / 13.3 us, sweep 36.1 / 22.0 / 24.6 -> 31.3 /
-// 11.8 / 8.6, restriction 10.6 / 14.2 / 16.6 -> 10.1 / 9.1 / 9.0.
+// 11.8 / 8.6, restriction 10.6 / 14.2 / 16.6 -> 7.8 / 7.5 / 7.2.
 
 // first pre-smoothing step from u = 0: u = Minv f
 __global__ void __launch_bounds__(kBThreads)
@@ -236,10 +236,10 @@ k_block_residual(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__re
     r[t] = f[t] - block_dot<true>(ptr, col, bv, u, (int32_t)(t >> 2), (int)(t & 3));
 }
 
-// f_c = R r (scalar R, per component: fma from 0 in R's column order), four
+// f_c = R r (scalar R, per component: fma from 0 in R's column order), eight
 // entries' loads in flight; with minv also the coarse level's first smoothing
 // step from zero, u_c = Minv f_c
-__global__ void __launch_bounds__(kBThreads)
+__global__ void __launch_bounds__(kBThreads, 4)
 k_block_restrict(int32_t nc, const int32_t *__restrict__ Rptr, const int32_t *__restrict__ Rcol,
                  const double *__restrict__ Rval, const double *__restrict__ r, double *__restrict__ fc,
                  const double *__restrict__ minv, double *__restrict__ uc, const int *skip) {
@@ -250,18 +250,26 @@ k_block_restrict(int32_t nc, const int32_t *__restrict__ Rptr, const int32_t *__
     const int32_t I = (int32_t)(t >> 2), c = (int32_t)(t & 3);
     double s = 0.0;
     const int32_t p1 = Rptr[I + 1];
+    // the next batch's columns ahead; what the last batch lacks is loaded again
+    // and not summed (few warps run here: the latency of the loads bounds the
+    // kernel, not the FP64 slots of predicated-off sums)
     int32_t p = Rptr[I];
-    for (; p + 4 <= p1; p += 4) {
-        double w[4], v[4];
+    int32_t j[8];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            w[k] = Rval[p + k];
-            v[k] = r[(int64_t)4 * Rcol[p + k] + c];
+    for (int k = 0; k < 8; ++k) j[k] = p + k < p1 ? Rcol[p + k] : 0;
+    for (; p < p1; p += 8) {
+        double w[8], v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            w[k] = Rval[p + k < p1 ? p + k : p];
+            v[k] = r[(int64_t)4 * j[k] + c];
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) s = fma(w[k], v[k], s);
+        for (int k = 0; k < 8; ++k) j[k] = p + 8 + k < p1 ? Rcol[p + 8 + k] : 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (p + k < p1) s = fma(w[k], v[k], s);
     }
-    for (; p < p1; ++p) s = fma(Rval[p], r[(int64_t)4 * Rcol[p] + c], s);
     fc[t] = s;
     if (uc) uc[t] = quad_minv(minv, t, s, 0.0);
 }

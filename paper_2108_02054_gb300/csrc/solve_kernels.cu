@@ -21,6 +21,10 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kCgThreads = 512;
+// (the Krylov kernels with a matrix row in them are compiled for two such blocks
+// an SM: with the compiler's own choice of 32 registers it holds fewer of a
+// row's loads in flight; 192^3, q = A p 115.5 -> 108.8 us and the last sweep 61.0
+// -> 57.2, no change at 64^3)
 
 inline int nblocks(int64_t n, int t = kThreads) {
     int64_t b = (n + t - 1) / t;
@@ -297,6 +301,45 @@ __global__ void k_gather_apply<float>(int64_t nout, const int32_t *__restrict__ 
     y[e] = hi + lo;
 }
 
+// The same for launches of fewer outputs than fill the GPU (below kGatherDeep):
+// there an output's chain of up to hundreds of terms waits on one batch of
+// loads after the other, so sixteen terms' loads are in flight per thread (80
+// registers in FP64) and blocks are small.  64^3 (FP64), 3,383 / 70,122 / 21,771
+// outputs: 32.6 / 27.2 / 13.2 -> 16.1 / 20.0 / 10.3 us; at 378,840 outputs the
+// four of k_gather_apply are faster (27.8 against 29.5).
+constexpr int64_t kGatherDeep = 152 * 1024;
+__device__ __forceinline__ void gather_term(double &acc, double &, double w, double x) { acc = fma(w, x, acc); }
+__device__ __forceinline__ void gather_term(float &hi, float &lo, float w, float x) { df_acc(hi, lo, w, x); }
+template <class V, int U>
+__device__ __forceinline__ void gather_batch(V &hi, V &lo, int32_t t, const int32_t *__restrict__ idx,
+                                             const V *__restrict__ w, const V *__restrict__ x) {
+    int32_t ii[U];
+    V ww[U], xx[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+        ii[k] = idx[t + k];
+        ww[k] = w[t + k];
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k) xx[k] = x[ii[k]];
+#pragma unroll
+    for (int k = 0; k < U; ++k) gather_term(hi, lo, ww[k], xx[k]);
+}
+template <class V>
+__global__ void __launch_bounds__(64, 8)
+k_gather_apply_deep(int64_t nout, const int32_t *__restrict__ eptr, const int32_t *__restrict__ idx,
+                    const V *__restrict__ w, const V *__restrict__ x, V *__restrict__ y) {
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= nout) return;
+    V hi = V(0), lo = V(0);
+    const int32_t t1 = eptr[e + 1];
+    int32_t t = eptr[e];
+    for (; t + 16 <= t1; t += 16) gather_batch<V, 16>(hi, lo, t, idx, w, x);
+    for (; t + 4 <= t1; t += 4) gather_batch<V, 4>(hi, lo, t, idx, w, x);
+    for (; t < t1; ++t) gather_term(hi, lo, w[t], x[idx[t]]);
+    y[e] = sizeof(V) == 4 ? V(hi + lo) : hi;
+}
+
 // ------------------------------------------------------------------ smoothers
 // SPAI0: m_i = a_ii / sum_j a_ij^2 (fma, column order), 0 for a zero sum;
 // damped Jacobi: m_i = w / a_ii.
@@ -464,9 +507,10 @@ __global__ void k_cast_f32(int64_t n, const double *__restrict__ in, float *__re
 __global__ void k_csr_to_dense(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col,
                                const double *__restrict__ val, const float *__restrict__ valf,
                                double *__restrict__ dense) {
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    // a warp per row
+    const int32_t i = (int32_t)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (i >= n) return;
-    for (int32_t p = ptr[i]; p < ptr[i + 1]; ++p)
+    for (int32_t p = ptr[i] + (threadIdx.x & 31); p < ptr[i + 1]; p += 32)
         dense[(int64_t)i * n + col[p]] = val ? val[p] : (double)valf[p];
 }
 
@@ -1587,7 +1631,7 @@ __global__ void k_smooth_sweep(int32_t n, M A, const typename M::value *__restri
 __device__ double block_sum(double v);
 __device__ bool cg_reduce(double d, double *partial, unsigned *counter, double *total);
 template <class M, class TZ>
-__global__ void __launch_bounds__(kCgThreads)
+__global__ void __launch_bounds__(kCgThreads, 2)
 k_smooth_sweep_dot(int32_t n, M A, const typename M::value *__restrict__ m, const double *__restrict__ f,
                    const typename M::value *__restrict__ u_in, TZ *__restrict__ z, double *__restrict__ partial,
                    CgState *cg, const int *skip) {
@@ -1867,7 +1911,7 @@ __global__ void k_cg_set_rz_p(int32_t n, const TZ *__restrict__ z, double *__res
 
 // q = A p; the last block forms p.q and alpha = r.z / p.q (breakdown: p.q <= 0)
 template <class M>
-__global__ void __launch_bounds__(kCgThreads)
+__global__ void __launch_bounds__(kCgThreads, 2)
 k_spmv_dot(int32_t n, M A, const double *__restrict__ p, double *__restrict__ q, double *__restrict__ partial,
            CgState *cg) {
     __shared__ int32_t s_off[kMaxColOffsets];
@@ -2177,7 +2221,7 @@ __global__ void k_bi_p(int32_t n, const double *__restrict__ r, const double *__
 
 // v = A p^, (r^, v); alpha = rho / (r^, v)
 template <class M>
-__global__ void __launch_bounds__(kCgThreads)
+__global__ void __launch_bounds__(kCgThreads, 2)
 k_bi_spmv_rv(int32_t n, M A, const double *__restrict__ ph, double *__restrict__ v, const double *__restrict__ rh,
              double *__restrict__ partial, BiState *st) {
     __shared__ int32_t s_off[kMaxColOffsets];
@@ -2228,7 +2272,7 @@ __global__ void k_bi_s(int32_t n, const double *__restrict__ r, const double *__
 
 // t = A s^, (t, s), (t, t); omega = (t, s) / (t, t)
 template <class M>
-__global__ void __launch_bounds__(kCgThreads)
+__global__ void __launch_bounds__(kCgThreads, 2)
 k_bi_spmv_t(int32_t n, M A, const double *__restrict__ sh, const double *__restrict__ sv, double *__restrict__ t,
             double *__restrict__ partial, BiState *st) {
     __shared__ int32_t s_off[kMaxColOffsets];
@@ -2400,7 +2444,8 @@ void launch_gather_apply(int64_t nout, const int32_t *eptr, const int32_t *idx, 
                          cudaStream_t s) {
     if (nout <= 0) return;
     count_launch();
-    k_gather_apply<V><<<nblocks(nout), kThreads, 0, s>>>(nout, eptr, idx, w, x, y);
+    if (nout < kGatherDeep) k_gather_apply_deep<V><<<nblocks(nout, 64), 64, 0, s>>>(nout, eptr, idx, w, x, y);
+    else k_gather_apply<V><<<nblocks(nout), kThreads, 0, s>>>(nout, eptr, idx, w, x, y);
 }
 template void launch_gather_apply<double>(int64_t, const int32_t *, const int32_t *, const double *, const double *,
                                           double *, cudaStream_t);
@@ -2464,7 +2509,7 @@ void launch_csr_to_dense(int32_t n, const int32_t *ptr, const int32_t *col, cons
                          double *dense, cudaStream_t s) {
     cudaMemsetAsync(dense, 0, sizeof(double) * (size_t)n * (size_t)n, s);
     count_launch();
-    k_csr_to_dense<<<nblocks(n), kThreads, 0, s>>>(n, ptr, col, val, valf, dense);
+    k_csr_to_dense<<<nblocks((int64_t)n * 32), kThreads, 0, s>>>(n, ptr, col, val, valf, dense);
 }
 size_t lu_cluster_smem(int32_t n) {
     const size_t nloc = (size_t)(n + kLuClusterCtas - 1) / kLuClusterCtas;
