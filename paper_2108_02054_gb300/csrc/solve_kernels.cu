@@ -1628,7 +1628,6 @@ __global__ void k_smooth_sweep(int32_t n, M A, const typename M::value *__restri
 
 // the V-cycle's last finest-level sweep fused with the CG product r.z:
 // z = u_in + m o (r - A u_in) and a per-block partial of r.z (block_sum order)
-__device__ double block_sum(double v);
 __device__ bool cg_reduce(double d, double *partial, unsigned *counter, double *total);
 template <class M, class TZ>
 __global__ void __launch_bounds__(kCgThreads, 2)
@@ -1813,7 +1812,7 @@ __device__ double cg_sum_partials(const double *partial, int nblk) {
 }
 
 // publish this block's partial; the last block returns the total (thread 0)
-__device__ bool cg_reduce(double d, double *partial, unsigned *counter, double *total) {
+__device__ bool bi_reduce(double d, double *partial, unsigned *counter, double *total) {
     d = block_sum(d);
     if (threadIdx.x == 0) partial[blockIdx.x] = d;
     if (!cg_last_block(counter)) return false;
@@ -1825,24 +1824,90 @@ __device__ bool cg_reduce(double d, double *partial, unsigned *counter, double *
     return true;
 }
 
-// two sums at once, each with the arithmetic (and so the result) of cg_reduce
-__device__ bool cg_reduce2(double d1, double d2, double *part1, double *part2, unsigned *counter, double *t1,
-                           double *t2) {
-    d1 = block_sum(d1);
-    d2 = block_sum(d2);
+// The CG kernels' reductions (K sums at once).  A warp's FP64 instruction takes
+// its sub-partition's pipe for 64 cycles whatever its lanes do, so summing 16
+// warps' values by five shuffle steps each (block_sum) keeps the pipes busy for
+// 1,280 cycles a block, and two blocks share an SM.  Here 64 threads first add
+// eight values each from shared memory, then two warps run the shuffle steps,
+// and in the last block the same 64 threads sum the partials; the other warps
+// are done after one barrier.  64^3: q = A p 11.5 -> 10.8 us, r update 10.9
+// -> 9.8, last sweep 10.4 -> 9.6; the step 2.70 -> 2.60 ms.  (BiCGStab keeps its sums' order.)
+constexpr int kSumThreads = 64;
+__device__ __forceinline__ void sum_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kSumThreads) : "memory"); }
+// sums of 64 threads' values (threads 0 .. 63 call), valid in thread 0
+template <int K>
+__device__ __forceinline__ void sum64(double (&a)[K], double (*s_w)[2]) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < K; ++k) a[k] += __shfl_xor_sync(0xffffffffu, a[k], o);
+    if (threadIdx.x == 32)
+#pragma unroll
+        for (int k = 0; k < K; ++k) s_w[k][1] = a[k];
+    sum_sync();
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int k = 0; k < K; ++k) a[k] += s_w[k][1];
+}
+// publishes the block's K sums; true in thread 0 of the last block, with the totals
+template <int K>
+__device__ __forceinline__ bool cg_reduce(const double (&v)[K], double *const (&part)[K], unsigned *counter,
+                                          double (&total)[K]) {
+    __shared__ double s_v[K][kCgThreads];
+    __shared__ double s_w[K][2];
+    __shared__ int s_last;
+#pragma unroll
+    for (int k = 0; k < K; ++k) s_v[k][threadIdx.x] = v[k];
+    __syncthreads();
+    if (threadIdx.x >= kSumThreads) return false;
+    double a[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) a[k] = s_v[k][threadIdx.x];
+#pragma unroll
+    for (int j = kSumThreads; j < kCgThreads; j += kSumThreads)
+#pragma unroll
+        for (int k = 0; k < K; ++k) a[k] += s_v[k][threadIdx.x + j];
+    sum64<K>(a, s_w);
     if (threadIdx.x == 0) {
-        part1[blockIdx.x] = d1;
-        part2[blockIdx.x] = d2;
+#pragma unroll
+        for (int k = 0; k < K; ++k) part[k][blockIdx.x] = a[k];
+        __threadfence();
+        s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
     }
-    if (!cg_last_block(counter)) return false;
-    const double a = cg_sum_partials(part1, gridDim.x);
-    const double b = cg_sum_partials(part2, gridDim.x);
-    if (threadIdx.x == 0) {
-        *t1 = a;
-        *t2 = b;
-        *counter = 0u;
-    }
+    sum_sync();
+    if (!s_last) return false;
+#pragma unroll
+    for (int k = 0; k < K; ++k) a[k] = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += kSumThreads)
+#pragma unroll
+        for (int k = 0; k < K; ++k) a[k] += __ldcg(part[k] + b);
+    sum64<K>(a, s_w);
+    if (threadIdx.x != 0) return false;
+#pragma unroll
+    for (int k = 0; k < K; ++k) total[k] = a[k];
+    *counter = 0u;
     return true;
+}
+__device__ __forceinline__ bool cg_reduce(double d, double *partial, unsigned *counter, double *total) {
+    const double v[1] = {d};
+    double *const part[1] = {partial};
+    double t[1];
+    const bool last = cg_reduce<1>(v, part, counter, t);
+    if (last) *total = t[0];
+    return last;
+}
+// two sums at once
+__device__ __forceinline__ bool cg_reduce2(double d1, double d2, double *part1, double *part2, unsigned *counter,
+                                           double *t1, double *t2) {
+    const double v[2] = {d1, d2};
+    double *const part[2] = {part1, part2};
+    double t[2];
+    const bool last = cg_reduce<2>(v, part, counter, t);
+    if (last) {
+        *t1 = t[0];
+        *t2 = t[1];
+    }
+    return last;
 }
 
 __device__ __forceinline__ void put_smooth0(const Smooth0Out &z0, int32_t i, double ri) {
@@ -2185,7 +2250,7 @@ __global__ void k_bi_init(int32_t n, const double *__restrict__ f, double *__res
         s = fma(fi, fi, s);
     }
     double ff = 0.0;
-    if (cg_reduce(s, partial, &st->ctr[BI_CTR_INIT], &ff) && threadIdx.x == 0) {
+    if (bi_reduce(s, partial, &st->ctr[BI_CTR_INIT], &ff) && threadIdx.x == 0) {
         st->nf = sqrt(ff);
         st->tol = tol;
         st->maxiter = maxiter;
@@ -2235,7 +2300,7 @@ k_bi_spmv_rv(int32_t n, M A, const double *__restrict__ ph, double *__restrict__
         d = fma(rh[i], s, d);
     }
     double rv = 0.0;
-    if (cg_reduce(d, partial, &st->ctr[BI_CTR_RV], &rv) && threadIdx.x == 0) {
+    if (bi_reduce(d, partial, &st->ctr[BI_CTR_RV], &rv) && threadIdx.x == 0) {
         st->rv = rv;
         if (!(rv != 0.0) || !isfinite(rv)) {
             st->status = AMG_ERR_BREAKDOWN;
@@ -2262,7 +2327,7 @@ __global__ void k_bi_s(int32_t n, const double *__restrict__ r, const double *__
         d = fma(si, si, d);
     }
     double ss = 0.0;
-    if (cg_reduce(d, partial, &st->ctr[BI_CTR_SS], &ss) && threadIdx.x == 0) {
+    if (bi_reduce(d, partial, &st->ctr[BI_CTR_SS], &ss) && threadIdx.x == 0) {
         st->sres = sqrt(ss) / st->nf;
         st->half = st->sres <= st->tol;
         st->need_true = st->half;
@@ -2352,7 +2417,7 @@ k_bi_true(int32_t n, M A, const double *__restrict__ f, const double *__restrict
         d = fma(ti, ti, d);
     }
     double tt = 0.0;
-    if (cg_reduce(d, partial, &st->ctr[BI_CTR_TRUE], &tt) && threadIdx.x == 0) {
+    if (bi_reduce(d, partial, &st->ctr[BI_CTR_TRUE], &tt) && threadIdx.x == 0) {
         st->tres = st->nf > 0.0 ? sqrt(tt) / st->nf : 0.0;
         if (!force) {
             if (st->tres <= st->tol) {
@@ -2387,7 +2452,7 @@ __global__ void k_bi_end(int32_t n, const double *__restrict__ t, const double *
             d = fma(rh[i], ti, d);
         }
         double rho = 0.0;
-        if (!cg_reduce(d, partial, &st->ctr[BI_CTR_RHO], &rho) || threadIdx.x != 0) return;
+        if (!bi_reduce(d, partial, &st->ctr[BI_CTR_RHO], &rho) || threadIdx.x != 0) return;
         st->rho_next = rho;
     } else if (blockIdx.x != 0 || threadIdx.x != 0) {
         return;
