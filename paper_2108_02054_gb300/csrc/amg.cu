@@ -76,6 +76,7 @@ struct amg_ctx {
     Level lev[kMaxLevels];
     int32_t nL = 0;
     double *lu = nullptr, *inv = nullptr, *luT = nullptr;
+    double *coarse_w = nullptr;  // A_L^-1 R, where it is small enough to solve with
     int32_t *piv = nullptr;
     bool have_setup = false;
     // system matrix of the solve (aliases level 0 except under full reuse)
@@ -209,7 +210,7 @@ void free_hierarchy(amg_ctx *ctx) {
     for (int l = 0; l < kMaxLevels; ++l) ctx->lev[l] = Level{};
     ctx->nlev = 0;
     ctx->have_setup = false;
-    ctx->lu = ctx->inv = ctx->luT = nullptr;
+    ctx->lu = ctx->inv = ctx->luT = ctx->coarse_w = nullptr;
     ctx->piv = nullptr;
     ctx->graph_valid = false;
     ctx->a_val_stale = false;
@@ -374,6 +375,7 @@ amg_status coarse_factor(amg_ctx *ctx) {
     launch_csr_to_dense(C.n, C.A_ptr, C.A_col, mx ? nullptr : C.A_val, mx ? C.A_valf : nullptr, ctx->lu, ctx->s);
     { ProfScope ps_(ctx, AMG_PROF_LU, true); launch_dense_lu(C.n, ctx->lu, ctx->piv, ctx->d_st, ctx->s, ctx->luT); }
     { ProfScope ps_(ctx, AMG_PROF_INV, true); launch_lu_inverse(C.n, ctx->lu, ctx->piv, ctx->inv, ctx->s, ctx->luT); }
+    if (ctx->coarse_w) launch_coarse_w(ctx->lev[ctx->nlev - 2], ctx->nL, ctx->inv, ctx->coarse_w, ctx->s);
     return AMG_OK;
 }
 
@@ -729,6 +731,8 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
     TRY(alloc(ctx, &ctx->piv, (size_t)nL));
     ctx->luT = nullptr;
     if (lu_wants_transpose((int32_t)nL)) TRY(alloc(ctx, &ctx->luT, (size_t)(nL * nL)));
+    if (!blockmode(ctx) && ctx->nlev > 1 && nL * ctx->lev[ctx->nlev - 2].n <= kCoarseWMax)
+        TRY(alloc(ctx, &ctx->coarse_w, (size_t)(nL * ctx->lev[ctx->nlev - 2].n)));
     if (mixed(ctx))
         for (int l = 1; l < ctx->nlev; ++l) {
             const Level &L = ctx->lev[l];
@@ -1030,8 +1034,10 @@ void enqueue_vcycle(amg_ctx *ctx, const double *r, TZ *z, const int *skip, doubl
     auto m_of = [&](int l) -> const V * { return (pre && l < nl - 1) ? Vops<V>::m(ctx->lev[l]) : nullptr; };
     auto u_of = [&](int l) -> V * { return (pre && l < nl - 1) ? Vops<V>::vec(ctx->lev[l]).u : nullptr; };
     V *cur[kMaxLevels];
+    // the restriction into the coarsest level comes with its solve (coarse_w)
+    const bool direct = ctx->coarse_w != nullptr;
     cur[0] = down_level<V, double>(ctx, 0, r, skip, u0_ready);
-    {
+    if (!(direct && nl == 2)) {
         ProfScope ps_(ctx, AMG_PROF_RESTRICT_L0);
         launch_restrict<V>(ctx->lev[0], Vops<V>::R(ctx->lev[0]), Vops<V>::vec(ctx->lev[0]).r,
                            Vops<V>::vec(ctx->lev[1]).f, m_of(1), u_of(1), skip, ctx->s);
@@ -1039,11 +1045,19 @@ void enqueue_vcycle(amg_ctx *ctx, const double *r, TZ *z, const int *skip, doubl
     for (int l = 1; l < nl - 1; ++l) {
         Level &L = ctx->lev[l];
         cur[l] = down_level<V, V>(ctx, l, Vops<V>::vec(L).f, skip, pre);
+        if (direct && l == nl - 2) break;
         launch_restrict<V>(L, Vops<V>::R(L), Vops<V>::vec(L).r, Vops<V>::vec(ctx->lev[l + 1]).f, m_of(l + 1),
                            u_of(l + 1), skip, ctx->s);
     }
     Level &Cst = ctx->lev[nl - 1];
-    { ProfScope ps_(ctx, AMG_PROF_COARSE, true); launch_coarse_solve<V, V, V>(Cst.n, ctx->inv, Vops<V>::vec(Cst).f, Vops<V>::vec(Cst).u, skip, ctx->s); }
+    {
+        ProfScope ps_(ctx, AMG_PROF_COARSE, true);
+        if (direct)
+            launch_coarse_from_residual<V>(ctx->lev[nl - 2].n, Cst.n, ctx->coarse_w, Vops<V>::vec(ctx->lev[nl - 2]).r,
+                                           Vops<V>::vec(Cst).u, skip, ctx->s);
+        else
+            launch_coarse_solve<V, V, V>(Cst.n, ctx->inv, Vops<V>::vec(Cst).f, Vops<V>::vec(Cst).u, skip, ctx->s);
+    }
     cur[nl - 1] = Vops<V>::vec(Cst).u;
     for (int l = nl - 2; l >= 1; --l) {
         Level &L = ctx->lev[l];

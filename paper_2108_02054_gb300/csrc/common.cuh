@@ -386,6 +386,13 @@ void launch_correct_sweep(const Level &L, const V *Pval, const V *APval, const V
                           const int *skip, cudaStream_t s);
 template <class V, class TF, class TO>
 void launch_coarse_solve(int32_t n, const double *inv, const TF *f, TO *u, const int *skip, cudaStream_t s);
+// the coarsest solve from the residual of the level above, u = W r, W = A_L^-1 R
+// (n_L x n, from that level's P and the explicit inverse)
+constexpr int64_t kCoarseWMax = 1 << 19;
+void launch_coarse_w(const Level &L, int32_t nL, const double *inv, double *W, cudaStream_t s);
+template <class V>
+void launch_coarse_from_residual(int32_t n, int32_t nL, const double *W, const V *r, V *u, const int *skip,
+                                 cudaStream_t s);
 template <class TI, class TO>
 void launch_copy_cast(int64_t n, const TI *in, TO *out, const int *skip, cudaStream_t s);
 

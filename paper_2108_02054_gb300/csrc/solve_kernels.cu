@@ -1505,6 +1505,57 @@ __global__ void k_coarse_solve(int32_t n, const double *__restrict__ inv, const 
     if (lane == 0) u[r] = (TO)s;
 }
 
+// The coarsest solve straight from the residual of the level above: with
+// W = A_L^-1 R (dense, n_L x n, formed at each refactorisation) it is u_L = W r,
+// one launch instead of the restriction and the solve, one block per coarse row.
+// Used while W is small (kCoarseWMax): its n_L n products replace latency, not
+// work.  FP64, 87 x 1,294 (64^3): 4.7 + 3.4 -> 3.7 us, and 6 us to form W; at
+// 255 x 4,151 4.5 + 4.6 -> 7.8 and 18, slower over a solve of 9 iterations.
+constexpr int kWThreads = 256;
+__global__ void k_coarse_w(int32_t n, int32_t nL, const int32_t *__restrict__ P_ptr, const int32_t *__restrict__ P_col,
+                           const double *__restrict__ P_val, const float *__restrict__ P_valf,
+                           const double *__restrict__ inv, double *__restrict__ W) {
+    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x, I = blockIdx.y;
+    if (i >= n) return;
+    double s = 0.0;  // R = P^T: column i of R is row i of P
+    for (int32_t p = P_ptr[i]; p < P_ptr[i + 1]; ++p)
+        s = fma(inv[(int64_t)I * nL + P_col[p]], P_valf ? (double)P_valf[p] : P_val[p], s);
+    W[(int64_t)I * n + i] = s;
+}
+template <class V>
+__global__ void __launch_bounds__(kWThreads)
+k_coarse_from_residual(int32_t n, const double *__restrict__ W, const V *__restrict__ r, V *__restrict__ u,
+                       const int *skip) {
+    __shared__ double s_v[kWThreads / 32];
+    pdl_wait();
+    if (skipped(skip)) return;
+    const double *__restrict__ w = W + (int64_t)blockIdx.x * n;
+    double s = 0.0, t = 0.0;  // two chains, four entries' loads in flight
+    int32_t i = threadIdx.x;
+    for (; i + 3 * kWThreads < n; i += 4 * kWThreads) {
+        const double a = w[i], b = w[i + kWThreads], c = w[i + 2 * kWThreads], d = w[i + 3 * kWThreads];
+        const V x = r[i], y = r[i + kWThreads], z = r[i + 2 * kWThreads], q = r[i + 3 * kWThreads];
+        s = fma(a, (double)x, s);
+        t = fma(b, (double)y, t);
+        s = fma(c, (double)z, s);
+        t = fma(d, (double)q, t);
+    }
+    for (; i < n; i += kWThreads) s = fma(w[i], (double)r[i], s);
+    s = warp_sum(s + t);
+    if ((threadIdx.x & 31) == 0) s_v[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v[kWThreads / 32];
+#pragma unroll
+        for (int k = 0; k < kWThreads / 32; ++k) v[k] = s_v[k];
+#pragma unroll
+        for (int o = kWThreads / 64; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < o; ++k) v[k] += v[k + o];
+        u[blockIdx.x] = (V)v[0];
+    }
+}
+
 // ------------------------------------------------------------------ V-cycle pieces
 // Every matrix-vector piece takes the matrix as a row policy:
 //  - CsrRows: LPR lanes per row (a power of two <= 32, chosen per level from
@@ -2757,6 +2808,21 @@ void launch_coarse_solve(int32_t n, const double *inv, const TF *f, TO *u, const
     count_launch();
     launch_pdl(k_coarse_solve<TF, TO>, nblocks((int64_t)n * 32, 128), 128, 0, s, n, inv, f, u, skip);
 }
+void launch_coarse_w(const Level &L, int32_t nL, const double *inv, double *W, cudaStream_t s) {
+    count_launch();
+    k_coarse_w<<<dim3((unsigned)nblocks(L.n), (unsigned)nL), kThreads, 0, s>>>(L.n, nL, L.P_ptr, L.P_col, L.P_val,
+                                                                              L.P_valf, inv, W);
+}
+template <class V>
+void launch_coarse_from_residual(int32_t n, int32_t nL, const double *W, const V *r, V *u, const int *skip,
+                                 cudaStream_t s) {
+    count_launch();
+    launch_pdl(k_coarse_from_residual<V>, (unsigned)nL, kWThreads, 0, s, n, W, r, u, skip);
+}
+template void launch_coarse_from_residual<double>(int32_t, int32_t, const double *, const double *, double *,
+                                                  const int *, cudaStream_t);
+template void launch_coarse_from_residual<float>(int32_t, int32_t, const double *, const float *, float *, const int *,
+                                                 cudaStream_t);
 template <class TI, class TO>
 void launch_copy_cast(int64_t n, const TI *in, TO *out, const int *skip, cudaStream_t s) {
     int64_t b = nblocks(n);
