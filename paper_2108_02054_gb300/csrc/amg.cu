@@ -50,6 +50,7 @@ struct FineChunks {
     const cudaEvent_t *ev;  // kHostChunks events on the copy stream
 };
 
+constexpr int kReadBack = 8;
 struct amg_ctx {
     amg_params prm{};
     cudaStream_t s = nullptr;
@@ -97,6 +98,7 @@ struct amg_ctx {
     BiState *h_bi = nullptr;  // pinned
     int *d_st = nullptr;
     int *h_st = nullptr;      // pinned
+    int32_t *h_rb = nullptr;  // pinned: sizes read back by the full setup (kReadBack)
     // host-buffer staging
     double *stage_val = nullptr, *stage_f = nullptr, *stage_u = nullptr;
     ProfData prof;
@@ -241,10 +243,19 @@ amg_status reset_status(amg_ctx *ctx) {
     return AMG_OK;
 }
 
-template <class T>
-amg_status read_scalar(amg_ctx *ctx, const T *d, T *h) {
-    CK(cudaMemcpyAsync(h, d, sizeof(T), cudaMemcpyDeviceToHost, ctx->s));
-    CK(cudaStreamSynchronize(ctx->s));
+// several counts and the device status in one synchronisation (an error in the
+// status comes before any use of the counts)
+struct ReadBack {
+    const int32_t *d;
+    int32_t *h;
+};
+amg_status read_back(amg_ctx *ctx, const char *where, std::initializer_list<ReadBack> list) {
+    int k = 0;
+    for (const ReadBack &r : list)
+        CK(cudaMemcpyAsync(ctx->h_rb + k++, r.d, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->s));
+    TRY(check_device(ctx, where));
+    k = 0;
+    for (const ReadBack &r : list) *r.h = ctx->h_rb[k++];
     return AMG_OK;
 }
 
@@ -288,8 +299,8 @@ amg_status alloc_level_vectors(amg_ctx *ctx, Level &L) {
     return AMG_OK;
 }
 
-// symbolic C = X*Y (pattern only), allocating C's arrays
-amg_status symbolic_product(amg_ctx *ctx, int32_t nrows, int32_t ncols, const int32_t *X_ptr, const int32_t *X_col,
+// symbolic C = X*Y (pattern only), allocating C's arrays (X_nnz entries in X)
+amg_status symbolic_product(amg_ctx *ctx, int32_t nrows, int32_t ncols, int32_t X_nnz, const int32_t *X_ptr, const int32_t *X_col,
                             const int32_t *Y_ptr, const int32_t *Y_col, int add_diag, int32_t **C_ptr,
                             int32_t **C_col, int32_t *C_nnz) {
     int32_t *len = nullptr;
@@ -301,32 +312,18 @@ amg_status symbolic_product(amg_ctx *ctx, int32_t nrows, int32_t ncols, const in
     CK(cudaMemsetAsync(d_max, 0, sizeof(int), ctx->s));
     launch_row_terms_max(nrows, X_ptr, X_col, Y_ptr, add_diag, d_max, ctx->s);
     int32_t max_terms = 0;
-    TRY(read_scalar(ctx, d_max, &max_terms));
+    TRY(read_back(ctx, "symbolic product", {{d_max, &max_terms}}));
     const int cap = spgemm_symbolic_cap(max_terms);
     // lanes per row from X's average row length (its entries are spread over the lanes)
-    int32_t xnnz = 0;
-    TRY(read_scalar(ctx, X_ptr + nrows, &xnnz));
-    const double avg = nrows > 0 ? (double)xnnz / (double)nrows : 0.0;
+    const double avg = nrows > 0 ? (double)X_nnz / (double)nrows : 0.0;
     const int lanes = avg <= 8.0 ? 8 : avg <= 16.0 ? 16 : 32;
     launch_spgemm_symbolic(nrows, ncols, X_ptr, X_col, Y_ptr, Y_col, add_diag, cap, lanes, len, nullptr, nullptr,
                            ctx->d_st, ctx->s);
     TRY(scan(ctx, len, *C_ptr, nrows));
-    TRY(check_device(ctx, "symbolic product"));
-    TRY(read_scalar(ctx, *C_ptr + nrows, C_nnz));
+    TRY(read_back(ctx, "symbolic product", {{*C_ptr + nrows, C_nnz}}));
     TRY(alloc(ctx, C_col, (size_t)*C_nnz));
     launch_spgemm_symbolic(nrows, ncols, X_ptr, X_col, Y_ptr, Y_col, add_diag, cap, lanes, len, *C_ptr, *C_col,
                            ctx->d_st, ctx->s);
-    return AMG_OK;
-}
-
-amg_status max_row(amg_ctx *ctx, int32_t n, const int32_t *ptr, int32_t *out) {
-    int *d = nullptr;
-    TRY(alloc(ctx, &d, 1));
-    CK(cudaMemsetAsync(d, 0, sizeof(int), ctx->s));
-    launch_row_maxlen(n, ptr, d, ctx->s);
-    int h = 0;
-    TRY(read_scalar(ctx, d, &h));
-    *out = h;
     return AMG_OK;
 }
 
@@ -620,13 +617,13 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         TRY(alloc(ctx, &scan_tmp, (size_t)scan_tmp_elems(L.n)));
         launch_strength(L.n, L.nnz, L.A_ptr, L.A_col, L.A_val, L.dia, theta * theta, L.strong, deg, ctx->s);
         int32_t nagg = run_aggregation(L.n, L.nnz, L.A_ptr, L.A_col, L.A_val, L.strong, deg, L.agg, state, m1, r1, root_id,
-                                       agg1, root_of, counter, ctx->d_st, scan_tmp, ctx->s);
+                                       agg1, root_of, counter, ctx->d_st, scan_tmp, ctx->h_rb, ctx->s);
         if (nagg < 0) {
             CK(cudaGetLastError());
             return set_err(ctx, AMG_ERR_CUDA, "aggregation did not complete");
         }
-        TRY(check_device(ctx, "aggregation"));
         if (nagg == 0 || nagg >= L.n) {
+            TRY(check_device(ctx, "aggregation"));
             // coarsening stalls: this level becomes the coarsest
             CK(cudaMemsetAsync(L.agg, 0xff, sizeof(int32_t) * (size_t)L.n, ctx->s));
             CK(cudaMemsetAsync(L.strong, 0, (size_t)L.nnz, ctx->s));
@@ -639,7 +636,7 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         TRY(alloc(ctx, &L.P_ptr, (size_t)L.n + 1));
         launch_p_count(L.n, L.nnz, L.A_ptr, L.A_col, L.strong, L.agg, p.smoothed, plen, ctx->s);
         TRY(scan(ctx, plen, L.P_ptr, L.n));
-        TRY(read_scalar(ctx, L.P_ptr + L.n, &L.nnzP));
+        TRY(read_back(ctx, "aggregation", {{L.P_ptr + L.n, &L.nnzP}}));
         TRY(alloc(ctx, &L.P_col, (size_t)L.nnzP));
         TRY(alloc(ctx, &L.P_val, (size_t)L.nnzP));
         launch_p_fill(L.n, L.nnz, L.A_ptr, L.A_col, L.A_val, L.strong, L.dia, L.agg, p.omega, p.smoothed, L.P_ptr, L.P_col,
@@ -660,39 +657,40 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         launch_sort_rows(nagg, L.R_ptr, L.R_col, L.R_val, ctx->s);
         L.lpr_r = choose_lpr(nagg, L.nnzR);
         // symbolic Galerkin product: AP = A*P, A_c = R*AP (+ diagonal)
-        TRY(symbolic_product(ctx, L.n, nagg, L.A_ptr, L.A_col, L.P_ptr, L.P_col, 0, &L.AP_ptr, &L.AP_col,
+        TRY(symbolic_product(ctx, L.n, nagg, L.nnz, L.A_ptr, L.A_col, L.P_ptr, L.P_col, 0, &L.AP_ptr, &L.AP_col,
                              &L.nnzAP));
         TRY(alloc(ctx, &L.AP_val, (size_t)L.nnzAP));
         L.lpr_ap = choose_lpr_ap(L.n, L.nnzAP);
         Level &C = ctx->lev[ctx->nlev];
         C.n = nagg;
-        TRY(symbolic_product(ctx, nagg, nagg, L.R_ptr, L.R_col, L.AP_ptr, L.AP_col, 1, &C.A_ptr, &C.A_col, &C.nnz));
+        TRY(symbolic_product(ctx, nagg, nagg, L.nnzR, L.R_ptr, L.R_col, L.AP_ptr, L.AP_col, 1, &C.A_ptr, &C.A_col, &C.nnz));
         TRY(alloc(ctx, &C.A_val, (size_t)C.nnz));
         TRY(alloc(ctx, &C.dia, (size_t)C.n));
         launch_check_pattern(C.n, C.nnz, C.A_ptr, C.A_col, C.dia, ctx->d_st, ctx->s);
-        TRY(max_row(ctx, L.n, L.AP_ptr, &L.max_ap_row));
-        TRY(max_row(ctx, C.n, C.A_ptr, &L.max_ac_row));
-        if (L.max_ap_row > 65535 || L.max_ac_row > 65535)
-            return set_err(ctx, AMG_ERR_CAPACITY, "Galerkin row longer than 65535 entries");
-        // gather metadata: slot of every term of the two numeric stages
-        int32_t *tc = nullptr;
+        // gather metadata: slot of every term of the two numeric stages; the
+        // longest rows and the term counts come back together
+        int32_t *tc = nullptr, *d_max = nullptr;
         TRY(alloc(ctx, &tc, (size_t)std::max(L.n, nagg)));
+        TRY(alloc(ctx, &d_max, 2));
+        CK(cudaMemsetAsync(d_max, 0, 2 * sizeof(int32_t), ctx->s));
+        launch_row_maxlen(L.n, L.AP_ptr, d_max, ctx->s);
+        launch_row_maxlen(C.n, C.A_ptr, d_max + 1, ctx->s);
         TRY(alloc(ctx, &L.t1ptr, (size_t)L.n + 1));
         launch_t1_count(L.n, L.A_ptr, L.A_col, L.P_ptr, tc, ctx->s);
         TRY(scan(ctx, tc, L.t1ptr, L.n));
-        int32_t nt1 = 0, nt2 = 0;
-        TRY(check_device(ctx, "term count"));
-        TRY(read_scalar(ctx, L.t1ptr + L.n, &nt1));
-        L.nt1 = nt1;
-        TRY(alloc(ctx, &L.slot1, (size_t)nt1));
-        launch_t1_fill(L.n, L.nnz, L.A_ptr, L.A_col, L.P_ptr, L.P_col, L.AP_ptr, L.AP_col, L.t1ptr, L.slot1, ctx->d_st,
-                       ctx->s);
         TRY(alloc(ctx, &L.t2ptr, (size_t)nagg + 1));
         launch_t2_count(nagg, L.R_ptr, L.R_col, L.AP_ptr, tc, ctx->s);
         TRY(scan(ctx, tc, L.t2ptr, nagg));
-        TRY(check_device(ctx, "term count"));
-        TRY(read_scalar(ctx, L.t2ptr + nagg, &nt2));
+        int32_t nt1 = 0, nt2 = 0;
+        TRY(read_back(ctx, "term count", {{d_max, &L.max_ap_row}, {d_max + 1, &L.max_ac_row}, {L.t1ptr + L.n, &nt1},
+                                          {L.t2ptr + nagg, &nt2}}));
+        if (L.max_ap_row > 65535 || L.max_ac_row > 65535)
+            return set_err(ctx, AMG_ERR_CAPACITY, "Galerkin row longer than 65535 entries");
+        L.nt1 = nt1;
         L.nt2 = nt2;
+        TRY(alloc(ctx, &L.slot1, (size_t)nt1));
+        launch_t1_fill(L.n, L.nnz, L.A_ptr, L.A_col, L.P_ptr, L.P_col, L.AP_ptr, L.AP_col, L.t1ptr, L.slot1, ctx->d_st,
+                       ctx->s);
         TRY(alloc(ctx, &L.slot2, (size_t)nt2));
         launch_t2_fill(nagg, L.R_ptr, L.R_col, L.AP_ptr, L.AP_col, C.A_ptr, C.A_col, L.t2ptr, L.slot2, ctx->d_st,
                        ctx->s);
@@ -1657,6 +1655,7 @@ amg_status amg_create(amg_ctx **out, const amg_params *prm, void *cuda_stream) {
         cudaMallocHost(&ctx->h_cg, sizeof(CgState)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_bi, sizeof(BiState)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_st, sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&ctx->h_rb, sizeof(int32_t) * kReadBack) != cudaSuccess ||
         cudaMalloc(&ctx->d_st, sizeof(int)) != cudaSuccess) {
         amg_destroy(ctx);
         return AMG_ERR_CUDA;
@@ -1695,6 +1694,7 @@ void amg_destroy(amg_ctx *ctx) {
     if (ctx->h_cg) cudaFreeHost(ctx->h_cg);
     if (ctx->h_bi) cudaFreeHost(ctx->h_bi);
     if (ctx->h_st) cudaFreeHost(ctx->h_st);
+    if (ctx->h_rb) cudaFreeHost(ctx->h_rb);
     if (ctx->d_st) cudaFree(ctx->d_st);
     delete ctx;
 }

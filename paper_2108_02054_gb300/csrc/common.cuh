@@ -271,11 +271,12 @@ void launch_check_pattern(int32_t n, int32_t nnz, const int32_t *ptr, const int3
 void launch_check_finite(int64_t nnz, const double *val, int *st, cudaStream_t s);
 void launch_strength(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const double *val, const int32_t *dia,
                      double eps2, uint8_t *strong, int32_t *deg, cudaStream_t s);
-// aggregation; returns the number of aggregates (host sync inside), or -1 on error
+// aggregation; returns the number of aggregates (host sync inside), or -1 on
+// error (h_pin: one pinned int for the counts read back)
 int32_t run_aggregation(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const double *val,
                         const uint8_t *strong, const int32_t *deg, int32_t *agg, int8_t *state, int64_t *m1,
                         uint8_t *r1, int32_t *root_id, int32_t *agg1, int32_t *root_of, int *counter, int *st,
-                        int64_t *scan_tmp, cudaStream_t s);
+                        int64_t *scan_tmp, int32_t *h_pin, cudaStream_t s);
 void launch_p_count(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const uint8_t *strong, const int32_t *agg,
                     int smoothed, int32_t *plen, cudaStream_t s);
 void launch_p_fill(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const double *val, const uint8_t *strong,

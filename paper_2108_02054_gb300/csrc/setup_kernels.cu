@@ -104,6 +104,30 @@ __global__ void k_scan_blocks(int64_t *__restrict__ bsum, int64_t nb) {
     if (threadIdx.x == 0) bsum[nb] = carry;
 }
 
+// a scan of at most one tile in one launch
+__global__ void k_scan_one(const int32_t *__restrict__ in, int32_t *__restrict__ out, int64_t n, int *st) {
+    __shared__ int64_t wt[32];
+    __shared__ int64_t tot;
+    const int64_t base = (int64_t)threadIdx.x * kScanItems;
+    int64_t v[kScanItems], s = 0;
+    for (int k = 0; k < kScanItems; ++k) {
+        v[k] = base + k < n ? in[base + k] : 0;
+        s += v[k];
+    }
+    int64_t e = block_exclusive_scan(s, wt, &tot);
+    for (int k = 0; k < kScanItems; ++k) {
+        if (base + k < n) {
+            if (e > INT32_MAX) atomicOr(st, DEV_ERR_OVERFLOW);
+            out[base + k] = (int32_t)e;
+        }
+        e += v[k];
+    }
+    if (threadIdx.x == 0) {
+        if (tot > INT32_MAX) atomicOr(st, DEV_ERR_OVERFLOW);
+        out[n] = (int32_t)tot;
+    }
+}
+
 __global__ void k_scan_final(const int32_t *__restrict__ in, int32_t *__restrict__ out, int64_t n,
                              const int64_t *__restrict__ bsum, int64_t nb, int *st) {
     __shared__ int64_t wt[32];
@@ -1282,6 +1306,11 @@ void scan_counts(const int32_t *in, int32_t *out, int64_t n, int *st, int64_t *t
         return;
     }
     int64_t nb = (n + kScanTile - 1) / kScanTile;
+    if (nb == 1) {
+        count_launch();
+        k_scan_one<<<1, kScanThreads, 0, s>>>(in, out, n, st);
+        return;
+    }
     count_launch();
     k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, tmp);
     count_launch();
@@ -1368,7 +1397,7 @@ void launch_strength(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *
 int32_t run_aggregation(int32_t n, int32_t nnz, const int32_t *ptr, const int32_t *col, const double *val,
                         const uint8_t *strong, const int32_t *deg, int32_t *agg, int8_t *state, int64_t *m1,
                         uint8_t *r1, int32_t *root_id, int32_t *agg1, int32_t *root_of, int *counter, int *st,
-                        int64_t *scan_tmp, cudaStream_t s) {
+                        int64_t *scan_tmp, int32_t *h_pin, cudaStream_t s) {
     const int nb = nblocks(n);
     count_launch();
     k_mis_init<<<nb, kThreads, 0, s>>>(n, deg, state);
@@ -1380,18 +1409,17 @@ int32_t run_aggregation(int32_t n, int32_t nnz, const int32_t *ptr, const int32_
         ROW_LANES(k_mis_r1, n, ptr, col, strong, state, r1);
         cudaMemsetAsync(counter, 0, sizeof(int), s);
         ROW_LANES(k_mis_exclude, n, ptr, col, strong, state, r1, counter);
-        int h = -1;
-        if (cudaMemcpyAsync(&h, counter, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -1;
+        if (cudaMemcpyAsync(h_pin, counter, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -1;
         if (cudaStreamSynchronize(s) != cudaSuccess) return -1;
-        if (h == 0) break;
+        if (*h_pin == 0) break;
         if (round == n) return -1;
     }
     count_launch();
     k_root_flags<<<nb, kThreads, 0, s>>>(n, state, agg);
     scan_counts(agg, root_id, n, st, scan_tmp, s);
-    int32_t nagg = 0;
-    if (cudaMemcpyAsync(&nagg, root_id + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -1;
+    if (cudaMemcpyAsync(h_pin, root_id + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess) return -1;
     if (cudaStreamSynchronize(s) != cudaSuccess) return -1;
+    const int32_t nagg = *h_pin;
     ROW_LANES(k_agg_phase1, n, ptr, col, strong, state, root_id, agg1, root_of);
     ROW_LANES(k_agg_phase2, n, ptr, col, val, strong, state, agg1, root_of, agg, st);
     return nagg;
