@@ -327,28 +327,17 @@ amg_status symbolic_product(amg_ctx *ctx, int32_t nrows, int32_t ncols, int32_t 
     return AMG_OK;
 }
 
-// Lanes per row for a level's matrix-vector kernels (A rows, R rows): about
-// sixteen entries per lane, then more lanes until the level offers enough
-// threads to fill the GPU (short fine-level rows keep one lane and the plain
-// sequential row sum).  Measured against eight and thirty-two entries per
-// lane: sixteen is fastest on the large levels at 128^3 and 192^3, and the
-// occupancy rule leaves the 64^3 levels as they were.
+// Lanes per row for a level's matrix-vector kernels (rows of A, of R, of A P):
+// about sixteen entries per lane, then more lanes until the level offers enough
+// threads to fill the GPU, while a lane keeps four entries (short fine-level
+// rows keep one lane and the plain sequential row sum).  Sixteen was measured
+// against eight and thirty-two on the large levels at 128^3 and 192^3.  Fewer
+// than four entries a lane cost more in FP64 shuffle sums, one step per
+// doubling, than the shorter chains save: solves at 301^2 / 64^3 / plain 71^3 /
+// a mesh with no such limit 57.5 / 80.5 / 80.2 / 79.5 us per iteration, four
+// entries 55.7 / 80.3 / 78.9 / 76.7, two 56.3 / 80.1 / 78.9 / 78.0, eight
+// 57.3 / 82.6 / 82.2 / 78.6.
 int choose_lpr(int64_t rows, int64_t nnz) {
-    if (rows <= 0) return 1;
-    const double avg = (double)nnz / (double)rows;
-    int p = 1;
-    while (p < 32 && 16.0 * p < avg) p *= 2;
-    while (p < 32 && rows * p < 152LL * 1024) p *= 2;
-    return p;
-}
-
-// Lanes per row for the correction and sweep through A P: as above, but with at
-// least four entries a lane, since every doubling adds a step to two FP64
-// shuffle sums.  FP64, us per launch with this rule / two entries a lane / the
-// rule above: 64^3 levels 1 and 2 (16 and 17 entries a row) 7.0 + 5.1 / 8.1 +
-// 4.7 / 8.0 + 5.4; plain aggregation 71^3 (4.4) 4.9 + 4.5 / 6.1 + 4.4 / 9.6 +
-// 5.7; a mesh (24 and 16) 5.7 + 5.6 / 7.5 + 4.6 / 12.3 + 4.6.
-int choose_lpr_ap(int64_t rows, int64_t nnz) {
     if (rows <= 0) return 1;
     const double avg = (double)nnz / (double)rows;
     int p = 1;
@@ -660,7 +649,7 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         TRY(symbolic_product(ctx, L.n, nagg, L.nnz, L.A_ptr, L.A_col, L.P_ptr, L.P_col, 0, &L.AP_ptr, &L.AP_col,
                              &L.nnzAP));
         TRY(alloc(ctx, &L.AP_val, (size_t)L.nnzAP));
-        L.lpr_ap = choose_lpr_ap(L.n, L.nnzAP);
+        L.lpr_ap = choose_lpr(L.n, L.nnzAP);
         Level &C = ctx->lev[ctx->nlev];
         C.n = nagg;
         TRY(symbolic_product(ctx, nagg, nagg, L.nnzR, L.R_ptr, L.R_col, L.AP_ptr, L.AP_col, 1, &C.A_ptr, &C.A_col, &C.nnz));
