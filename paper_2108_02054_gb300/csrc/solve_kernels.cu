@@ -546,7 +546,7 @@ __device__ __forceinline__ KeyIdx better(KeyIdx a, KeyIdx b) {
 // with a lazy row permutation: rows are not moved during the elimination,
 // perm[i] names the physical row at position i, and the factors are written
 // out in position order at the end.  Larger ones use the cluster kernel (up to
-// kLuClusterN rows) or the global-memory kernel.
+// kLuClusterN rows), panels (up to kLuWideN) or the global-memory kernel.
 constexpr int kLuSmemN = 160;
 constexpr int kLuClusterN = 448;   // 8 CTAs x 56 rows x 448 columns fit in 227 KB each
 constexpr int kLuThreads = 512;
@@ -1166,6 +1166,170 @@ k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int3
     cluster.sync();
 }
 
+// ---- the coarsest LU for kLuClusterN < n <= kLuWideN (the 4 x 4 block systems
+// stop at 256 nodes, 1,024 rows): panels of kLuPanel columns
+// The elimination is n dependent steps, each a pivot search over the rows that
+// are left, and n^3 / 3 FP64 multiply-adds, 0.2 G at n = 860: one block needs
+// 60 ms for those, the chip 0.4.  So a step's search and multipliers run on one
+// block and only within its panel, one row per thread in registers (rows are
+// not moved: pos is the row's position, as in the lazy kernels above), and the
+// rest of the matrix takes a whole panel at once, a block per strip of columns.
+// Every entry still takes its updates one by one in step order, so factors and
+// pivots are bit for bit those of k_dense_lu.  src[i] is the position before the
+// panel of the row that ends at i; src[n] tells later launches that the matrix
+// is singular.
+constexpr int kLuWideN = 1024;
+constexpr int kLuPanel = 16;
+constexpr int kLuStrip = 4;  // a strip lies inside a panel or outside it
+static_assert(kLuPanel % kLuStrip == 0 && kLuPanel * kLuStrip == 64, "one warp solves a strip's top");
+__global__ void __launch_bounds__(kLuWideN)
+k_lu_panel(int32_t n, int32_t k0, double *__restrict__ g, int32_t *__restrict__ piv, int32_t *__restrict__ src, int *st) {
+    constexpr int NB = kLuPanel;
+    __shared__ unsigned long long s_key[32];
+    __shared__ int32_t s_pos[32];
+    __shared__ double s_row[NB];
+    __shared__ DivRecip s_rc;
+    const int32_t m = n - k0, nb = min(NB, m), t = threadIdx.x;
+    const int lane = t & 31, warp = t >> 5, nw = (int)(blockDim.x >> 5);
+    if (k0 > 0 && src[n] != 0) return;
+    const bool valid = t < m;
+    double v[NB];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) v[j] = valid && j < nb ? g[(int64_t)(k0 + t) * n + k0 + j] : 0.0;
+    int32_t pos = k0 + t;
+    // lanes past the last row carry no candidate
+    for (int w = t; w < 32; w += blockDim.x) s_key[w] = 0ull;
+    __syncthreads();
+    if (t == 0 && k0 == 0) src[n] = 0;
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+        if (j >= nb) break;  // block-uniform
+        const int32_t k = k0 + j;
+        const bool left = valid && pos >= k;
+        // largest magnitude, then the first position: in the warp, then over the warps
+        unsigned long long key = left ? mag_key(v[j]) : 0ull;
+        unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+        unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+        unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+        unsigned bp = __reduce_min_sync(0xffffffffu, left && hi == mh && lo == ml ? (unsigned)pos : 0xffffffffu);
+        if (lane == 0) {
+            s_key[warp] = ((unsigned long long)mh << 32) | ml;
+            s_pos[warp] = (int32_t)bp;
+        }
+        __syncthreads();
+        key = s_key[lane];
+        hi = (unsigned)(key >> 32);
+        lo = (unsigned)key;
+        mh = __reduce_max_sync(0xffffffffu, hi);
+        ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+        if ((mh | ml) == 0u) {  // block-uniform: no entry but zeros and NaNs
+            if (t == 0) {
+                atomicOr(st, DEV_ERR_SINGULAR);
+                src[n] = 1;
+            }
+            for (int32_t q = k + t; q < n; q += blockDim.x) piv[q] = q;
+            return;
+        }
+        const int32_t p = (int32_t)__reduce_min_sync(
+            0xffffffffu, lane < nw && hi == mh && lo == ml ? (unsigned)s_pos[lane] : 0xffffffffu);
+        if (left && pos == p) {
+#pragma unroll
+            for (int c = 0; c < NB; ++c) s_row[c] = v[c];
+            s_rc = div_recip(v[j]);
+            piv[k] = p;
+            pos = k;
+        } else if (pos == k) {
+            pos = p;
+        }
+        __syncthreads();
+        if (valid && pos > k) {
+            const double l = div_rn(v[j], s_rc);
+            v[j] = l;
+#pragma unroll
+            for (int c = j + 1; c < NB; ++c) v[c] = fma(-l, s_row[c], v[c]);
+        }
+    }
+    if (!valid) return;
+    src[pos] = k0 + t;
+#pragma unroll
+    for (int j = 0; j < NB; ++j)
+        if (j < nb) g[(int64_t)pos * n + k0 + j] = v[j];
+}
+
+// the panel's row exchanges in a strip of columns and, right of the panel, its
+// steps: the top rows by one warp (two rows and a column per lane), the others
+// one row per thread
+constexpr int kLuUpdateThreads = 256;
+static_assert(kLuUpdateThreads == kLuPanel * kLuPanel, "one thread stages each entry of the panel's top");
+__global__ void __launch_bounds__(kLuUpdateThreads, 2)
+k_lu_update(int32_t n, int32_t k0, double *__restrict__ g, const int32_t *__restrict__ src) {
+    constexpr int NB = kLuPanel, CW = kLuStrip;
+    extern __shared__ double sm_strip[];  // the strip's rows from k0 on, exchanged
+    __shared__ double s_u[NB][CW], s_l[NB][NB + 1];
+    const int32_t m = n - k0, c0 = blockIdx.x * CW, t = threadIdx.x;
+    if (src[n] != 0 || (c0 >= k0 && c0 < k0 + NB)) return;  // block-uniform
+    const bool right = c0 >= k0 + NB;  // then the panel is full and m > NB
+    if (right) s_l[t / NB][t % NB] = g[(int64_t)(k0 + t / NB) * n + k0 + t % NB];
+    for (int32_t e = t; e < m * CW; e += kLuUpdateThreads) {
+        const int32_t i = e / CW, c = c0 + e % CW, from = src[k0 + i];
+        if (c < n && (right || from != k0 + i)) sm_strip[e] = g[(int64_t)from * n + c];
+    }
+    __syncthreads();
+    if (!right) {
+        for (int32_t e = t; e < m * CW; e += kLuUpdateThreads) {
+            const int32_t i = e / CW, c = c0 + e % CW;
+            if (src[k0 + i] != k0 + i) g[(int64_t)(k0 + i) * n + c] = sm_strip[e];
+        }
+        return;
+    }
+    if (t < 32) {
+        const int j0 = t / CW, c = t % CW, j1 = j0 + NB / 2;
+        const bool in = c0 + c < n;
+        double a0 = in ? sm_strip[j0 * CW + c] : 0.0, a1 = in ? sm_strip[j1 * CW + c] : 0.0;
+#pragma unroll
+        for (int k = 0; k < NB - 1; ++k) {
+            const double u = __shfl_sync(0xffffffffu, k < NB / 2 ? a0 : a1, (k % (NB / 2)) * CW + c);
+            if (k < NB / 2 && j0 > k) a0 = fma(-s_l[j0][k], u, a0);
+            if (j1 > k) a1 = fma(-s_l[j1][k], u, a1);
+        }
+        s_u[j0][c] = a0;
+        s_u[j1][c] = a1;
+        if (in) {
+            g[(int64_t)(k0 + j0) * n + c0 + c] = a0;
+            g[(int64_t)(k0 + j1) * n + c0 + c] = a1;
+        }
+    }
+    __syncthreads();
+    // (volatile: the 64 values stay in shared memory, not in registers)
+    const volatile double (*u)[CW] = s_u;
+    for (int32_t i = NB + t; i < m; i += kLuUpdateThreads) {
+        double *row = g + (int64_t)(k0 + i) * n;
+        double l[NB], a[CW];
+#pragma unroll
+        for (int k = 0; k < NB; ++k) l[k] = row[k0 + k];
+#pragma unroll
+        for (int c = 0; c < CW; ++c) a[c] = c0 + c < n ? sm_strip[i * CW + c] : 0.0;
+#pragma unroll
+        for (int k = 0; k < NB; ++k)
+#pragma unroll
+            for (int c = 0; c < CW; ++c) a[c] = fma(-l[k], u[k][c], a[c]);
+#pragma unroll
+        for (int c = 0; c < CW; ++c)
+            if (c0 + c < n) row[c0 + c] = a[c];
+    }
+}
+
+// out = in^T, both n x n row-major
+__global__ void __launch_bounds__(256) k_transpose(int32_t n, const double *__restrict__ in, double *__restrict__ out) {
+    __shared__ double tile[32][33];
+    const int32_t x = threadIdx.x, bx = blockIdx.x * 32, by = blockIdx.y * 32;
+    for (int32_t y = threadIdx.y; y < 32; y += 8)
+        if (by + y < n && bx + x < n) tile[y][x] = in[(int64_t)(by + y) * n + bx + x];
+    __syncthreads();
+    for (int32_t y = threadIdx.y; y < 32; y += 8)
+        if (bx + y < n && by + x < n) out[(int64_t)(bx + y) * n + by + x] = tile[x][y];
+}
+
 __global__ void __launch_bounds__(1024) k_dense_lu(int32_t n, double *__restrict__ a, int32_t *__restrict__ piv,
                                                    int *st) {
     __shared__ KeyIdx wbest[32];
@@ -1337,20 +1501,25 @@ k_lu_inverse_rows(int32_t n, const double *__restrict__ lu_g, const int32_t *__r
     if (valid) inv[(int64_t)r * n + j] = x;
 }
 
-// explicit inverse from column-major factors (kLuSmemN < n <= kLuClusterN): one
+// explicit inverse from column-major factors (kLuSmemN < n <= kLuWideN): one
 // block per column of A^-1 with one row per thread, as k_lu_inverse_rows, the
 // factors read from L2 (contiguous across the threads) a batch of steps ahead,
 // since no factor depends on a step.  n = 212 / 255: 84 / 111 us (one warp per
 // column: 267 / 364); a step is one barrier and one fma over all warps.
+// Above kLuClusterN rows the back substitution divides by U's diagonal, as
+// k_lu_inverse does there (NMAX = kLuWideN).
 constexpr int kInvAhead = 8;
-__global__ void __launch_bounds__((kLuClusterN + 31) / 32 * 32)
+template <int NMAX>
+__global__ void __launch_bounds__((NMAX + 31) / 32 * 32)
 k_lu_inverse_t(int32_t n, const double *__restrict__ luT, const int32_t *__restrict__ piv, double *__restrict__ inv) {
-    __shared__ double xs[kLuClusterN];     // x_k as each step finalises it
-    __shared__ int32_t pv[kLuClusterN];
+    constexpr bool divide = NMAX > kLuClusterN;
+    __shared__ double xs[NMAX];     // x_k as each step finalises it
+    __shared__ int32_t pv[NMAX];
     const int32_t j = blockIdx.x, r = threadIdx.x;
     const bool valid = r < n;
     if (valid) pv[r] = piv[r];
-    const double rd = valid ? 1.0 / luT[(int64_t)r * n + r] : 0.0;
+    const double ud = valid ? luT[(int64_t)r * n + r] : 1.0;
+    const double rd = divide ? 0.0 : 1.0 / ud;
     const int32_t rc = valid ? r : 0;
     __syncthreads();
     int32_t pos = j;
@@ -1393,7 +1562,7 @@ k_lu_inverse_t(int32_t n, const double *__restrict__ luT, const int32_t *__restr
             const int32_t k = k0 - q;
             if (k < 0) break;  // block-uniform
             if (r == k) {
-                x = x * rd;
+                x = divide ? x / ud : x * rd;
                 xs[k] = x;
             }
             __syncthreads();
@@ -2671,7 +2840,7 @@ size_t lu_cluster_smem(int32_t n) {
     const size_t nloc = (size_t)(n + kLuClusterCtas - 1) / kLuClusterCtas;
     return (nloc * n + n + nloc) * sizeof(double) + 2 * (size_t)n * sizeof(int32_t);
 }
-bool lu_wants_transpose(int32_t n) { return n > kLuSmemN && n <= kLuClusterN; }
+bool lu_wants_transpose(int32_t n) { return n > kLuSmemN && n <= kLuWideN; }
 void launch_dense_lu(int32_t n, double *a, int32_t *piv, int *st, cudaStream_t s, double *aT) {
     static bool attr = false;
     const int max_bytes = kLuSmemN * kLuSmemN * (int)sizeof(double);
@@ -2687,6 +2856,20 @@ void launch_dense_lu(int32_t n, double *a, int32_t *piv, int *st, cudaStream_t s
         cudaFuncSetAttribute(k_dense_lu_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)lu_cluster_smem(kLuClusterN));
         attr = true;
+    }
+    if (aT && n > kLuClusterN && n <= kLuWideN) {
+        int32_t *src = (int32_t *)aT;  // n + 1 entries, until the transpose
+        for (int32_t k0 = 0; k0 < n; k0 += kLuPanel) {
+            count_launch();
+            k_lu_panel<<<1, (unsigned)((n - k0 + 31) / 32 * 32), 0, s>>>(n, k0, a, piv, src, st);
+            count_launch();
+            k_lu_update<<<(unsigned)((n + kLuStrip - 1) / kLuStrip), kLuUpdateThreads,
+                          (size_t)(n - k0) * kLuStrip * sizeof(double), s>>>(n, k0, a, src);
+        }
+        const unsigned tiles = (unsigned)((n + 31) / 32);
+        count_launch();
+        k_transpose<<<dim3(tiles, tiles), dim3(32, 8), 0, s>>>(n, a, aT);
+        return;
     }
     count_launch();
     if (n > kLuPipeMinN && n <= 128)
@@ -2704,9 +2887,11 @@ void launch_dense_lu(int32_t n, double *a, int32_t *piv, int *st, cudaStream_t s
 }
 void launch_lu_inverse(int32_t n, const double *lu, const int32_t *piv, double *inv, cudaStream_t s,
                        const double *luT) {
-    if (luT && n > kLuSmemN && n <= kLuClusterN) {
+    if (luT && lu_wants_transpose(n)) {
+        const unsigned threads = (unsigned)((n + 31) / 32 * 32);
         count_launch();
-        k_lu_inverse_t<<<(unsigned)n, (unsigned)((n + 31) / 32 * 32), 0, s>>>(n, luT, piv, inv);
+        if (n <= kLuClusterN) k_lu_inverse_t<kLuClusterN><<<(unsigned)n, threads, 0, s>>>(n, luT, piv, inv);
+        else k_lu_inverse_t<kLuWideN><<<(unsigned)n, threads, 0, s>>>(n, luT, piv, inv);
         return;
     }
     static bool attr = false;

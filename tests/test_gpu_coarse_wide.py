@@ -1,5 +1,6 @@
 """The coarsest LU between 128 and 256 rows (eight compute warps, message rows
-in a ring that later steps reuse) and its inverse, against the oracle."""
+in a ring that later steps reuse) and between 449 and 1,024 (panels of 16
+columns), and their inverses, against the oracle."""
 import numpy as np
 import pytest
 
@@ -18,7 +19,7 @@ def dense(M):
             torch.arange(n, dtype=torch.int32, device="cuda").repeat(n), torch.tensor(M.ravel(), device="cuda"))
 
 
-@pytest.mark.parametrize("n", [129, 153, 159, 192, 224, 255, 256, 257])
+@pytest.mark.parametrize("n", [129, 153, 159, 192, 224, 255, 256, 257, 449, 463, 464, 481, 511, 1009, 1023, 1024, 1025])
 def test_factors_and_inverse(n):
     """Tied small-integer pivots: factors and pivots bit for bit, twice on one
     context (nothing is left behind), and the V-cycle (the inverse times r)
@@ -38,9 +39,9 @@ def test_factors_and_inverse(n):
     assert np.linalg.norm(z - ref) <= 10 * n * 2.3e-16 * np.linalg.cond(M) * np.linalg.norm(ref)
 
 
-@pytest.mark.parametrize("j", [0, 39, 40, 41, 127, 128, 200, 253, 254])
-def test_zero_column(j):
-    n = 255
+@pytest.mark.parametrize("n,j", [(255, j) for j in (0, 39, 40, 41, 127, 128, 200, 253, 254)]
+                         + [(467, j) for j in (0, 1, 15, 16, 463, 464, 466)])
+def test_zero_column(n, j):
     rng = np.random.default_rng(700 + j)
     M = rng.integers(-3, 4, (n, n)).astype(np.float64) + np.eye(n) * 20.0
     Z = M.copy()
