@@ -198,15 +198,15 @@ def algorithmic_bytes(slot, lv, s, cb=4, noff=0):
     n, nnz = L0["n"], L0["nnz"]
     if 0 < noff <= 8 and slot in ("cg_spmv", "smooth0_l0", "sweep_l0"):
         return {"cg_spmv": n + 8 * nnz + 16 * n, "smooth0_l0": n + nnz * s + 2 * n * s + 8 * n,
-                "sweep_l0": n + nnz * s + 2 * n * s + 16 * n}[slot]
+                "sweep_l0": n + nnz * s + 3 * n * s + 8 * n}[slot]
     nc, nnzP = L0["nagg"], L0["nnzP"]
     nnzc = lv[1]["nnz"] if len(lv) > 1 else 0
     if slot == "cg_spmv":      # q = A p, p.q: ptr, col, val(f64), p, q
         return 4 * (n + 1) + (cb + 8) * nnz + 16 * n
     if slot == "smooth0_l0":   # r = f - A u0 (u0 = m o f, written with f): ptr, col, val, u0, f(f64), r
         return 4 * (n + 1) + nnz * (cb + s) + n * s + 8 * n + n * s
-    if slot == "sweep_l0":     # z = u + m (f - A u): ptr, col, val, m, f(f64), u, z(f64)
-        return 4 * (n + 1) + nnz * (cb + s) + n * s + 8 * n + n * s + 8 * n
+    if slot == "sweep_l0":     # z = u + m (f - A u): ptr, col, val, m, f(f64), u, z
+        return 4 * (n + 1) + nnz * (cb + s) + n * s + 8 * n + n * s + n * s
     if slot == "restrict_l0":  # f_c = R r
         return 4 * (nc + 1) + nnzP * (4 + s) + n * s + nc * s
     if slot == "prolong_l0":   # u += P u_c
@@ -217,10 +217,10 @@ def algorithmic_bytes(slot, lv, s, cb=4, noff=0):
         return 4 * (nc + 1) + nnzP * (4 + s) + nnzc * s
     if slot == "ingest":       # fine values in (f64), hierarchy copy out, smoother diagonal
         return 4 * (n + 1) + 8 * nnz + (8 if s == 8 else 12) * nnz + n * s
-    if slot in ("cg_update",):  # u, p, q, r in; u, r out; u0 = m o r (m in, u0 out)
-        return 8 * n * 6 + 2 * n * s
-    if slot == "cg_p":
-        return 8 * n * 3
+    if slot == "cg_update":    # r, q in, r out; u0 = m o r (m in, u0 out); mixed: z_old in
+        return 8 * n * 3 + (2 if s == 8 else 3) * n * s
+    if slot == "cg_p":         # z, p, u in; p, u out
+        return 8 * n * 4 + n * s
     if slot == "dot":
         return 8 * n * 2
     return None
@@ -235,12 +235,12 @@ def algorithmic_flops(slot, lv, mixed=False):
     L0 = lv[0]
     n, nnz, nnzP = L0["n"], L0["nnz"], L0["nnzP"]
     if mixed:
-        return {"cg_spmv": 2 * nnz + 2 * n, "cg_update": 8 * n, "cg_p": 2 * n}.get(slot)
+        return {"cg_spmv": 2 * nnz + 2 * n, "cg_update": 6 * n, "cg_p": 4 * n}.get(slot)
     return {"cg_spmv": 2 * nnz + 2 * n,                  # q = A p, p.q
             "smooth0_l0": 2 * nnz + n,                   # r = f - A u0
             "sweep_l0": 2 * nnz + 5 * n,                 # z = u + m (f - A u), r.z
             "restrict_l0": 2 * nnzP, "prolong_l0": 2 * nnzP,
-            "cg_update": 7 * n, "cg_p": 2 * n}.get(slot)
+            "cg_update": 5 * n, "cg_p": 4 * n}.get(slot)
 
 
 # GB300 FP64 (non-tensor) peak from its unit counts: 152 SMs x 2 FP64 FMA per
