@@ -1170,7 +1170,7 @@ k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int3
 // stop at 256 nodes, 1,024 rows): panels of kLuPanel columns
 // The elimination is n dependent steps, each a pivot search over the rows that
 // are left, and n^3 / 3 FP64 multiply-adds, 0.2 G at n = 860: one block needs
-// 60 ms for those, the chip 0.4.  So a step's search and multipliers run on one
+// over 60 ms for those, the chip 0.4.  So a step's search and multipliers run on one
 // block and only within its panel, one row per thread in registers (rows are
 // not moved: pos is the row's position, as in the lazy kernels above), and the
 // rest of the matrix takes a whole panel at once, a block per strip of columns.
@@ -1178,6 +1178,8 @@ k_dense_lu_pipe(int32_t n, double *__restrict__ g, double *__restrict__ gT, int3
 // pivots are bit for bit those of k_dense_lu.  src[i] is the position before the
 // panel of the row that ends at i; src[n] tells later launches that the matrix
 // is singular.
+// n = 860: 73.4 -> 4.4 ms; a panel 37 us (32 rows: step latency) to 73 (860
+// rows: the FP64 pipe of one SM), an update 9 to 39.
 constexpr int kLuWideN = 1024;
 constexpr int kLuPanel = 16;
 constexpr int kLuStrip = 4;  // a strip lies inside a panel or outside it
@@ -1504,23 +1506,29 @@ k_lu_inverse_rows(int32_t n, const double *__restrict__ lu_g, const int32_t *__r
 // explicit inverse from column-major factors (kLuSmemN < n <= kLuWideN): one
 // block per column of A^-1 with one row per thread, as k_lu_inverse_rows, the
 // factors read from L2 (contiguous across the threads) a batch of steps ahead,
-// since no factor depends on a step.  n = 212 / 255: 84 / 111 us (one warp per
-// column: 267 / 364); a step is one barrier and one fma over all warps.
+// since no factor depends on a step.  A batch's rows lie in one warp, which
+// takes its steps by shuffles; the rows beyond take the batch after one barrier,
+// each in step order, and warps with none left skip it (a predicated-off FP64
+// instruction would still take its slot).
+// n = 212 / 255 / 860: 56 / 70 / 2,424 us (a barrier a step 84 / 111 / 3,960, one
+// warp per column 267 / 364 / 12,845).
 // Above kLuClusterN rows the back substitution divides by U's diagonal, as
-// k_lu_inverse does there (NMAX = kLuWideN).
+// k_lu_inverse does there (NMAX = kLuWideN), with the integer quotient.
 constexpr int kInvAhead = 8;
+static_assert(32 % kInvAhead == 0, "a batch lies in one warp");
 template <int NMAX>
 __global__ void __launch_bounds__((NMAX + 31) / 32 * 32)
 k_lu_inverse_t(int32_t n, const double *__restrict__ luT, const int32_t *__restrict__ piv, double *__restrict__ inv) {
     constexpr bool divide = NMAX > kLuClusterN;
-    __shared__ double xs[NMAX];     // x_k as each step finalises it
+    constexpr int B = kInvAhead;
+    __shared__ double xs[2][B];  // a batch's x, final
     __shared__ int32_t pv[NMAX];
-    const int32_t j = blockIdx.x, r = threadIdx.x;
+    const int32_t j = blockIdx.x, r = threadIdx.x, w0 = r & ~31;
     const bool valid = r < n;
     if (valid) pv[r] = piv[r];
     const double ud = valid ? luT[(int64_t)r * n + r] : 1.0;
     const double rd = divide ? 0.0 : 1.0 / ud;
-    const int32_t rc = valid ? r : 0;
+    const double *__restrict__ col = luT + (valid ? r : 0);
     __syncthreads();
     int32_t pos = j;
     for (int32_t k = 0; k < n; ++k) {
@@ -1531,45 +1539,64 @@ k_lu_inverse_t(int32_t n, const double *__restrict__ luT, const int32_t *__restr
     }
     double x = valid && r == pos ? 1.0 : 0.0;
     // L y = P e_j (unit lower triangular); entries before pos stay zero
-    double l[kInvAhead];
+    double l[B];
+    int32_t k0 = pos / B * B;
 #pragma unroll
-    for (int q = 0; q < kInvAhead; ++q) l[q] = luT[(int64_t)min(pos + q, n - 1) * n + rc];
-    for (int32_t k0 = pos; k0 < n - 1; k0 += kInvAhead) {
-        double nl[kInvAhead];
+    for (int q = 0; q < B; ++q) l[q] = col[(int64_t)min(k0 + q, n - 1) * n];
+    for (; k0 < n; k0 += B) {
+        double nl[B], *xb = xs[(k0 / B) & 1];
 #pragma unroll
-        for (int q = 0; q < kInvAhead; ++q) nl[q] = luT[(int64_t)min(k0 + kInvAhead + q, n - 1) * n + rc];
+        for (int q = 0; q < B; ++q) nl[q] = col[(int64_t)min(k0 + B + q, n - 1) * n];
+        if (w0 == (k0 & ~31)) {
 #pragma unroll
-        for (int q = 0; q < kInvAhead; ++q) {
-            const int32_t k = k0 + q;
-            if (k >= n - 1) break;  // block-uniform
-            if (r == k) xs[k] = x;
-            __syncthreads();
-            if (valid && r > k) x = fma(-l[q], xs[k], x);
+            for (int q = 0; q < B; ++q) {
+                const double xk = __shfl_sync(0xffffffffu, x, (k0 + q) & 31);
+                if (k0 + q >= pos && valid && r > k0 + q) x = fma(-l[q], xk, x);
+            }
+            if (r >= k0 && r < k0 + B) xb[r - k0] = x;
+        }
+        __syncthreads();
+        if (w0 > k0) {
+#pragma unroll
+            for (int q = 0; q < B; ++q)
+                if (k0 + q >= pos) x = fma(-l[q], xb[q], x);
         }
 #pragma unroll
-        for (int q = 0; q < kInvAhead; ++q) l[q] = nl[q];
+        for (int q = 0; q < B; ++q) l[q] = nl[q];
     }
     // U x = y
+    k0 = (n - 1) / B * B;
 #pragma unroll
-    for (int q = 0; q < kInvAhead; ++q) l[q] = luT[(int64_t)max(n - 1 - q, 0) * n + rc];
+    for (int q = 0; q < B; ++q) l[q] = col[(int64_t)min(k0 + q, n - 1) * n];
     __syncthreads();
-    for (int32_t k0 = n - 1; k0 >= 0; k0 -= kInvAhead) {
-        double nl[kInvAhead];
+    for (; k0 >= 0; k0 -= B) {
+        double nl[B], *xb = xs[(k0 / B) & 1];
 #pragma unroll
-        for (int q = 0; q < kInvAhead; ++q) nl[q] = luT[(int64_t)max(k0 - kInvAhead - q, 0) * n + rc];
+        for (int q = 0; q < B; ++q) nl[q] = col[(int64_t)max(k0 - B + q, 0) * n];
+        if (w0 == (k0 & ~31)) {
+            DivRecip rc;
+            if constexpr (divide) rc = div_recip(ud);
 #pragma unroll
-        for (int q = 0; q < kInvAhead; ++q) {
-            const int32_t k = k0 - q;
-            if (k < 0) break;  // block-uniform
-            if (r == k) {
-                x = divide ? x / ud : x * rd;
-                xs[k] = x;
+            for (int q = B - 1; q >= 0; --q) {
+                const int32_t k = k0 + q;
+                if (k >= n) continue;  // warp-uniform
+                if (r == k) {
+                    if constexpr (divide) x = div_rn(x, rc);
+                    else x = x * rd;
+                }
+                const double xk = __shfl_sync(0xffffffffu, x, k & 31);
+                if (r < k) x = fma(-l[q], xk, x);
             }
-            __syncthreads();
-            if (valid && r < k) x = fma(-l[q], xs[k], x);
+            if (r >= k0 && r < k0 + B) xb[r - k0] = x;
+        }
+        __syncthreads();
+        if (w0 + 32 <= k0) {
+#pragma unroll
+            for (int q = B - 1; q >= 0; --q)
+                if (k0 + q < n) x = fma(-l[q], xb[q], x);
         }
 #pragma unroll
-        for (int q = 0; q < kInvAhead; ++q) l[q] = nl[q];
+        for (int q = 0; q < B; ++q) l[q] = nl[q];
     }
     if (valid) inv[(int64_t)r * n + j] = x;
 }
