@@ -1386,42 +1386,20 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// explicit inverse from the LU factors: one warp per column j of A^-1, in
-// column (axpy) form so that no step needs a reduction; the factors, the
-// pivots, the reciprocals of U's diagonal and each warp's column are staged
-// in shared memory when they fit (the reciprocals keep an FP64 division off
-// every back-substitution step)
+// explicit inverse from the LU factors (n > kLuWideN): one warp per column j of
+// A^-1, in column (axpy) form so that no step needs a reduction
 constexpr int kInvWarps = 4;
 __global__ void __launch_bounds__(kInvWarps * 32)
-k_lu_inverse(int32_t n, const double *__restrict__ lu_g, const int32_t *__restrict__ piv, double *__restrict__ inv) {
-    extern __shared__ double sm_inv[];
+k_lu_inverse(int32_t n, const double *__restrict__ lu, const int32_t *__restrict__ piv, double *__restrict__ inv) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const bool staged = n <= kLuSmemN;
-    const int64_t nn = (int64_t)n * n;
-    const double *lu = lu_g;
-    const int32_t *pv = piv;
-    const double *rd = nullptr;
-    if (staged) {
-        for (int64_t e = threadIdx.x; e < nn; e += blockDim.x) sm_inv[e] = lu_g[e];
-        double *srd = sm_inv + nn + (int64_t)kInvWarps * n;
-        for (int32_t e = threadIdx.x; e < n; e += blockDim.x) srd[e] = 1.0 / lu_g[(int64_t)e * n + e];
-        int32_t *spv = (int32_t *)(srd + n);
-        for (int32_t e = threadIdx.x; e < n; e += blockDim.x) spv[e] = piv[e];
-        lu = sm_inv;
-        pv = spv;
-        rd = srd;
-    }
-    __syncthreads();
     const int32_t j = blockIdx.x * kInvWarps + w;
     if (j >= n) return;  // warp-uniform; no block barrier follows
-    double *x;
-    int64_t xs;
-    if (staged) { x = sm_inv + nn + (int64_t)w * n; xs = 1; }
-    else { x = inv + j; xs = n; }
+    double *x = inv + j;
+    const int64_t xs = n;
     // P e_j is the unit vector at the position that the row swaps move j to
     int32_t pos = j;
     for (int32_t k = 0; k < n; ++k) {
-        const int32_t p = pv[k];
+        const int32_t p = piv[k];
         if (p < 0 || p >= n || p == k) continue;
         if (pos == k) pos = p;
         else if (pos == p) pos = k;
@@ -1436,22 +1414,22 @@ k_lu_inverse(int32_t n, const double *__restrict__ lu_g, const int32_t *__restri
     }
     // U x = y
     for (int32_t k = n - 1; k >= 0; --k) {
-        if (lane == 0) x[k * xs] = rd ? x[k * xs] * rd[k] : x[k * xs] / lu[(int64_t)k * n + k];
+        if (lane == 0) x[k * xs] = x[k * xs] / lu[(int64_t)k * n + k];
         __syncwarp();
         const double xk = x[k * xs];
         for (int32_t r = lane; r < k; r += 32) x[r * xs] = fma(-lu[(int64_t)r * n + k], xk, x[r * xs]);
         __syncwarp();
     }
-    if (staged)
-        for (int32_t r = lane; r < n; r += 32) inv[(int64_t)r * n + j] = x[r];
 }
 
-// explicit inverse from the LU factors (n <= kLuSmemN): one block per column
+// explicit inverse from the LU factors (n <= kInvRowsN): one block per column
 // j of A^-1 with one row per thread (so each substitution step costs one fma
 // and one block barrier, not a warp's serial chunks), the factors staged in
-// shared memory.  The arithmetic per entry is that of k_lu_inverse: L y =
-// P e_j, then U x = y with x_k = y_k * (1 / u_kk), each in step order.
-__global__ void __launch_bounds__((kLuSmemN + 31) / 32 * 32)
+// shared memory: L y = P e_j, then U x = y with x_k = y_k * (1 / u_kk), each in
+// step order.  Up to four warps of rows: n = 87 / 153 here 20.2 / 52 us, with
+// the kernel below 21.9 / 38.4.
+constexpr int kInvRowsN = 128;
+__global__ void __launch_bounds__(kInvRowsN)
 k_lu_inverse_rows(int32_t n, const double *__restrict__ lu_g, const int32_t *__restrict__ piv,
                   double *__restrict__ inv) {
     extern __shared__ __align__(16) double sm_iv[];
@@ -1503,15 +1481,15 @@ k_lu_inverse_rows(int32_t n, const double *__restrict__ lu_g, const int32_t *__r
     if (valid) inv[(int64_t)r * n + j] = x;
 }
 
-// explicit inverse from column-major factors (kLuSmemN < n <= kLuWideN): one
+// explicit inverse from column-major factors (kInvRowsN < n <= kLuWideN): one
 // block per column of A^-1 with one row per thread, as k_lu_inverse_rows, the
 // factors read from L2 (contiguous across the threads) a batch of steps ahead,
 // since no factor depends on a step.  A batch's rows lie in one warp, which
 // takes its steps by shuffles; the rows beyond take the batch after one barrier,
 // each in step order, and warps with none left skip it (a predicated-off FP64
 // instruction would still take its slot).
-// n = 212 / 255 / 860: 56 / 70 / 2,424 us (a barrier a step 84 / 111 / 3,960, one
-// warp per column 267 / 364 / 12,845).
+// n = 153 / 212 / 255 / 860: 38 / 56 / 70 / 2,424 us (k_lu_inverse_rows at 153: 52;
+// a barrier a step 84 / 111 / 3,960, one warp per column 267 / 364 / 12,845).
 // Above kLuClusterN rows the back substitution divides by U's diagonal, as
 // k_lu_inverse does there (NMAX = kLuWideN), with the integer quotient.
 constexpr int kInvAhead = 8;
@@ -2867,7 +2845,7 @@ size_t lu_cluster_smem(int32_t n) {
     const size_t nloc = (size_t)(n + kLuClusterCtas - 1) / kLuClusterCtas;
     return (nloc * n + n + nloc) * sizeof(double) + 2 * (size_t)n * sizeof(int32_t);
 }
-bool lu_wants_transpose(int32_t n) { return n > kLuSmemN && n <= kLuWideN; }
+bool lu_wants_transpose(int32_t n) { return n > kInvRowsN && n <= kLuWideN; }
 void launch_dense_lu(int32_t n, double *a, int32_t *piv, int *st, cudaStream_t s, double *aT) {
     static bool attr = false;
     const int max_bytes = kLuSmemN * kLuSmemN * (int)sizeof(double);
@@ -2922,16 +2900,13 @@ void launch_lu_inverse(int32_t n, const double *lu, const int32_t *piv, double *
         return;
     }
     static bool attr = false;
-    const int max_bytes = (kLuSmemN * kLuSmemN + (kInvWarps + 1) * kLuSmemN) * (int)sizeof(double) +
-                          kLuSmemN * (int)sizeof(int32_t);
     if (!attr) {
-        cudaFuncSetAttribute(k_lu_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
         cudaFuncSetAttribute(k_lu_inverse_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (kLuSmemN * kLuSmemN + kLuSmemN) * (int)sizeof(double) + kLuSmemN * (int)sizeof(int32_t));
+                             (kInvRowsN * kInvRowsN + kInvRowsN) * (int)sizeof(double) + kInvRowsN * (int)sizeof(int32_t));
         attr = true;
     }
     count_launch();
-    if (n <= kLuSmemN) {
+    if (n <= kInvRowsN) {
         const unsigned threads = (unsigned)((n + 31) / 32 * 32);
         k_lu_inverse_rows<<<(unsigned)n, threads,
                             ((size_t)n * n + (size_t)n) * sizeof(double) + (size_t)n * sizeof(int32_t), s>>>(n, lu, piv,
