@@ -347,7 +347,9 @@ int choose_lpr(int64_t rows, int64_t nnz) {
 }
 
 // the coarsest direct solver: dense LU (FP64) and its explicit inverse
-amg_status coarse_factor(amg_ctx *ctx) {
+// (a0: the finest level's FP64 values in CSR order, which are the coarsest's
+// where there is one level; a stencil's CSR array does not follow new values)
+amg_status coarse_factor(amg_ctx *ctx, const double *a0) {
     Level &C = ctx->lev[ctx->nlev - 1];
     if (blockmode(ctx)) {
         const int32_t n4 = ctx->nL;
@@ -358,7 +360,8 @@ amg_status coarse_factor(amg_ctx *ctx) {
         return AMG_OK;
     }
     const bool mx = mixed(ctx);
-    launch_csr_to_dense(C.n, C.A_ptr, C.A_col, mx ? nullptr : C.A_val, mx ? C.A_valf : nullptr, ctx->lu, ctx->s);
+    const double *a = ctx->nlev == 1 ? a0 : C.A_val;
+    launch_csr_to_dense(C.n, C.A_ptr, C.A_col, mx ? nullptr : a, mx ? C.A_valf : nullptr, ctx->lu, ctx->s);
     { ProfScope ps_(ctx, AMG_PROF_LU, true); launch_dense_lu(C.n, ctx->lu, ctx->piv, ctx->d_st, ctx->s, ctx->luT); }
     { ProfScope ps_(ctx, AMG_PROF_INV, true); launch_lu_inverse(C.n, ctx->lu, ctx->piv, ctx->inv, ctx->s, ctx->luT); }
     if (ctx->coarse_w) launch_coarse_w(ctx->lev[ctx->nlev - 2], ctx->nL, ctx->inv, ctx->coarse_w, ctx->s);
@@ -419,7 +422,7 @@ amg_status block_numeric_rebuild(amg_ctx *ctx, const double *d_val, bool galerki
             { ProfScope ps_(ctx, AMG_PROF_RAP_L0, l == 0); launch_block_gather(C.nnz, L.g2_ptr, L.g2_idx, L.g2_w, L.APb, C.Ab, ctx->s); }
         }
     }
-    return coarse_factor(ctx);
+    return coarse_factor(ctx, nullptr);
 }
 
 // numeric part shared by the full setup and the partial rebuild (Alg. 4 body)
@@ -494,7 +497,7 @@ amg_status numeric_rebuild(amg_ctx *ctx, const double *d_val, bool galerkin, con
             else launch_smoother_f64(C.n, C.A_ptr, C.A_val, C.dia, p.smoother, p.jacobi_omega, C.m, ctx->s);
         }
     }
-    return coarse_factor(ctx);
+    return coarse_factor(ctx, a64);
 }
 
 // Two-byte column offsets for every level without the one-byte form: A's
