@@ -468,7 +468,9 @@ k_ingest_stencil(int32_t row0, int32_t n, const int32_t *__restrict__ ptr, const
     if (mf) mf[i] = f64_to_f32_rn(mi);
 }
 
-// row masks of a stencil pattern (an offset missing from the table flags the status word)
+// row masks of a stencil pattern.  The status word is flagged for a column that
+// a row holds twice (the caller's pattern is wrong) and for an offset missing
+// from the table (which holds every offset of the pattern)
 __global__ void k_stencil_mask(int32_t n, const int32_t *__restrict__ ptr, const int32_t *__restrict__ col, Stencil S,
                                uint8_t *__restrict__ mask, int *st) {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -480,7 +482,8 @@ __global__ void k_stencil_mask(int32_t n, const int32_t *__restrict__ ptr, const
 #pragma unroll
         for (int k = 0; k < kMaxStencil; ++k)
             if (k < S.noff && S.off[k] == d) bit = 1u << k;
-        if (bit == 0u || (m & bit)) atomicOr(st, DEV_ERR_STATE);
+        if (bit == 0u) atomicOr(st, DEV_ERR_STATE);
+        if (m & bit) atomicOr(st, DEV_ERR_PATTERN);
         m |= bit;
     }
     mask[i] = (uint8_t)m;
