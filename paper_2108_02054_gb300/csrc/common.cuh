@@ -175,9 +175,14 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     // a launch error stays the runtime's last error, read by the status check
     (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
-// four consecutive doubles from a 32-byte boundary in one load
+// four consecutive doubles from a 32-byte boundary in one load (an ordinary one,
+// so that the compiler keeps it after pdl_wait() and behind earlier stores)
 __device__ __forceinline__ void load32(const double *p, double (&v)[4]) {
-    asm("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p));
+    const double4_32a x = *reinterpret_cast<const double4_32a *>(p);
+    v[0] = x.x;
+    v[1] = x.y;
+    v[2] = x.z;
+    v[3] = x.w;
 }
 // 4 x 4 blocks, one thread per unknown t = 4 node + r, whole quads active:
 // component r of base + Minv_node v (fma from base, component order), where
