@@ -56,6 +56,7 @@ struct amg_ctx {
     cudaStream_t s = nullptr;
     cudaMemPool_t pool = nullptr;
     std::vector<void *> hier;     // hierarchy allocations (replaced by every full setup)
+    std::vector<void *> temp;     // scratch of a setup's current piece (free_temp)
     std::vector<void *> persist;  // context-lifetime allocations
     std::string err;
     // fine pattern (persistent)
@@ -71,7 +72,6 @@ struct amg_ctx {
     // fill it: the finest level's kernels then read its values by diagonals
     Stencil sten;
     uint8_t *sten_mask = nullptr;
-    bool a_val_stale = false;  // stencil form: A_val (CSR) is older than S_val
     // hierarchy
     int nlev = 0;
     Level lev[kMaxLevels];
@@ -80,10 +80,11 @@ struct amg_ctx {
     double *coarse_w = nullptr;  // A_L^-1 R, where it is small enough to solve with
     int32_t *piv = nullptr;
     bool have_setup = false;
-    // system matrix of the solve (aliases level 0 except under full reuse)
-    double *A_sys = nullptr;
-    double *A_sys_own = nullptr;
-    double *S_sys = nullptr, *S_sys_own = nullptr;  // the same by diagonals (stencil form)
+    // system matrix of the solve (aliases level 0 except under full reuse, where
+    // sys_own holds it): CSR or block values, or by diagonals (stencil form)
+    double *A_sys = nullptr, *S_sys = nullptr;
+    double *sys_own = nullptr;
+    size_t sys_own_vals = 0;
     // CG
     double *cg_r = nullptr, *cg_z = nullptr, *cg_p = nullptr, *cg_q = nullptr, *cg_t = nullptr;
     // per-block partial sums of the CG reductions, one set per reduction so
@@ -206,7 +207,23 @@ amg_status alloc(amg_ctx *ctx, T **p, size_t count, bool persistent = false) {
     return AMG_OK;
 }
 
+// Scratch that only a setup's current piece uses: back in the pool, in stream
+// order, once the piece's kernels are enqueued, so that the next allocations
+// take its place instead of growing the pool
+template <class T>
+amg_status alloc_temp(amg_ctx *ctx, T **p, size_t count) {
+    TRY(alloc(ctx, p, count));
+    ctx->temp.push_back(ctx->hier.back());
+    ctx->hier.pop_back();
+    return AMG_OK;
+}
+void free_temp(amg_ctx *ctx) {
+    for (void *p : ctx->temp) cudaFreeAsync(p, ctx->s);
+    ctx->temp.clear();
+}
+
 void free_hierarchy(amg_ctx *ctx) {
+    free_temp(ctx);
     for (void *p : ctx->hier) cudaFreeAsync(p, ctx->s);
     ctx->hier.clear();
     for (int l = 0; l < kMaxLevels; ++l) ctx->lev[l] = Level{};
@@ -215,7 +232,6 @@ void free_hierarchy(amg_ctx *ctx) {
     ctx->lu = ctx->inv = ctx->luT = ctx->coarse_w = nullptr;
     ctx->piv = nullptr;
     ctx->graph_valid = false;
-    ctx->a_val_stale = false;
 }
 
 // read the device status word (synchronises the stream) and map it
@@ -261,7 +277,7 @@ amg_status read_back(amg_ctx *ctx, const char *where, std::initializer_list<Read
 
 amg_status scan(amg_ctx *ctx, const int32_t *in, int32_t *out, int64_t n) {
     int64_t *tmp = nullptr;
-    TRY(alloc(ctx, &tmp, (size_t)scan_tmp_elems(n)));
+    TRY(alloc_temp(ctx, &tmp, (size_t)scan_tmp_elems(n)));
     scan_counts(in, out, n, ctx->d_st, tmp, ctx->s);
     return AMG_OK;
 }
@@ -304,11 +320,11 @@ amg_status symbolic_product(amg_ctx *ctx, int32_t nrows, int32_t ncols, int32_t 
                             const int32_t *Y_ptr, const int32_t *Y_col, int add_diag, int32_t **C_ptr,
                             int32_t **C_col, int32_t *C_nnz) {
     int32_t *len = nullptr;
-    TRY(alloc(ctx, &len, (size_t)nrows));
+    TRY(alloc_temp(ctx, &len, (size_t)nrows));
     TRY(alloc(ctx, C_ptr, (size_t)nrows + 1));
     // the hash tables are sized for the longest row of terms
     int *d_max = nullptr;
-    TRY(alloc(ctx, &d_max, 1));
+    TRY(alloc_temp(ctx, &d_max, 1));
     CK(cudaMemsetAsync(d_max, 0, sizeof(int), ctx->s));
     launch_row_terms_max(nrows, X_ptr, X_col, Y_ptr, add_diag, d_max, ctx->s);
     int32_t max_terms = 0;
@@ -348,7 +364,7 @@ int choose_lpr(int64_t rows, int64_t nnz) {
 
 // the coarsest direct solver: dense LU (FP64) and its explicit inverse
 // (a0: the finest level's FP64 values in CSR order, which are the coarsest's
-// where there is one level; a stencil's CSR array does not follow new values)
+// where there is one level; a stencil level holds its own by diagonals only)
 amg_status coarse_factor(amg_ctx *ctx, const double *a0) {
     Level &C = ctx->lev[ctx->nlev - 1];
     if (blockmode(ctx)) {
@@ -379,9 +395,9 @@ amg_status build_gather(amg_ctx *ctx, int l) {
     const int64_t tmax = std::max(nt1, nt2);
     int32_t *perm = nullptr, *idx_tmp = nullptr;
     double *w_tmp = nullptr;
-    TRY(alloc(ctx, &perm, (size_t)tmax));
-    TRY(alloc(ctx, &idx_tmp, (size_t)tmax));
-    TRY(alloc(ctx, &w_tmp, (size_t)tmax));
+    TRY(alloc_temp(ctx, &perm, (size_t)tmax));
+    TRY(alloc_temp(ctx, &idx_tmp, (size_t)tmax));
+    TRY(alloc_temp(ctx, &w_tmp, (size_t)tmax));
     // stage 1: one output per entry of AP
     TRY(alloc(ctx, &L.g1_ptr, (size_t)L.nnzAP + 1));
     TRY(alloc(ctx, &L.g1_idx, (size_t)nt1));
@@ -400,6 +416,7 @@ amg_status build_gather(amg_ctx *ctx, int l) {
     CK(cudaMemcpyAsync(L.g2_ptr + C.nnz, L.t2ptr + L.nc, sizeof(int32_t), cudaMemcpyDeviceToDevice, ctx->s));
     launch_stage2_terms(L.nc, L.R_ptr, L.R_col, L.R_val, L.AP_ptr, L.t2ptr, idx_tmp, w_tmp, ctx->s);
     launch_permute_terms(nt2, perm, idx_tmp, w_tmp, L.g2_idx, mx ? nullptr : L.g2_w, mx ? L.g2_wf : nullptr, ctx->s);
+    free_temp(ctx);
     L.gather_ready = true;
     return AMG_OK;
 }
@@ -435,7 +452,6 @@ amg_status numeric_rebuild(amg_ctx *ctx, const double *d_val, bool galerkin, con
     // a stencil's values go to their diagonals only; the finest stage 1 reads
     // the caller's CSR values (FP64) or their FP32 copy
     const double *a64 = sten ? d_val : F.A_val;
-    if (sten && d_val != F.A_val) ctx->a_val_stale = true;
     auto ingest = [&](int32_t r0, int32_t r1) {
         if (sten) {
             launch_ingest_stencil(r0, r1, F.A_ptr, d_val, F.sten, p.smoother, p.jacobi_omega, F.S_val,
@@ -510,7 +526,7 @@ amg_status numeric_rebuild(amg_ctx *ctx, const double *d_val, bool galerkin, con
 amg_status build_delta16(amg_ctx *ctx) {
     if (blockmode(ctx)) return AMG_OK;
     int *flags = nullptr;
-    TRY(alloc(ctx, &flags, (size_t)(3 * kMaxLevels)));
+    TRY(alloc_temp(ctx, &flags, (size_t)(3 * kMaxLevels)));
     CK(cudaMemsetAsync(flags, 0, sizeof(int) * 3 * kMaxLevels, ctx->s));
     int16_t *buf[kMaxLevels] = {}, *pbuf[kMaxLevels] = {}, *apbuf[kMaxLevels] = {};
     float ratio[kMaxLevels] = {};
@@ -535,6 +551,7 @@ amg_status build_delta16(amg_ctx *ctx) {
     int h[3 * kMaxLevels] = {};
     CK(cudaMemcpyAsync(h, flags, sizeof(h), cudaMemcpyDeviceToHost, ctx->s));
     CK(cudaStreamSynchronize(ctx->s));
+    free_temp(ctx);
     for (int l = 0; l < ctx->nlev; ++l) {
         if (buf[l] && h[l] == 0) ctx->lev[l].A_c16 = buf[l];
         if (pbuf[l] && h[kMaxLevels + l] == 0) {
@@ -568,7 +585,8 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         F.A_coff = ctx->fine_coff;
         F.A_ncoff = ctx->fine_ncoff;
     }
-    TRY(alloc(ctx, &F.A_val, (size_t)nnz));
+    // (a stencil level's CSR values are the caller's, and read during the setup only)
+    if (!F.sten.noff) TRY(alloc(ctx, &F.A_val, (size_t)nnz));
     TRY(alloc(ctx, &F.dia, (size_t)n));
     launch_check_pattern(n, nnz, F.A_ptr, F.A_col, F.dia, ctx->d_st, ctx->s);
     launch_check_finite((int64_t)nvals(ctx), d_val, ctx->d_st, ctx->s);
@@ -577,7 +595,7 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         TRY(alloc(ctx, &F.Ab, nvals(ctx)));
         CK(cudaMemcpyAsync(F.Ab, d_val, sizeof(double) * nvals(ctx), cudaMemcpyDeviceToDevice, ctx->s));
         launch_block_norms(nnz, F.Ab, F.A_val, ctx->s);
-    } else {
+    } else if (!F.sten.noff) {
         CK(cudaMemcpyAsync(F.A_val, d_val, sizeof(double) * (size_t)nnz, cudaMemcpyDeviceToDevice, ctx->s));
     }
     TRY(check_device(ctx, "full setup input"));
@@ -585,6 +603,7 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
     double theta = p.theta;
     for (;;) {
         Level &L = ctx->lev[ctx->nlev - 1];
+        const double *A_val = L.sten.noff ? d_val : L.A_val;
         TRY(alloc_level_vectors(ctx, L));
         TRY(alloc(ctx, &L.agg, (size_t)L.n));
         TRY(alloc(ctx, &L.strong, (size_t)L.nnz));
@@ -598,22 +617,23 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         int64_t *m1 = nullptr, *scan_tmp = nullptr;
         uint8_t *r1 = nullptr;
         int *counter = nullptr;
-        TRY(alloc(ctx, &deg, (size_t)L.n));
-        TRY(alloc(ctx, &root_id, (size_t)L.n + 1));
-        TRY(alloc(ctx, &agg1, (size_t)L.n));
-        TRY(alloc(ctx, &root_of, (size_t)L.n));
-        TRY(alloc(ctx, &state, (size_t)L.n));
-        TRY(alloc(ctx, &m1, (size_t)L.n));
-        TRY(alloc(ctx, &r1, (size_t)L.n));
-        TRY(alloc(ctx, &counter, 1));
-        TRY(alloc(ctx, &scan_tmp, (size_t)scan_tmp_elems(L.n)));
-        launch_strength(L.n, L.nnz, L.A_ptr, L.A_col, L.A_val, L.dia, theta * theta, L.strong, deg, ctx->s);
-        int32_t nagg = run_aggregation(L.n, L.nnz, L.A_ptr, L.A_col, L.A_val, L.strong, deg, L.agg, state, m1, r1, root_id,
+        TRY(alloc_temp(ctx, &deg, (size_t)L.n));
+        TRY(alloc_temp(ctx, &root_id, (size_t)L.n + 1));
+        TRY(alloc_temp(ctx, &agg1, (size_t)L.n));
+        TRY(alloc_temp(ctx, &root_of, (size_t)L.n));
+        TRY(alloc_temp(ctx, &state, (size_t)L.n));
+        TRY(alloc_temp(ctx, &m1, (size_t)L.n));
+        TRY(alloc_temp(ctx, &r1, (size_t)L.n));
+        TRY(alloc_temp(ctx, &counter, 1));
+        TRY(alloc_temp(ctx, &scan_tmp, (size_t)scan_tmp_elems(L.n)));
+        launch_strength(L.n, L.nnz, L.A_ptr, L.A_col, A_val, L.dia, theta * theta, L.strong, deg, ctx->s);
+        int32_t nagg = run_aggregation(L.n, L.nnz, L.A_ptr, L.A_col, A_val, L.strong, deg, L.agg, state, m1, r1, root_id,
                                        agg1, root_of, counter, ctx->d_st, scan_tmp, ctx->h_rb, ctx->s);
         if (nagg < 0) {
             CK(cudaGetLastError());
             return set_err(ctx, AMG_ERR_CUDA, "aggregation did not complete");
         }
+        free_temp(ctx);
         if (nagg == 0 || nagg >= L.n) {
             TRY(check_device(ctx, "aggregation"));
             // coarsening stalls: this level becomes the coarsest
@@ -624,19 +644,19 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         L.nc = nagg;
         // smoothed prolongation
         int32_t *plen = nullptr;
-        TRY(alloc(ctx, &plen, (size_t)L.n));
+        TRY(alloc_temp(ctx, &plen, (size_t)L.n));
         TRY(alloc(ctx, &L.P_ptr, (size_t)L.n + 1));
         launch_p_count(L.n, L.nnz, L.A_ptr, L.A_col, L.strong, L.agg, p.smoothed, plen, ctx->s);
         TRY(scan(ctx, plen, L.P_ptr, L.n));
         TRY(read_back(ctx, "aggregation", {{L.P_ptr + L.n, &L.nnzP}}));
         TRY(alloc(ctx, &L.P_col, (size_t)L.nnzP));
         TRY(alloc(ctx, &L.P_val, (size_t)L.nnzP));
-        launch_p_fill(L.n, L.nnz, L.A_ptr, L.A_col, L.A_val, L.strong, L.dia, L.agg, p.omega, p.smoothed, L.P_ptr, L.P_col,
+        launch_p_fill(L.n, L.nnz, L.A_ptr, L.A_col, A_val, L.strong, L.dia, L.agg, p.omega, p.smoothed, L.P_ptr, L.P_col,
                       L.P_val, ctx->s);
         // R = P^T
         int32_t *cnt = nullptr, *cursor = nullptr;
-        TRY(alloc(ctx, &cnt, (size_t)nagg));
-        TRY(alloc(ctx, &cursor, (size_t)nagg));
+        TRY(alloc_temp(ctx, &cnt, (size_t)nagg));
+        TRY(alloc_temp(ctx, &cursor, (size_t)nagg));
         CK(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)nagg, ctx->s));
         CK(cudaMemsetAsync(cursor, 0, sizeof(int32_t) * (size_t)nagg, ctx->s));
         launch_count_cols(L.nnzP, L.P_col, cnt, ctx->s);
@@ -662,8 +682,8 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
         // gather metadata: slot of every term of the two numeric stages; the
         // longest rows and the term counts come back together
         int32_t *tc = nullptr, *d_max = nullptr;
-        TRY(alloc(ctx, &tc, (size_t)std::max(L.n, nagg)));
-        TRY(alloc(ctx, &d_max, 2));
+        TRY(alloc_temp(ctx, &tc, (size_t)std::max(L.n, nagg)));
+        TRY(alloc_temp(ctx, &d_max, 2));
         CK(cudaMemsetAsync(d_max, 0, 2 * sizeof(int32_t), ctx->s));
         launch_row_maxlen(L.n, L.AP_ptr, d_max, ctx->s);
         launch_row_maxlen(C.n, C.A_ptr, d_max + 1, ctx->s);
@@ -696,7 +716,7 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
             launch_block_gather(C.nnz, L.g2_ptr, L.g2_idx, L.g2_w, L.APb, C.Ab, ctx->s);
             launch_block_norms(C.nnz, C.Ab, C.A_val, ctx->s);
         } else {
-            launch_ap_numeric_f64(L, L.A_val, ctx->s);
+            launch_ap_numeric_f64(L, A_val, ctx->s);
             launch_rap_numeric_f64(L, C.A_ptr, C.A_val, ctx->s);
         }
         TRY(check_device(ctx, "Galerkin product"));
@@ -707,6 +727,7 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
             launch_cast_f32(L.nnzP, L.P_val, L.P_valf, ctx->s);
             launch_cast_f32(L.nnzR, L.R_val, L.R_valf, ctx->s);
         }
+        free_temp(ctx);
         ctx->nlev++;
         if (p.theta_halving) theta = theta * 0.5;
     }
@@ -731,7 +752,7 @@ amg_status full_setup_impl(amg_ctx *ctx, const double *d_val) {
             if (l + 1 < ctx->nlev) launch_cast_f32(L.nnzAP, L.AP_val, L.AP_valf, ctx->s);
         }
     TRY(build_delta16(ctx));
-    TRY(numeric_rebuild(ctx, blockmode(ctx) ? ctx->lev[0].Ab : ctx->lev[0].A_val, false));
+    TRY(numeric_rebuild(ctx, blockmode(ctx) ? F.Ab : F.sten.noff ? d_val : F.A_val, false));
     TRY(check_device(ctx, "full setup"));
     ctx->have_setup = true;
     ctx->setup_gen += 1;
@@ -748,6 +769,8 @@ amg_status ensure_persistent(amg_ctx *ctx, int32_t n, int32_t nnz) {
     ctx->fine_ncoff = 0;
     ctx->sten = Stencil{};
     ctx->sten_mask = nullptr;
+    ctx->sys_own = nullptr;
+    ctx->sys_own_vals = 0;
     ctx->n = n;
     ctx->nnz = nnz;
     TRY(alloc(ctx, &ctx->fine_ptr, (size_t)n + 1, true));
@@ -783,8 +806,22 @@ amg_status ensure_persistent(amg_ctx *ctx, int32_t n, int32_t nnz) {
     TRY(alloc(ctx, &ctx->stage_val, nvals(ctx), true));
     TRY(alloc(ctx, &ctx->stage_f, nv, true));
     TRY(alloc(ctx, &ctx->stage_u, nv, true));
-    ctx->A_sys_own = ctx->S_sys_own = nullptr;
-    if (ctx->prm.mode == AMG_MODE_FULL_REUSE) TRY(alloc(ctx, &ctx->A_sys_own, nvals(ctx), true));
+    return AMG_OK;
+}
+
+// full reuse: the system matrix is apart from the hierarchy's
+bool own_sys(const amg_ctx *ctx) { return ctx->prm.mode == AMG_MODE_FULL_REUSE; }
+amg_status alloc_sys(amg_ctx *ctx) {
+    if (!own_sys(ctx)) return AMG_OK;
+    const size_t want = ctx->sten.noff ? ctx->sten.nvals(ctx->n) : nvals(ctx);
+    if (ctx->sys_own && ctx->sys_own_vals >= want) return AMG_OK;
+    if (ctx->sys_own) {
+        ctx->persist.erase(std::find(ctx->persist.begin(), ctx->persist.end(), (void *)ctx->sys_own));
+        CK(cudaFreeAsync(ctx->sys_own, ctx->s));
+        ctx->sys_own = nullptr;
+    }
+    TRY(alloc(ctx, &ctx->sys_own, want, true));
+    ctx->sys_own_vals = want;
     return AMG_OK;
 }
 
@@ -803,8 +840,6 @@ amg_status stencil_pattern(amg_ctx *ctx, const std::vector<int32_t> &off) {
     TRY(reset_status(ctx));
     launch_stencil_mask(ctx->n, ctx->fine_ptr, ctx->fine_col, S, ctx->sten_mask, ctx->d_st, ctx->s);
     TRY(check_device(ctx, "stencil pattern"));
-    if (ctx->A_sys_own && !ctx->S_sys_own)
-        TRY(alloc(ctx, &ctx->S_sys_own, (size_t)(((int64_t)ctx->n + 31) / 32 * 32 * kMaxStencil), true));
     ctx->sten = S;
     return AMG_OK;
 }
@@ -818,8 +853,7 @@ amg_status compress_pattern(amg_ctx *ctx) {
     ctx->fine_ncoff = 0;
     ctx->sten = Stencil{};
     if (blockmode(ctx) || ctx->n >= (1 << 30)) return AMG_OK;
-    if (!ctx->fine_cidx) {
-        TRY(alloc(ctx, &ctx->fine_cidx, (size_t)ctx->nnz, true));
+    if (!ctx->fine_coff) {
         TRY(alloc(ctx, &ctx->fine_coff, (size_t)kMaxColOffsets, true));
         TRY(alloc(ctx, &ctx->coff_table, (size_t)kColOffsetSlots, true));
         TRY(alloc(ctx, &ctx->coff_count, 1, true));
@@ -843,6 +877,7 @@ amg_status compress_pattern(amg_ctx *ctx) {
         ctx->fine_ncoff = cnt;
         return AMG_OK;
     }
+    if (!ctx->fine_cidx) TRY(alloc(ctx, &ctx->fine_cidx, (size_t)ctx->nnz, true));
     CK(cudaMemcpyAsync(ctx->fine_coff, off.data(), sizeof(int32_t) * off.size(), cudaMemcpyHostToDevice, ctx->s));
     TRY(reset_status(ctx));
     launch_col_offsets_encode(ctx->n, ctx->fine_ptr, ctx->fine_col, ctx->fine_coff, cnt, ctx->fine_cidx, ctx->d_st,
@@ -866,6 +901,7 @@ amg_status set_pattern(amg_ctx *ctx, int32_t n, int32_t nnz, const int32_t *d_pt
     if (check_device(ctx, "row pointers") != AMG_OK)
         return set_err(ctx, AMG_ERR_PATTERN, "row pointers: not 0 at row 0, decreasing, or not ending at nnz");
     TRY(compress_pattern(ctx));
+    TRY(alloc_sys(ctx));
     ctx->pattern_ok = true;
     return AMG_OK;
 }
@@ -889,18 +925,17 @@ FineMat fine_mat(const amg_ctx *ctx) {
 }
 
 void update_sys(amg_ctx *ctx) {
-    ctx->A_sys = ctx->A_sys_own ? ctx->A_sys_own : blockmode(ctx) ? ctx->lev[0].Ab : ctx->lev[0].A_val;
-    ctx->S_sys = ctx->A_sys_own ? ctx->S_sys_own : ctx->lev[0].S_val;
+    ctx->A_sys = own_sys(ctx) ? ctx->sys_own : blockmode(ctx) ? ctx->lev[0].Ab : ctx->lev[0].A_val;
+    ctx->S_sys = own_sys(ctx) ? ctx->sys_own : ctx->lev[0].S_val;
 }
 
-// full reuse: the system matrix is apart from the hierarchy's
 amg_status copy_sys(amg_ctx *ctx, const double *d_val) {
-    if (!ctx->A_sys_own) return AMG_OK;
+    if (!own_sys(ctx)) return AMG_OK;
     if (ctx->sten.noff) {
-        launch_csr_to_stencil(ctx->n, ctx->fine_ptr, d_val, ctx->sten, ctx->S_sys_own, ctx->s);
+        launch_csr_to_stencil(ctx->n, ctx->fine_ptr, d_val, ctx->sten, ctx->sys_own, ctx->s);
         return AMG_OK;
     }
-    CK(cudaMemcpyAsync(ctx->A_sys_own, d_val, sizeof(double) * nvals(ctx), cudaMemcpyDeviceToDevice, ctx->s));
+    CK(cudaMemcpyAsync(ctx->sys_own, d_val, sizeof(double) * nvals(ctx), cudaMemcpyDeviceToDevice, ctx->s));
     return AMG_OK;
 }
 
@@ -1664,6 +1699,7 @@ amg_status amg_create(amg_ctx **out, const amg_params *prm, void *cuda_stream) {
 void amg_destroy(amg_ctx *ctx) {
     if (!ctx) return;
     cudaStreamSynchronize(ctx->s);
+    free_temp(ctx);
     for (void *p : ctx->hier) cudaFreeAsync(p, ctx->s);
     for (void *p : ctx->persist) cudaFreeAsync(p, ctx->s);
     cudaStreamSynchronize(ctx->s);
@@ -1779,10 +1815,11 @@ amg_status prepare_chunks(amg_ctx *ctx) {
         const int32_t nc = L.nc;
         std::vector<int32_t> last((size_t)nc, -1);
         int32_t *d_last = nullptr;
-        TRY(alloc(ctx, &d_last, (size_t)nc));
+        TRY(alloc_temp(ctx, &d_last, (size_t)nc));
         launch_row_last(nc, L.R_ptr, L.R_col, d_last, ctx->s);
         CK(cudaMemcpyAsync(last.data(), d_last, sizeof(int32_t) * (size_t)nc, cudaMemcpyDeviceToHost, ctx->s));
         CK(cudaStreamSynchronize(ctx->s));
+        free_temp(ctx);
         int32_t I = 0, pmax = -1;
         for (int c = 1; c <= kHostChunks; ++c) {
             const int32_t lim = ctx->ck_row[c];  // rows before this have landed with chunks 0 .. c - 1
@@ -1976,14 +2013,10 @@ amg_status amg_export_csr(amg_ctx *ctx, int32_t level, int32_t which, int32_t *d
     if (d_ptr) CK(cudaMemcpyAsync(d_ptr, ptr, sizeof(int32_t) * ((size_t)nrows + 1), cudaMemcpyDeviceToDevice, ctx->s));
     if (d_col) CK(cudaMemcpyAsync(d_col, col, sizeof(int32_t) * (size_t)nnz, cudaMemcpyDeviceToDevice, ctx->s));
     if (d_val) {
-        if (which == 0 && level == 0 && ctx->a_val_stale) {
-            // a stencil's last values are held by diagonals
-            launch_stencil_to_csr(L.n, L.A_ptr, L.S_val, L.sten, L.A_val, ctx->s);
-            ctx->a_val_stale = false;
-        }
         if (blockmode(ctx) && which == 0)
             CK(cudaMemcpyAsync(d_val, L.Ab, sizeof(double) * 16 * (size_t)nnz, cudaMemcpyDeviceToDevice, ctx->s));
         else if (mixed(ctx) && valf) launch_copy_cast<float, double>(nnz, valf, d_val, nullptr, ctx->s);
+        else if (which == 0 && L.sten.noff) launch_stencil_to_csr(L.n, L.A_ptr, L.S_val, L.sten, d_val, ctx->s);
         else CK(cudaMemcpyAsync(d_val, val, sizeof(double) * (size_t)nnz, cudaMemcpyDeviceToDevice, ctx->s));
     }
     CK(cudaStreamSynchronize(ctx->s));

@@ -100,7 +100,7 @@ struct Level {
     int A_ncoff = 0;
     int16_t *A_c16 = nullptr;
     ColIdx cols() const { return ColIdx{A_col, A_cidx, A_coff, A_ncoff, A_c16}; }
-    double *A_val = nullptr;   // FP64 values (level 0: the hierarchy's copy of the fine matrix)
+    double *A_val = nullptr;   // FP64 values (level 0: a copy of the fine matrix, none with sten)
     float *A_valf = nullptr;   // FP32 values (mixed precision)
     // the finest level's values by diagonals, when its pattern is a stencil
     Stencil sten;
