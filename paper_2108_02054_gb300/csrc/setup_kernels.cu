@@ -291,10 +291,19 @@ k_poisson_vals(int dim, int N, int64_t n, int top, const double *__restrict__ rh
 // plane through kLogPlanes planes, a cell's density exp(theta) kept in
 // registers for its own plane and the next, the plane's tile (with N cells on
 // either side for the y neighbours) in shared memory.  An FP64 exponential is
-// some 25 instructions of the slow pipe and a cell's seven densities bounded the
-// kernels; this forms about 1 + 2 N / 256 + 1/4 per cell.  Used while a tile
-// fits (kLogTile cells), else the direct kernels above and below.
-constexpr int kLogPlanes = 8, kLogTile = 4096;
+// some 25 instructions of the slow pipe and a cell's seven densities bound the
+// direct kernels above and below; this forms about 1 + 2 N / 256 + 1/4 per cell.
+// It is used where it is the faster form (and a tile fits, kLogTile cells):
+// - 2D below 384 cells a side, where the halo leaves fewer than four
+//   exponentials a cell of the direct form's five.  Values, marching against
+//   direct: 256^2 13.4 / 16.5 us, 320^2 19.4 / 22.2, 384^2 30.1 / 29.3, 512^2
+//   50.7 / 48.5, 1,024^2 298 / 177, 1,900^2 1,719 / 601.
+// - 3D from three quarters of the SMs' number of blocks on: a block's chain of
+//   eight planes takes 55 us however few there are.  16^3 49.6 / 14.4 us, 32^3
+//   55.2 / 14.3, 48^3 56.5 / 30.4, 58^3 57.3 / 55.3, 60^3 57.5 / 57.9, 64^3 57.7 /
+//   67.7, 128^3 274 / 493.
+// (The gradient's times cross at the same sizes.)
+constexpr int kLogPlanes = 8, kLogTile = 4096, kLogWide2d = 384, kLogBlocks3d = 114;
 template <class Cell>
 __device__ __forceinline__ void march_log(int dim, int N, const double *__restrict__ theta, Cell cell) {
     extern __shared__ double s_tile[];  // 256 + 2 N densities: cell t of the tile at t + N
@@ -1330,11 +1339,13 @@ void launch_poisson_cols(int dim, int N, const int32_t *ptr, int32_t *col, cudaS
     k_poisson_cols<<<nblocks(n), kThreads, 0, s>>>(dim, N, n, ptr, col);
 }
 namespace {
-// the marching kernels' grid (tiles of a plane, chunks of planes), when a tile fits
+// the marching kernels' grid (tiles of a plane, chunks of planes), where they
+// are the faster form and a tile fits
 bool log_grid(int dim, int N, dim3 &g, size_t &smem) {
     if (256 + 2 * N > kLogTile) return false;
-    const int64_t P = (int64_t)N * N;
-    g = dim3((unsigned)((P + 255) / 256), (unsigned)((dim == 3 ? N + kLogPlanes - 1 : kLogPlanes) / kLogPlanes));
+    const int64_t tiles = ((int64_t)N * N + 255) / 256, chunks = dim == 3 ? (N + kLogPlanes - 1) / kLogPlanes : 1;
+    if (dim == 2 ? N >= kLogWide2d : tiles * chunks < kLogBlocks3d) return false;
+    g = dim3((unsigned)tiles, (unsigned)chunks);
     smem = sizeof(double) * (size_t)(256 + 2 * N);
     return g.y <= 65535;
 }
