@@ -1025,25 +1025,6 @@ void up_finest(amg_ctx *ctx, const double *f, V *u, TZ *out, double *rz_partial,
     }
 }
 
-// post-smoothing on level l; the last sweep writes `out` (type TO) when given
-template <class V, class TF, class TO>
-void up_level(amg_ctx *ctx, int l, const TF *f, V *u, TO *out, const int *skip) {
-    Level &L = ctx->lev[l];
-    VecSet<V> &v = Vops<V>::vec(L);
-    const V *A = Vops<V>::A(L), *m = Vops<V>::m(L);
-    V *t = (u == v.u) ? v.t : v.u;
-    const int npost = ctx->prm.npost;
-    for (int k = 0; k < npost; ++k) {
-        if (k == npost - 1 && out) {
-            { ProfScope ps_(ctx, AMG_PROF_SWEEP_L0, l == 0); launch_smooth_sweep<V, TF, TO>(L, A, m, f, u, out, skip, ctx->s); }
-            return;
-        }
-        launch_smooth_sweep<V, TF, V>(L, A, m, f, u, t, skip, ctx->s);
-        std::swap(u, t);
-    }
-    if (out) launch_copy_cast<V, TO>(L.n, u, out, skip, ctx->s);
-}
-
 template <class V, class TZ>
 void enqueue_vcycle(amg_ctx *ctx, const double *r, TZ *z, const int *skip, double *rz_partial, bool u0_ready) {
     const int nl = ctx->nlev;

@@ -548,9 +548,11 @@ __device__ __forceinline__ KeyIdx better(KeyIdx a, KeyIdx b) {
 // Small matrices (n <= kLuSmemN) are factorised in shared memory by one block
 // with a lazy row permutation: rows are not moved during the elimination,
 // perm[i] names the physical row at position i, and the factors are written
-// out in position order at the end.  Larger ones use the cluster kernel (up to
-// kLuClusterN rows), panels (up to kLuWideN) or the global-memory kernel.
-constexpr int kLuSmemN = 160;
+// out in position order at the end.  Larger ones use the pipelined cluster
+// kernel (up to kLuPipeN rows; slower below, with fewer steps to pipeline), the
+// row-cyclic one (up to kLuClusterN), panels (up to kLuWideN) or the
+// global-memory kernel.
+constexpr int kLuSmemN = 48;
 constexpr int kLuClusterN = 448;   // 8 CTAs x 56 rows x 448 columns fit in 227 KB each
 constexpr int kLuThreads = 512;
 __global__ void __launch_bounds__(kLuThreads) k_dense_lu_smem(int32_t n, double *__restrict__ g,
@@ -615,7 +617,7 @@ __global__ void __launch_bounds__(kLuThreads) k_dense_lu_smem(int32_t n, double 
     for (int64_t e = tid; e < nn; e += kLuThreads) g[e] = a[(int64_t)perm[e / n] * n + e % n];
 }
 
-// Mid-size matrices (kLuSmemN < n <= kLuClusterN) are factorised by one
+// Mid-size matrices (kLuPipeN < n <= kLuClusterN) are factorised by one
 // thread-block cluster of eight CTAs (eight SMs' FP64 pipes): physical row r
 // lives in the shared memory of CTA r % 8.  Each step, every CTA ranks its own
 // rows (positions >= k; ties to the lower position), the CTAs read the eight
@@ -777,14 +779,13 @@ k_dense_lu_cluster(int32_t n, double *__restrict__ g, double *__restrict__ gT, i
 // its own that step k waited for).  So slot k % R, last used by step k - R,
 // is free: k - R < b_q B - 1 for every b_q >= k / B - C + 1.
 constexpr int kLuPipeN = 256;
-constexpr int kLuPipeMinN = 48;  // below: the one-CTA kernel is faster (fewer steps to pipeline)
 constexpr int kLuPipeB = 4;      // columns per ownership block
 // CTAs and warps: eight CTAs at every size; eight compute warps for 128 < n <=
 // 256.  n = 153 / 212 / 255: 226 / 332 / 430 us (sixteen CTAs, a non-portable
 // cluster: 235 / 324 / 393), where the one-CTA kernel took 569 at 153 and the
 // row-cyclic cluster kernel 722 / 876; n = 87 with four warps 103.  The owner's
 // step (about 2,000 cycles) bounds it, and at 255 the trailing updates too.
-constexpr int kLuPipeWideC = 8;
+constexpr int kLuPipeC = 8;
 // W compute warps, one row per lane (and the sender warp); C CTAs
 __host__ __device__ constexpr int lu_pipe_threads(int W) { return (W + 1) * 32; }
 __host__ __device__ constexpr int lu_pipe_ring(int C, int B) { return C * B + 8; }
@@ -2851,16 +2852,11 @@ size_t lu_cluster_smem(int32_t n) {
 bool lu_wants_transpose(int32_t n) { return n > kInvRowsN && n <= kLuWideN; }
 void launch_dense_lu(int32_t n, double *a, int32_t *piv, int *st, cudaStream_t s, double *aT) {
     static bool attr = false;
-    const int max_bytes = kLuSmemN * kLuSmemN * (int)sizeof(double);
     if (!attr) {
-        cudaFuncSetAttribute(k_dense_lu_pipe<8, kLuPipeB, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)lu_pipe_smem(128, 8, kLuPipeB));
-        cudaFuncSetAttribute(k_dense_lu_pipe<kLuPipeWideC, kLuPipeB, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)lu_pipe_smem(kLuPipeN, kLuPipeWideC, kLuPipeB));
-        if (kLuPipeWideC > 8)
-            cudaFuncSetAttribute(k_dense_lu_pipe<kLuPipeWideC, kLuPipeB, 8>,
-                                 cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        cudaFuncSetAttribute(k_dense_lu_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
+        cudaFuncSetAttribute(k_dense_lu_pipe<kLuPipeC, kLuPipeB, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)lu_pipe_smem(128, kLuPipeC, kLuPipeB));
+        cudaFuncSetAttribute(k_dense_lu_pipe<kLuPipeC, kLuPipeB, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)lu_pipe_smem(kLuPipeN, kLuPipeC, kLuPipeB));
         cudaFuncSetAttribute(k_dense_lu_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)lu_cluster_smem(kLuClusterN));
         attr = true;
@@ -2880,14 +2876,14 @@ void launch_dense_lu(int32_t n, double *a, int32_t *piv, int *st, cudaStream_t s
         return;
     }
     count_launch();
-    if (n > kLuPipeMinN && n <= 128)
-        k_dense_lu_pipe<8, kLuPipeB, 4>
-            <<<8, lu_pipe_threads(4), lu_pipe_smem(n, 8, kLuPipeB), s>>>(n, a, aT, piv, st);
-    else if (n > 128 && n <= kLuPipeN)
-        k_dense_lu_pipe<kLuPipeWideC, kLuPipeB, 8>
-            <<<kLuPipeWideC, lu_pipe_threads(8), lu_pipe_smem(n, kLuPipeWideC, kLuPipeB), s>>>(n, a, aT, piv, st);
-    else if (n <= kLuSmemN)
+    if (n <= kLuSmemN)
         k_dense_lu_smem<<<1, kLuThreads, (size_t)n * n * sizeof(double), s>>>(n, a, piv, st);
+    else if (n <= 128)
+        k_dense_lu_pipe<kLuPipeC, kLuPipeB, 4>
+            <<<kLuPipeC, lu_pipe_threads(4), lu_pipe_smem(n, kLuPipeC, kLuPipeB), s>>>(n, a, aT, piv, st);
+    else if (n <= kLuPipeN)
+        k_dense_lu_pipe<kLuPipeC, kLuPipeB, 8>
+            <<<kLuPipeC, lu_pipe_threads(8), lu_pipe_smem(n, kLuPipeC, kLuPipeB), s>>>(n, a, aT, piv, st);
     else if (n <= kLuClusterN)
         k_dense_lu_cluster<<<kLuClusterCtas, kLuClusterThreads, lu_cluster_smem(n), s>>>(n, a, aT, piv, st);
     else
@@ -3067,7 +3063,6 @@ INST_V(double, double, double)
 INST_V(float, float, float)
 INST_V(float, double, double)
 INST_V(float, double, float)
-INST_V(float, float, double)
 #undef INST_V
 template void launch_smooth0_residual<double, double>(const Level &, const double *, const double *, const double *,
                                                       double *, double *, const int *, cudaStream_t);
