@@ -44,3 +44,29 @@ def held(precision, mode, smoothed):
 def test_device_memory_of_a_hierarchy(case):
     held(*case)  # (first use: the runtime's own memory)
     assert held(*case) <= LIMITS[case]
+
+
+def test_full_reuse_matrix_across_forms_of_one_size():
+    """One context, patterns of the same rows and entries held by diagonals and
+    in CSR in turn: the full-reuse system matrix is made again where its form
+    needs more, and each solve is with the last step's values."""
+    n = 600
+    i = torch.arange(n - 1, device="cuda")
+    G = B.AMG(mode=B.MODE_FULL_REUSE, coarse_enough=50)
+    f = torch.linspace(-1.0, 1.0, n, dtype=torch.float64, device="cuda")
+    for diagonals in (False, True, False, True, True):
+        j = i + 1 if diagonals else torch.where(i + 1 + i % 7 < n, i + 1 + i % 7, i + 1)
+        A = torch.eye(n, dtype=torch.float64, device="cuda") * 0.1
+        for a, b in ((i, j), (j, i)):
+            A.index_put_((a, b), torch.tensor(-1.0, dtype=torch.float64, device="cuda"))
+            A.diagonal().index_add_(0, a, torch.ones(n - 1, dtype=torch.float64, device="cuda"))
+        S = A.to_sparse_csr()
+        ptr, col, val = S.crow_indices().int(), S.col_indices().int(), S.values().contiguous()
+        assert val.numel() == 3 * n - 2
+        G.full_setup(ptr, col, val)
+        assert G.pattern_info() == (1, 3 if diagonals else 15)
+        for scale in (1.0, 1.25):
+            G.step(val * scale)
+            u, info = G.solve(f, 1e-9)
+            assert info.status == 0
+            assert torch.linalg.norm(f - scale * (A @ u)) <= 1.01e-9 * torch.linalg.norm(f)
